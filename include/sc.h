@@ -432,7 +432,8 @@ int sc_probe_fma_peak(int kind, void *cuda_stream, double *flops_per_s);
  * TRSM tiles, RL assembly pairs, device-loop items, warp-block units, SIMT
  * tiles split along the inner dimension (added atomically), target-owned RL
  * assembly slabs (deterministic plans) and the tensor-core tiles that are 256
- * columns wide. Errors: -1, -2, -3. */
+ * columns wide. SC_FP64 products are counted as the SIMT tiles they cover, also
+ * where they run on the tensor cores as products of slices. Errors: -1, -2, -3. */
 int sc_plan_stats(const sc_symbolic *s, int precision, int64_t *out, int nout);
 
 /* Host-side check of the device schedule of s (no device work): recomputes,
@@ -459,7 +460,8 @@ int sc_plan_stats(const sc_symbolic *s, int precision, int64_t *out, int nout);
  *   schedule, a launch plan (FP64 or tensor-core) with a product tile split
  *   along the inner dimension, or a target row of an RL assembly pair that no
  *   slab of its target owns, or a slab whose pairs are not one target's in
- *   source order).
+ *   source order; 14 an FP64 launch plan whose source blocks of tensor-core
+ *   products miss rows or columns, are split more than once or overlap).
  * Returns SC_OK, SC_ERR_INTERNAL when a violation is found, -1 / -2 for NULL
  * arguments. */
 int sc_check_schedule(const sc_symbolic *s, int64_t *out, int nout);

@@ -361,7 +361,8 @@ class Symbolic:
     CHECK_KINDS = {0: "ok", 1: "source range", 2: "target range", 3: "trapezoid", 4: "not an ancestor",
                    5: "level order", 6: "critical flag", 7: "run mapping", 8: "RL pool", 9: "RL relind",
                    10: "plain write outside the own panel", 11: "entry mapping",
-                   12: "tensor-core K range", 13: "deterministic plan"}
+                   12: "tensor-core K range", 13: "deterministic plan",
+                   14: "slice blocks"}
 
     def save(self, path) -> None:
         """sc_symbolic_save: the analysis on disk (factor later without analysing again)."""

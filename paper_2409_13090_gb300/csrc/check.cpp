@@ -244,6 +244,7 @@ extern "C" int sc_check_schedule(const sc_symbolic *s, int64_t *out, int nout) {
             if (bad_kind) bad_level = (int64_t)lv;
         }
         if (!bad_kind && s->opt.deterministic) bad_kind = det_plan_check(s, &bad_level);
+        if (!bad_kind) bad_kind = split_plan_check(s, &bad_level);
         int64_t v[] = {tasks, products, entries, bad_level, bad_kind};
         for (int i = 0; i < nout && i < 5; i++) out[i] = v[i];
         return bad_kind ? SC_ERR_INTERNAL : SC_OK;

@@ -88,6 +88,22 @@ struct BlkDev {
     int32_t bs, pad;
 };
 
+// Source block of FP64 products on the tensor cores (split_gemm.cuh): rows
+// row0 .. row0 + rows - 1 and columns kx0 .. kx0 + k - 1 of a panel, cut into FP16
+// slices in the level's half of the slice pool.
+struct SplitBlk {
+    int64_t src;     // offset of (row0, kx0) in the factor storage
+    int64_t piece0;  // first row of the slice pool (rows of 32 values)
+    int32_t ld, rows, k, row0;
+    int32_t exp0;    // first row exponent
+    int32_t pad;
+};
+// 64 rows of a source block: the work of one CTA of the splitting kernel.
+struct SplitUnit {
+    int32_t blk, row0;
+};
+constexpr int kSplitRows = 64;
+
 constexpr int kLoopSmemBytes = 48 * 1024;
 
 // Target-owned RL assembly (deterministic plans): rows [row0, row1) of Lnz(P)

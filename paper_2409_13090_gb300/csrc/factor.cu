@@ -7,6 +7,7 @@
 
 #include "kernels.cuh"
 #include "numeric.h"
+#include "split_gemm.cuh"
 #include "tc_gemm.cuh"
 
 namespace sc {
@@ -280,6 +281,16 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
             E();
             launches++;
         }
+        if constexpr (sizeof(T) == 8) {
+            if (pl.sp_cnt) {
+                B(kProfTc);
+                launch_split_gemm((double *)lnz, (double *)pool, h->d_tasks, h->d_gemm + pl.sp_off, pl.sp_cnt,
+                                  h->d_split_of_task, h->d_splits, h->d_exps, h->d_slice_maps, h->d_err,
+                                  (long long)s->opt.spin_limit, h->num_sms, ps);
+                E();
+                launches++;
+            }
+        }
         if constexpr (sizeof(T) == 4) {
             if (pl.tc_cnt) {
                 B(kProfTc);
@@ -330,6 +341,17 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
                                                            h->d_lo);
             E();
             launches++;
+        }
+        if constexpr (sizeof(T) == 8) {
+            // the level's half of the slice pool was last read by the products of level
+            // lv - 2, which this stream has waited for (ev_rest, at level lv - 1)
+            if (p.split_cnt) {
+                B(kProfTc);
+                launch_split((const double *)lnz, h->d_splits, h->d_split_units + p.split_off, p.split_cnt,
+                             h->d_slices, h->d_exps, st);
+                E();
+                launches++;
+            }
         }
         // Lookahead: level lv's products into chunks two or more levels up run on
         // st3, overlapping level lv+1's POTRF, TRSM and device loops; level lv+1's
@@ -385,6 +407,16 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
             E();
             launches++;
         }
+        if constexpr (sizeof(T) == 8) {
+            if (p.rlsp_cnt) {
+                B(kProfRlUpd);
+                launch_split_gemm((double *)lnz, (double *)pool, h->d_tasks, h->d_gemm + p.rlsp_off, p.rlsp_cnt,
+                                  h->d_split_of_task, h->d_splits, h->d_exps, h->d_slice_maps, h->d_err,
+                                  (long long)s->opt.spin_limit, h->num_sms, st);
+                E();
+                launches++;
+            }
+        }
         if (p.rls_cnt) {
             B(kProfRlUpd);
             k_small_tasks<T><<<(p.rls_cnt + 7) / 8, 256, 0, st>>>(lnz, pool, h->d_tasks, h->d_small + p.rls_off,
@@ -433,7 +465,7 @@ int set_smem_attrs() {
     SC_CUDA(cudaFuncSetAttribute(k_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, kPotrfSmem));
     SC_CUDA(cudaFuncSetAttribute(k_level<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPotrfSmem));
     SC_CUDA(cudaFuncSetAttribute(k_level<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPotrfSmem));
-    if (!tc_gemm_init()) return SC_ERR_CUDA;
+    if (!tc_gemm_init() || !split_gemm_init()) return SC_ERR_CUDA;
     done = true;
     return SC_OK;
 }
@@ -452,6 +484,12 @@ struct Plan {
     std::vector<LoopItem> loops;
     std::vector<LevelPlan> levels;
     int64_t inv_size = 0;  // elements of the diagonal-block inverses
+    // FP64 products on the tensor cores (empty without them)
+    std::vector<SplitBlk> splits;
+    std::vector<SplitUnit> split_units;
+    std::vector<int32_t> split_of_task;  // per task: its source block (0 where it has none)
+    int64_t slice_pieces = 0;            // rows of the slice pool, both halves
+    int64_t exps = 0;                    // row exponents, both halves
     double class_flops[kProfClasses] = {};
     // fused plans: the units of every level's k_level launch, then the tail launch's
     std::vector<FlowUnit> flow;
@@ -493,8 +531,12 @@ void build_flow(Plan &P, bool lookahead) {
 
 // lookahead: split each level's tiled products into those that target chunks
 // of the next level (crit) and the rest (targets two or more levels up).
-void build_plan(const sc_symbolic *s, int precision, Plan &P, bool lookahead) {
+// split64: FP64 products on the tensor cores (split_route) instead of SIMT tiles.
+void build_plan(const sc_symbolic *s, int precision, Plan &P, bool lookahead, bool split64) {
     const Knobs kn = knobs_of(s->tune);
+    split64 = split64 && precision == SC_FP64;
+    int64_t half_pieces[2] = {0, 0}, half_exps[2] = {0, 0};  // largest level of each parity
+    std::vector<int32_t> split_of_sn(split64 ? s->nsuper : 0, -1);  // the level's block of a source supernode
     const bool det = s->opt.deterministic != 0;
     P.cd.resize(s->chunks.size());
     int64_t inv = 0;
@@ -535,8 +577,29 @@ void build_plan(const sc_symbolic *s, int precision, Plan &P, bool lookahead) {
         // product tasks: tensor-core tiles (TF32), SIMT tiles, warp tasks
         std::vector<int32_t> ids_small;
         std::vector<ThinUnit> units_thin[2];
-        std::vector<GemmTile> g_simt[2], g_tc[2], g_tc64[2], g_tc256[2];
+        std::vector<GemmTile> g_simt[2], g_tc[2], g_tc64[2], g_tc256[2], g_sp[2];
         const bool split = lookahead;
+        // the level's source blocks for FP64 products on the tensor cores: one per source
+        // supernode (all of a level's products of a supernode read the same columns), its
+        // rows from the first one that a routed product reads
+        const size_t blk0 = P.splits.size();
+        auto use_split = [&](const Task &t) {
+            if (!split64 || is_small(t) || !split_route(t, s->sup_ptr[t.src + 1] - s->sup_ptr[t.src])) return false;
+            const int32_t m = (int32_t)(s->gl_ptr[t.src + 1] - s->gl_ptr[t.src]), r = std::min(t.a_row, t.b_row);
+            int32_t &b = split_of_sn[t.src];
+            if (b < 0) {
+                b = (int32_t)P.splits.size();
+                P.splits.push_back(SplitBlk{s->lnz_off[t.src] + t.kx0, 0, s->lnz_ld[t.src], m - r, t.k, r, 0, 0});  // src, piece0, exp0: below
+            } else if (r < P.splits[b].row0) {
+                P.splits[b].rows = m - r;
+                P.splits[b].row0 = r;
+            }
+            return true;
+        };
+        auto set_split = [&](const Task &t, int32_t id) {
+            P.split_of_task.resize(id + 1, 0);
+            P.split_of_task[id] = split_of_sn[t.src];
+        };
         for (Task t : L.tasks) {
             int32_t id = (int32_t)P.tasks.size();
             const int cls = split && !(t.flags & kTaskCrit) ? 1 : 0;  // 0 crit, 1 rest
@@ -551,6 +614,10 @@ void build_plan(const sc_symbolic *s, int precision, Plan &P, bool lookahead) {
             } else if (bn) {
                 if (bn == 256 && kn.tc_multicast) tc_tile_pairs_of(t, id, g_tc256[cls]);
                 else tc_tiles_of(t, id, bn, bn == 256 ? g_tc256[cls] : bn == 128 ? g_tc[cls] : g_tc64[cls]);
+                P.class_flops[kProfTc] += task_flops(t);
+            } else if (use_split(t)) {
+                set_split(t, id);
+                split_tiles_of(t, id, g_sp[cls]);
                 P.class_flops[kProfTc] += task_flops(t);
             } else if (std::min(t.m, t.n) <= std::min(kn.thin_dim, kThinDim) && !(t.flags & kTaskStoreU)) {
                 // a 64 x 64 tile would be mostly padding: warp blocks, kThinWarps per CTA
@@ -577,6 +644,9 @@ void build_plan(const sc_symbolic *s, int precision, Plan &P, bool lookahead) {
             pl.tc256_off = (int32_t)P.gemm.size();
             P.gemm.insert(P.gemm.end(), g_tc256[cls].begin(), g_tc256[cls].end());
             pl.tc256_cnt = (int32_t)g_tc256[cls].size();
+            pl.sp_off = (int32_t)P.gemm.size();
+            P.gemm.insert(P.gemm.end(), g_sp[cls].begin(), g_sp[cls].end());
+            pl.sp_cnt = (int32_t)g_sp[cls].size();
             pl.thin_off = (int32_t)P.thin.size();
             P.thin.insert(P.thin.end(), units_thin[cls].begin(), units_thin[cls].end());
             pl.thin_cnt = (int32_t)units_thin[cls].size();
@@ -597,14 +667,46 @@ void build_plan(const sc_symbolic *s, int precision, Plan &P, bool lookahead) {
         P.class_flops[kProfLoop] += L.loop_flops;
         // RL update matrices and assembly
         std::vector<int32_t> rl_small;
-        std::vector<GemmTile> rl_g;
+        std::vector<GemmTile> rl_g, rl_sp;
         for (const Task &t : L.rl_tasks) {
             int32_t id = (int32_t)P.tasks.size();
             P.tasks.push_back(t);
-            if (is_small(t)) rl_small.push_back(id);
-            else tiles_of(t, id, rl_g, det);
+            if (is_small(t)) {
+                rl_small.push_back(id);
+            } else if (use_split(t)) {
+                set_split(t, id);
+                split_tiles_of(t, id, rl_sp);
+            } else {
+                tiles_of(t, id, rl_g, det);
+            }
             P.class_flops[kProfRlUpd] += task_flops(t);
         }
+        p.rlsp_off = (int32_t)P.gemm.size();
+        P.gemm.insert(P.gemm.end(), rl_sp.begin(), rl_sp.end());
+        p.rlsp_cnt = (int32_t)rl_sp.size();
+        // slices and exponents of the level's blocks, from the start of the level's half
+        // (the offsets of odd levels get the even half's size added below)
+        p.split_off = (int32_t)P.split_units.size();
+        {
+            int64_t piece = 0, exp = 0;
+            for (size_t b = blk0; b < P.splits.size(); b++) {
+                SplitBlk &bk = P.splits[b];
+                bk.src += (int64_t)bk.row0 * bk.ld;
+                bk.piece0 = piece;
+                bk.exp0 = (int32_t)exp;
+                bk.pad = (int32_t)(lv % 2);
+                piece += (int64_t)((bk.k + sp::BK - 1) / sp::BK) * sp::S * bk.rows;
+                exp += bk.rows;
+                for (int32_t r = 0; r < bk.rows; r += kSplitRows) P.split_units.push_back(SplitUnit{(int32_t)b, r});
+            }
+            half_pieces[lv % 2] = std::max(half_pieces[lv % 2], piece);
+            half_exps[lv % 2] = std::max(half_exps[lv % 2], exp);
+            for (const Task &t : L.tasks)
+                if (split64) split_of_sn[t.src] = -1;
+            for (const Task &t : L.rl_tasks)
+                if (split64) split_of_sn[t.src] = -1;
+        }
+        p.split_cnt = (int32_t)P.split_units.size() - p.split_off;
         p.rlg_off = (int32_t)P.gemm.size();
         P.gemm.insert(P.gemm.end(), rl_g.begin(), rl_g.end());
         p.rlg_cnt = (int32_t)rl_g.size();
@@ -645,14 +747,27 @@ void build_plan(const sc_symbolic *s, int precision, Plan &P, bool lookahead) {
             }
         }
     }
+    for (SplitBlk &bk : P.splits)
+        if (bk.pad) {
+            bk.piece0 += half_pieces[0];
+            bk.exp0 += (int32_t)half_exps[0];
+        }
+    P.slice_pieces = half_pieces[0] + half_pieces[1];
+    P.exps = half_exps[0] + half_exps[1];
+    P.split_of_task.resize(P.tasks.size(), 0);
 }
 
 }  // namespace
 
+// one persistent launch per level (SIMT tiles only): FP64 and FP32, RLB schedule
+static bool fused_plan(const sc_symbolic *s, int precision) {
+    return knobs_of(s->tune).fused && s->opt.variant == SC_RLB && (precision == SC_FP64 || precision == SC_FP32);
+}
+
 int det_plan_check(const sc_symbolic *s, int64_t *bad_level) {
     for (int precision : {SC_FP64, SC_TF32}) {
         Plan P;
-        build_plan(s, precision, P, false);
+        build_plan(s, precision, P, false, true);
         for (size_t lv = 0; lv < P.levels.size(); lv++) {
             const LevelPlan &p = P.levels[lv];
             *bad_level = (int64_t)lv;
@@ -663,9 +778,10 @@ int det_plan_check(const sc_symbolic *s, int64_t *bad_level) {
             };
             for (const ProdLists *pl : {&p.crit, &p.rest})
                 if (split_in(pl->gemm_off, pl->gemm_cnt) || split_in(pl->tc_off, pl->tc_cnt) ||
-                    split_in(pl->tc64_off, pl->tc64_cnt) || split_in(pl->tc256_off, pl->tc256_cnt))
+                    split_in(pl->tc64_off, pl->tc64_cnt) || split_in(pl->tc256_off, pl->tc256_cnt) ||
+                    split_in(pl->sp_off, pl->sp_cnt))
                     return 13;
-            if (split_in(p.rlg_off, p.rlg_cnt)) return 13;
+            if (split_in(p.rlg_off, p.rlg_cnt) || split_in(p.rlsp_off, p.rlsp_cnt)) return 13;
             if (!p.rlp_cnt) continue;
             // slabs: inside the level's pairs, one target each, sources ascending (pool offsets
             // follow the level's source order), groups disjoint and ascending, a group's row
@@ -705,9 +821,69 @@ int det_plan_check(const sc_symbolic *s, int64_t *bad_level) {
     return 0;
 }
 
+int split_plan_check(const sc_symbolic *s, int64_t *bad_level) {
+    Plan P;
+    build_plan(s, SC_FP64, P, false, true);
+    std::vector<int64_t> half_end(2, 0);  // slice rows used by the levels of each parity
+    int64_t odd0 = INT64_MAX;
+    for (size_t lv = 0; lv < P.levels.size(); lv++) {
+        const LevelPlan &p = P.levels[lv];
+        *bad_level = (int64_t)lv;
+        int64_t end = -1;
+        for (int32_t u = p.split_off; u < p.split_off + p.split_cnt; u++) {
+            const SplitUnit &su = P.split_units[u];
+            const SplitBlk &b = P.splits[su.blk];
+            // every row of a block once: its units in order, blocks one after another
+            const bool head = u == p.split_off || P.split_units[u - 1].blk != su.blk;
+            if (su.row0 != (head ? 0 : P.split_units[u - 1].row0 + kSplitRows) || su.row0 >= b.rows) return 14;
+            const bool tail = u + 1 == p.split_off + p.split_cnt || P.split_units[u + 1].blk != su.blk;
+            if (tail && su.row0 + kSplitRows < b.rows) return 14;
+            if (!head) continue;
+            // slices inside the pool, after the previous block's; exponents likewise
+            if (b.rows < 1 || b.k < 1 || (end >= 0 && b.piece0 < end) || b.exp0 < 0 || b.exp0 + (int64_t)b.rows > P.exps)
+                return 14;
+            if (lv % 2) odd0 = std::min(odd0, b.piece0);
+            end = b.piece0 + (int64_t)((b.k + sp::BK - 1) / sp::BK) * sp::S * b.rows;
+            half_end[lv % 2] = std::max(half_end[lv % 2], end);
+            if (b.piece0 < 0 || end > P.slice_pieces) return 14;
+        }
+        auto tiles_ok = [&](int32_t off, int32_t cnt) {
+            for (int32_t i = off; i < off + cnt; i++) {
+                const Task &t = P.tasks[P.gemm[i].task];
+                const int32_t bi = P.split_of_task[P.gemm[i].task];
+                if (bi < 0 || bi >= (int32_t)P.splits.size()) return false;
+                const SplitBlk &b = P.splits[bi];
+                const int32_t ld = s->lnz_ld[t.src];
+                // the block is this level's, and holds the product's rows and columns, 16-byte aligned
+                bool mine = false;
+                for (int32_t u = p.split_off; !mine && u < p.split_off + p.split_cnt;
+                     u += std::max(1, (P.splits[P.split_units[u].blk].rows + kSplitRows - 1) / kSplitRows))
+                    mine = P.split_units[u].blk == bi;
+                if (!mine || b.k != t.k || b.ld != ld ||
+                    b.src != s->lnz_off[t.src] + (int64_t)b.row0 * ld + t.kx0 || b.src % 2 || ld % 2)
+                    return false;
+                for (int32_t r : {t.a_row, t.b_row})
+                    if (r < b.row0) return false;
+                if (t.a_row + t.m > b.row0 + b.rows || t.b_row + t.n > b.row0 + b.rows) return false;
+                while (i + 1 < off + cnt && P.gemm[i + 1].task == P.gemm[i].task) i++;
+            }
+            return true;
+        };
+        if (!tiles_ok(p.crit.sp_off, p.crit.sp_cnt) || !tiles_ok(p.rest.sp_off, p.rest.sp_cnt) ||
+            !tiles_ok(p.rlsp_off, p.rlsp_cnt))
+            return 14;
+    }
+    // the two halves apart: a level's products may still read theirs while the next
+    // level's are being written
+    *bad_level = (int64_t)P.levels.size() - 1;
+    if (odd0 != INT64_MAX && half_end[0] > odd0) return 14;
+    *bad_level = -1;
+    return 0;
+}
+
 int plan_stats(const sc_symbolic *s, int precision, int64_t *out, int nout) {
     Plan P;
-    build_plan(s, precision, P, false);
+    build_plan(s, precision, P, false, false);  // FP64: the products as the SIMT tiles they cover
     int64_t small_tasks = 0, tile_tasks = 0;
     for (const LevelPlan &l : P.levels) small_tasks += l.small_cnt + l.rls_cnt;
     tile_tasks = (int64_t)P.tasks.size() - small_tasks;
@@ -715,7 +891,7 @@ int plan_stats(const sc_symbolic *s, int precision, int64_t *out, int nout) {
     for (const LevelPlan &l : P.levels) {
         tc256_tiles += l.crit.tc256_cnt + l.rest.tc256_cnt;
         tc_tiles += l.crit.tc_cnt + l.crit.tc64_cnt + l.crit.tc256_cnt + l.rest.tc_cnt + l.rest.tc64_cnt +
-                    l.rest.tc256_cnt;
+                    l.rest.tc256_cnt + l.crit.sp_cnt + l.rest.sp_cnt + l.rlsp_cnt;
         simt_tiles += l.crit.gemm_cnt + l.rest.gemm_cnt + l.rlg_cnt;
     }
     for (const GemmTile &g : P.gemm) split_tiles += g.ks >= 0;
@@ -787,12 +963,32 @@ int numeric_create(sc_symbolic *s, int precision, sc_numeric **out) {
         if ((rc = upload(h->d_tmap_of_sn, tmap_of_sn, bytes))) return fail(rc);
     }
     Plan P;
-    // one persistent launch per level: SIMT precisions, RLB schedule
     const Knobs kn = knobs_of(s->tune);
-    h->fused = kn.fused && s->opt.variant == SC_RLB && (precision == SC_FP64 || precision == SC_FP32);
+    h->fused = fused_plan(s, precision);
     // lookahead needs concurrent work: the captured graph's branches, or the fused launches
     h->lookahead = (h->use_graph || h->fused) && s->opt.variant == SC_RLB && kn.lookahead;
-    build_plan(s, precision, P, h->lookahead);
+    build_plan(s, precision, P, h->lookahead, !h->fused);
+    if (!P.splits.empty()) {
+        // the slice pool; without room for it (or with more rows than a tensor map's
+        // coordinate reaches) every FP64 product stays on the SIMT tiles
+        const size_t pool = (size_t)P.slice_pieces * sp::BK * sizeof(uint16_t);
+        if (P.slice_pieces > INT32_MAX || cudaMalloc((void **)&h->d_slices, pool) != cudaSuccess ||
+            cudaMalloc((void **)&h->d_exps, (size_t)P.exps * sizeof(int32_t)) != cudaSuccess) {
+            cudaGetLastError();
+            if (h->d_slices) cudaFree(h->d_slices);
+            h->d_slices = nullptr;
+            P = Plan();
+            build_plan(s, precision, P, h->lookahead, false);
+        } else {
+            bytes += (int64_t)pool + P.exps * (int64_t)sizeof(int32_t);
+            std::vector<CUtensorMap> maps;
+            if ((rc = split_encode_maps(h->d_slices, P.slice_pieces, maps))) return fail(rc);
+            if ((rc = upload(h->d_slice_maps, maps, bytes))) return fail(rc);
+            if ((rc = upload(h->d_splits, P.splits, bytes))) return fail(rc);
+            if ((rc = upload(h->d_split_units, P.split_units, bytes))) return fail(rc);
+            if ((rc = upload(h->d_split_of_task, P.split_of_task, bytes))) return fail(rc);
+        }
+    }
     if (h->fused) {
         build_flow(P, h->lookahead);
         h->flow_tail_off = P.flow_tail_off;
@@ -1006,7 +1202,8 @@ void numeric_free(sc_numeric *h) {
                     h->d_loops, h->d_tmaps, h->d_tmap_of_sn, h->d_err, h->d_inv, h->d_x, h->d_r, h->d_b, h->d_xbest, h->d_y, h->d_z, h->d_acc, h->d_red,
                     h->d_dep_ptr, h->d_dep, h->d_sync, h->d_serr, h->d_hi, h->d_lo, h->d_thin,
                     h->d_cgz, h->d_cgp, h->d_cgq, h->d_cgs, h->d_solve_units, h->d_flow, h->d_flow_ctr,
-                    h->d_flow_need, h->d_task_chunk, h->d_sn_chunk};
+                    h->d_flow_need, h->d_task_chunk, h->d_sn_chunk, h->d_splits, h->d_split_units, h->d_split_of_task,
+                    h->d_slices, h->d_exps, h->d_slice_maps};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (h->sym) h->sym->refs--;

@@ -18,7 +18,8 @@ struct ProdLists {
     int32_t tc64_off = 0, tc64_cnt = 0;     // GemmTile (tensor cores, 64-column tiles)
     int32_t tc256_off = 0, tc256_cnt = 0;   // GemmTile (tensor cores, 256-column tiles)
     int32_t thin_off = 0, thin_cnt = 0;     // ThinUnits of tasks with min(m, n) <= 8 (warp-block kernel)
-    bool any() const { return gemm_cnt || tc_cnt || tc64_cnt || tc256_cnt || thin_cnt; }
+    int32_t sp_off = 0, sp_cnt = 0;         // GemmTile (FP64 on the tensor cores: slice products)
+    bool any() const { return gemm_cnt || tc_cnt || tc64_cnt || tc256_cnt || thin_cnt || sp_cnt; }
 };
 
 // Launch plan of one level: offsets/counts into the flat device work lists.
@@ -29,7 +30,9 @@ struct LevelPlan {
     int32_t trsm_off = 0, trsm_cnt = 0;     // TrsmTile
     ProdLists crit, rest;
     int32_t small_off = 0, small_cnt = 0;   // task ids (warp kernel)
+    int32_t split_off = 0, split_cnt = 0;   // SplitUnit: source rows cut into FP16 slices (FP64)
     int32_t rlg_off = 0, rlg_cnt = 0;       // GemmTile of RL update matrices
+    int32_t rlsp_off = 0, rlsp_cnt = 0;     // GemmTile of RL update matrices (FP64 on the tensor cores)
     int32_t rls_off = 0, rls_cnt = 0;       // task ids of small RL update matrices
     int32_t loop_off = 0, loop_cnt = 0;     // LoopItem (device-side RLB loops), one CTA per item
     int32_t loopw_off = 0, loopw_cnt = 0;   // LoopItem of supernodes narrower than 32 columns, one warp per item
@@ -84,6 +87,14 @@ struct sc_numeric {
     float *d_lo = nullptr;            // SC_TF32X3: tf32(x - hi)
     int32_t nmaps = 0;                // panels with tensor maps (lo maps follow hi maps for SC_TF32X3)
     int32_t *d_rlrelind = nullptr;
+    // FP64 products on the tensor cores: source blocks, splitting units, the block of
+    // each task, the slice pool (one half per parity of the level), row exponents
+    sc::SplitBlk *d_splits = nullptr;
+    sc::SplitUnit *d_split_units = nullptr;
+    int32_t *d_split_of_task = nullptr;
+    uint16_t *d_slices = nullptr;
+    int32_t *d_exps = nullptr;
+    CUtensorMap *d_slice_maps = nullptr;
     // solve
     int32_t *d_glbind = nullptr;
     int32_t *d_perm = nullptr;

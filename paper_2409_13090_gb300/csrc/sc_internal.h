@@ -99,6 +99,16 @@ inline int tc_route_width(const Task &t, int src_width, int min_k, int wide_n, b
     return 0;
 }
 
+// Does an FP64 product run on the tensor cores as products of FP16 slices
+// (split_gemm.cuh)? The source panel needs 16-byte aligned rows (|J| >= 16: row
+// stride a multiple of 4, panel 256-byte aligned; kx0 even), K >= 16, and enough
+// work: a tile of slice products takes some 6 us, the time in which an SM's FP64
+// pipe makes about 24,000 multiply-adds.
+constexpr double kSplitMinWork = 32768;
+inline bool split_route(const Task &t, int src_width) {
+    return src_width >= 16 && t.k >= 16 && t.kx0 % 2 == 0 && (double)t.m * t.n * t.k >= kSplitMinWork;
+}
+
 // Field ranges of sc_tune_table (0 = default everywhere).
 inline bool tune_valid(const sc_tune_table &t) {
     auto in = [](int32_t v, int32_t lo, int32_t hi) { return v == 0 || (v >= lo && v <= hi); };
@@ -217,5 +227,11 @@ int build_schedule(sc_symbolic *s);
 // a target row of an RL assembly pair not owned by exactly one slab of its
 // target, or a slab whose pairs are not one target's in source order.
 int det_plan_check(const sc_symbolic *s, int64_t *bad_level);
+// 14 when an FP64 plan's source blocks of tensor-core products (split_gemm.cuh)
+// are wrong (0 if none are; the level in *bad_level): a product's rows or columns
+// not in its block, a block not of the product's level or misaligned, rows of a block not split
+// exactly once, slices of two blocks of a level overlapping, or the slices of
+// levels of different parity not apart.
+int split_plan_check(const sc_symbolic *s, int64_t *bad_level);
 int compose_relind(const int32_t *rJC, int64_t lenJC, const int32_t *rCP, int64_t lenCP, int32_t *out);
 }  // namespace sc

@@ -465,11 +465,8 @@ inline void tc_tiles_of(const Task &t, int32_t id, int bn, std::vector<GemmTile>
         }
 }
 
-// Encodes two 2D tensor maps per panel of width >= 16 (dims {ld_J, m_J}, boxes
-// {32, 128} and {32, 64}, 128-byte swizzle, zero fill outside the panel):
-// maps[2 * tmap_of_sn[J]] and maps[2 * tmap_of_sn[J] + 1].
-inline int tc_encode_maps(const sc_symbolic *s, float *d_lnz, std::vector<CUtensorMap> &maps,
-                          std::vector<int32_t> &tmap_of_sn) {
+// cuTensorMapEncodeTiled of the driver; NULL when it has none
+inline PFN_cuTensorMapEncodeTiled_v12000 tc_map_encoder() {
     static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
     if (!encode) {
         void *fn = nullptr;
@@ -477,9 +474,19 @@ inline int tc_encode_maps(const sc_symbolic *s, float *d_lnz, std::vector<CUtens
         if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) !=
                 cudaSuccess ||
             q != cudaDriverEntryPointSuccess || !fn)
-            return SC_ERR_CUDA;
+            return nullptr;
         encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
     }
+    return encode;
+}
+
+// Encodes two 2D tensor maps per panel of width >= 16 (dims {ld_J, m_J}, boxes
+// {32, 128} and {32, 64}, 128-byte swizzle, zero fill outside the panel):
+// maps[2 * tmap_of_sn[J]] and maps[2 * tmap_of_sn[J] + 1].
+inline int tc_encode_maps(const sc_symbolic *s, float *d_lnz, std::vector<CUtensorMap> &maps,
+                          std::vector<int32_t> &tmap_of_sn) {
+    PFN_cuTensorMapEncodeTiled_v12000 encode = tc_map_encoder();
+    if (!encode) return SC_ERR_CUDA;
     tmap_of_sn.assign(s->nsuper, -1);
     maps.clear();
     for (int64_t J = 0; J < s->nsuper; J++) {

@@ -1,0 +1,102 @@
+"""FP64 products on the tensor cores as products of FP16 slices (needs a GB300).
+
+The sizes are the edges of the path: inner dimensions around a 32-column stage
+and around the 128 columns between two drains of the accumulators, row and
+column counts around the 128 x 64 tile, chunk widths that start a product's
+columns at 24 (16-byte aligned) or 33 (not: such products stay on the SIMT
+tiles), rows of very different scale, and a row holding a NaN.
+
+Tolerance: a factor entry is sqrt-sized against its row, |L_ij| <= sqrt(a_ii); the
+oracle's own rounding of n sequential multiply-adds is below n u sqrt(a_ii), so the
+two agree within 2 n u sqrt(a_ii) (n <= 700, u = 2^-53: 1.6e-13), here 1e-12.
+"""
+import numpy as np
+import pytest
+
+import oracle
+import paper_2409_13090_gb300 as sc
+from paper_2409_13090_gb300 import inputs
+from tests.test_gpu_tc import _dense
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-12
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    sc.build()
+    oracle.build()
+
+
+def _row_scale(A):
+    d = A.values[A.colptr[:-1]]  # natural ordering: the diagonal is first in its column
+    return np.sqrt(d)[np.repeat(np.arange(A.n), A.n)]
+
+
+def _factors(A, **kw):
+    sym = sc.Symbolic(A, ordering="natural", **kw)
+    assert sym.check_schedule()["ok"]
+    num = sym.factor(A.values, precision="fp64")
+    return sym, num, num.profile(A.values)["gemm_tc"]["launches"]
+
+
+@pytest.mark.parametrize("chunk", [64, 24, 33])
+@pytest.mark.parametrize("n", [97, 128, 129, 191, 193, 257, 320, 385, 700])
+def test_dense_sizes_around_the_tiles(n, chunk):
+    A = _dense(n, n)
+    sym, num, launches = _factors(A, chunk=chunk)
+    assert num.rc == 0 and (launches > 0 or n < 128)
+    o = oracle.Oracle(A, None, pr=True)
+    assert o.factor() == 0
+    err = np.abs(num.export_L() - o.L_supernodal())
+    assert (err <= TOL * _row_scale(A)).all(), err.max()
+
+
+def test_rows_of_very_different_scale():
+    """D A D with D = 2^-60 .. 2^60 in random order: the factor is D L, every row
+    to the accuracy of its own scale (the scaling itself is exact)."""
+    A = _dense(300, 5)
+    d = 2.0 ** np.random.default_rng(3).integers(-60, 61, size=A.n)
+    cols = np.repeat(np.arange(A.n), np.diff(A.colptr))
+    A.values *= d[A.rowind] * d[cols]
+    _, num, launches = _factors(A)
+    assert num.rc == 0 and launches > 0
+    o = oracle.Oracle(A, None, pr=True)
+    assert o.factor() == 0
+    err = np.abs(num.export_L() - o.L_supernodal())
+    assert (err <= TOL * _row_scale(A)).all()
+
+
+def test_nan_reaches_the_pivot():
+    """A NaN in A's first column at row 200 of 300: rows below row 200 and the
+    pivot of column 201 (1-based) see it, the columns before do not."""
+    A = _dense(300, 6)
+    v = A.values.copy()
+    v[A.colptr[0] + 200] = np.nan
+    sym = sc.Symbolic(A, ordering="natural")
+    num = sym.factor(v, precision="fp64")
+    assert num.rc == 201
+    good = sym.factor(A.values, precision="fp64")
+    L, G = num.export_L().reshape(300, 300), good.export_L().reshape(300, 300)
+    assert np.abs(L[:200, :200] - G[:200, :200]).max() <= TOL * np.abs(G).max()
+
+
+@pytest.mark.parametrize("variant", ["rlb", "rl"])
+def test_irregular_updates_between_supernodes(variant):
+    """Products into ancestors (atomic adds, or update matrices stored and then
+    assembled) of a 3D 27-point matrix, merged and not."""
+    A = inputs.stencil_3d_27pt(13, 11, 12, seed=9)
+    for merge in (0.0, 0.3):
+        sym = sc.Symbolic(A, ordering="grid_nd", grid=A.grid, variant=variant, merge=merge)
+        assert sym.check_schedule()["ok"]
+        num = sym.factor(A.values, precision="fp64")
+        p = num.profile(A.values)
+        assert num.rc == 0 and p["gemm_tc"]["launches"] > 0
+        o = oracle.Oracle(A, oracle.nd_grid(*A.grid, 8), pr=True, merge=merge)
+        assert o.factor() == 0
+        Lo = o.L_supernodal()
+        num.refactor(A.values)
+        assert np.abs(num.export_L() - Lo).max() <= TOL * np.abs(Lo).max()
