@@ -67,6 +67,7 @@ SC_HD inline int block_rows(int rows, int nb, int ni_min, bool lower) {
 }
 
 constexpr int kMaxChunk = 64;
+constexpr int kNarrowChunk = 16;  // solve tiles of chunks up to this width take a warp, wider ones a CTA
 
 // Supernode descriptor for the device-side RLB loops.
 struct SnDev {

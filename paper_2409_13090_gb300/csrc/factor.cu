@@ -83,6 +83,66 @@ __global__ void __launch_bounds__(256) k_inverse(const float *__restrict__ lnz, 
 }
 
 
+// FP64 inverses of the factored diagonal blocks of the chunks wider than
+// kNarrowChunk, for the solve sweeps of FP64 factors: L_cc in 16 x 16 blocks; the
+// diagonal ones by substitution (a warp each, a lane per column), then block
+// diagonal by block diagonal W_ij = -W_ii sum_{j <= k < i} L_ik W_kj. Bound by the
+// FP64 pipe (some 41,000 clocks a block and SM).
+constexpr int kInv64Smem = 2 * kMaxChunk * (kMaxChunk + 1) * 8;
+__global__ void __launch_bounds__(256) k_inverse64(const double *__restrict__ lnz, const ChunkDev *__restrict__ chunks,
+                                                   const int32_t *__restrict__ list, double *__restrict__ inv) {
+    extern __shared__ double smem_potrf[];
+    __shared__ double rinv[kMaxChunk];
+    const ChunkDev ch = chunks[list[blockIdx.x]];
+    const int w = ch.w;
+    if (w <= kNarrowChunk) return;
+    auto l = reinterpret_cast<double (*)[kMaxChunk + 1]>(smem_potrf);
+    auto v = l + kMaxChunk;
+    load_block(l, lnz + ch.off + (int64_t)ch.c0 * ch.ld + ch.c0, ch.ld, w);
+    __syncthreads();
+    if (threadIdx.x < kMaxChunk) rinv[threadIdx.x] = threadIdx.x < w ? 1.0 / l[threadIdx.x][threadIdx.x] : 0.0;
+    __syncthreads();
+    const int nbk = (w + 15) / 16;
+    if ((int)threadIdx.x / 32 < nbk && threadIdx.x % 32 < 16) {
+        const int o = threadIdx.x / 32 * 16, j = threadIdx.x % 32;
+        double x[16];
+#pragma unroll
+        for (int i = 0; i < 16; i++) {
+            double s = i == j ? 1.0 : 0.0;
+#pragma unroll
+            for (int t = 0; t < i; t++) s -= l[o + i][o + t] * x[t];
+            x[i] = s * rinv[o + i];
+        }
+#pragma unroll
+        for (int i = 0; i < 16; i++) v[o + i][o + j] = i >= j ? x[i] : 0.0;
+    }
+    __syncthreads();
+    for (int d = 1; d < nbk; d++) {
+        const int total = (nbk - d) * 256;
+        // the sums, in the (unused) transposed place
+        for (int e = threadIdx.x; e < total; e += 256) {
+            const int bj = e / 256, bi = bj + d, r = e / 16 % 16, c = e % 16;
+            double s = 0.0;
+            for (int k = 16 * bj; k < 16 * bi; k++) s += l[16 * bi + r][k] * v[k][16 * bj + c];
+            v[16 * bj + r][16 * bi + c] = s;
+        }
+        __syncthreads();
+        for (int e = threadIdx.x; e < total; e += 256) {
+            const int bj = e / 256, bi = bj + d, r = e / 16 % 16, c = e % 16;
+            double s = 0.0;
+#pragma unroll
+            for (int k = 0; k < 16; k++) s -= v[16 * bi + r][16 * bi + k] * v[16 * bj + k][16 * bi + c];
+            v[16 * bi + r][16 * bj + c] = s;
+        }
+        __syncthreads();
+    }
+    double *out = inv + ch.inv;
+    for (int e = threadIdx.x; e < w * w; e += 256) {
+        const int r = e / w, c = e % w;
+        out[e] = r >= c ? v[r][c] : 0.0;
+    }
+}
+
 // ---- one persistent launch per level (SIMT precisions, RLB)
 // Bounded wait until *flag >= target (acquire at GPU scope); gives up, setting
 // *err, after spin_limit polls or once another CTA has given up.
@@ -241,6 +301,18 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
     E();
     launches += 2;
     const double tau = s->opt.pivot_tau;
+    // diagonal-block inverses for the solve, all chunks in one launch
+    auto launch_inverses = [&]() {
+        const int32_t nch = (int32_t)s->chunks.size();
+        if (!nch) return;
+        B(kProfPotrf);
+        if constexpr (sizeof(T) == 4)
+            k_inverse<<<nch, 256, kPotrfSmem, st>>>((const float *)lnz, h->d_chunks, h->d_potrf, (float *)h->d_inv);
+        else
+            k_inverse64<<<nch, 256, kInv64Smem, st>>>((const double *)lnz, h->d_chunks, h->d_potrf, (double *)h->d_inv);
+        E();
+        launches++;
+    };
     if (h->fused && !prof) {
         // one persistent launch per level, then the tail of lookahead products
         const size_t nch = s->chunks.size(), nlev = h->plans.size();
@@ -261,13 +333,7 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
             k_level<T><<<grid, 256, kPotrfSmem, st>>>(a);
             launches++;
         }
-        if constexpr (sizeof(T) == 4) {
-            const int32_t nchk = (int32_t)s->chunks.size();
-            if (nchk) {
-                k_inverse<<<nchk, 256, kPotrfSmem, st>>>((const float *)lnz, h->d_chunks, h->d_potrf, (float *)h->d_inv);
-                launches++;
-            }
-        }
+        launch_inverses();
         SC_CUDA(cudaGetLastError());
         h->kernel_launches = launches;
         return SC_OK;
@@ -442,16 +508,7 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
         }
     }
     if (st3 && nlev) SC_CUDA(cudaStreamWaitEvent(st, h->ev_rest[(nlev - 1) % 2], 0));  // join the lookahead branch
-    if constexpr (sizeof(T) == 4) {
-        // diagonal-block inverses for the solve, all chunks in one launch
-        const int32_t nch = (int32_t)s->chunks.size();
-        if (nch) {
-            B(kProfPotrf);
-            k_inverse<<<nch, 256, kPotrfSmem, st>>>((const float *)lnz, h->d_chunks, h->d_potrf, (float *)h->d_inv);
-            E();
-            launches++;
-        }
-    }
+    launch_inverses();
     SC_CUDA(cudaGetLastError());
     h->kernel_launches = launches;
     return SC_OK;
@@ -462,6 +519,7 @@ int set_smem_attrs() {
     if (done) return SC_OK;
     SC_CUDA(cudaFuncSetAttribute(k_potrf<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPotrfSmem));
     SC_CUDA(cudaFuncSetAttribute(k_potrf<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPotrfSmem));
+    SC_CUDA(cudaFuncSetAttribute(k_inverse64, cudaFuncAttributeMaxDynamicSharedMemorySize, kInv64Smem));
     SC_CUDA(cudaFuncSetAttribute(k_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, kPotrfSmem));
     SC_CUDA(cudaFuncSetAttribute(k_level<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPotrfSmem));
     SC_CUDA(cudaFuncSetAttribute(k_level<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPotrfSmem));
@@ -968,6 +1026,8 @@ int numeric_create(sc_symbolic *s, int precision, sc_numeric **out) {
     // lookahead needs concurrent work: the captured graph's branches, or the fused launches
     h->lookahead = (h->use_graph || h->fused) && s->opt.variant == SC_RLB && kn.lookahead;
     build_plan(s, precision, P, h->lookahead, !h->fused);
+    if (cudaMalloc(&h->d_inv, (size_t)std::max<int64_t>(1, P.inv_size) * h->elt) != cudaSuccess) return fail(SC_ERR_OOM);
+    bytes += P.inv_size * (int64_t)h->elt;
     if (!P.splits.empty()) {
         // the slice pool; without room for it (or with more rows than a tensor map's
         // coordinate reaches) every FP64 product stays on the SIMT tiles
@@ -1008,11 +1068,6 @@ int numeric_create(sc_symbolic *s, int precision, sc_numeric **out) {
         const size_t words = nch * kFlowStride + P.levels.size() + 1;
         if (cudaMalloc((void **)&h->d_flow_ctr, words * sizeof(int32_t)) != cudaSuccess) return fail(SC_ERR_OOM);
         bytes += (int64_t)(words * sizeof(int32_t));
-    }
-    if (precision != SC_FP64) {
-        if (cudaMalloc(&h->d_inv, (size_t)std::max<int64_t>(1, P.inv_size) * sizeof(float)) != cudaSuccess)
-            return fail(SC_ERR_OOM);
-        bytes += P.inv_size * 4;
     }
     std::copy(P.class_flops, P.class_flops + kProfClasses, h->class_flops);
     h->plans = P.levels;

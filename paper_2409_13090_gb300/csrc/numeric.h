@@ -82,7 +82,7 @@ struct sc_numeric {
     CUtensorMap *d_tmaps = nullptr;   // one per panel of width >= 16 (SC_TF32)
     int32_t *d_tmap_of_sn = nullptr;
     int32_t *d_err = nullptr;         // nonzero after a bounded device wait gave up
-    void *d_inv = nullptr;            // FP32 inverses of the chunks' diagonal blocks (FP32 / TF32 factors)
+    void *d_inv = nullptr;            // inverses of the chunks' diagonal blocks, in the factor's precision (FP64: the wide ones)
     float *d_hi = nullptr;            // SC_TF32X3: tf32(x) of every final factor entry (same layout as Lnz)
     float *d_lo = nullptr;            // SC_TF32X3: tf32(x - hi)
     int32_t nmaps = 0;                // panels with tensor maps (lo maps follow hi maps for SC_TF32X3)

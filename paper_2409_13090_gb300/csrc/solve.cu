@@ -19,6 +19,7 @@
 
 #include "kernels.cuh"
 #include "numeric.h"
+#include "sweep64.cuh"
 
 namespace sc {
 
@@ -134,52 +135,6 @@ __global__ void k_perm_out(double *__restrict__ X, int64_t ldx, const T *__restr
     int r = (int)(i % nb);
     double *dst = X + (int64_t)(r0 + r) * ldx + perm[k];
     *dst = add ? *dst + (double)z[i] : (double)z[i];
-}
-
-// Stages the chunk's diagonal block L_cc and its reciprocal pivots, then scales
-// it for division-free substitution: scale_cols: l[j][k] = L_jk / L_kk (j > k,
-// forward); otherwise l[k][j] = L_kj / L_kk (j < k, backward).
-template <typename T>
-__device__ void load_diag(T (*l)[kMaxChunk + 1], T *rinv, const T *lnz, const ChunkDev &ch, bool scale_cols) {
-    stage_block(l, lnz + ch.off + (int64_t)ch.c0 * ch.ld + ch.c0, ch.ld, ch.w, ch.w);
-    __syncthreads();
-    if (threadIdx.x < ch.w) rinv[threadIdx.x] = T(1) / l[threadIdx.x][threadIdx.x];
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < ch.w * ch.w; idx += blockDim.x) {
-        const int r = idx / ch.w, c = idx % ch.w;
-        if (r > c) l[r][c] *= scale_cols ? rinv[c] : rinv[r];
-    }
-    __syncthreads();
-}
-
-// v[0..w) of one right-hand side held by a warp (lane i: entries i and i+32).
-// Forward substitution on the numerators u_k = x_k - sum_{q<k} L_kq v_q with
-// the column-scaled block M_jk = L_jk / L_kk: u_j -= M_jk u_k; then v = u / L_kk.
-// Each step's critical path is one shuffle and one FMA.
-template <typename T>
-__device__ void warp_lower_solve(const T (*m)[kMaxChunk + 1], const T *rinv, int w, T &x0, T &x1) {
-    const int lane = threadIdx.x % 32;
-    for (int k = 0; k < w; k++) {
-        const T uk = __shfl_sync(0xffffffffu, k < 32 ? x0 : x1, k & 31);
-        if (lane > k) x0 -= m[lane][k] * uk;
-        if (lane + 32 > k && lane + 32 < w) x1 -= m[lane + 32][k] * uk;
-    }
-    if (lane < w) x0 *= rinv[lane];
-    if (lane + 32 < w) x1 *= rinv[lane + 32];
-}
-
-// Backward substitution with L_cc^T on numerators, row-scaled block
-// M_kj = L_kj / L_kk: for k = w-1..0: t_j -= M_kj t_k (j < k); then z = t / L_kk.
-template <typename T>
-__device__ void warp_upper_solve(const T (*m)[kMaxChunk + 1], const T *rinv, int w, T &x0, T &x1) {
-    const int lane = threadIdx.x % 32;
-    for (int k = w - 1; k >= 0; k--) {
-        const T tk = __shfl_sync(0xffffffffu, k < 32 ? x0 : x1, k & 31);
-        if (lane < k) x0 -= m[k][lane] * tk;
-        if (lane + 32 < k) x1 -= m[k][lane + 32] * tk;
-    }
-    if (lane < w) x0 *= rinv[lane];
-    if (lane + 32 < w) x1 *= rinv[lane + 32];
 }
 
 // Thread mapping of the sweeps' block products (256 threads over a 64-row
@@ -316,7 +271,7 @@ __device__ __forceinline__ int grab_tile(int32_t *work, int total, int32_t *err,
 // ---- tiles of narrow chunks (w <= kSmallW): one warp per tile, eight per CTA
 // (a SolveUnit with cnt > 0). v / z of the diagonal step are kept in a
 // per-warp shared-memory slice of kSmallW rows of ldv values.
-constexpr int kSmallW = 16;
+constexpr int kSmallW = kNarrowChunk;
 
 // Forward step of one narrow tile by one warp: wait for the chunk's arrivals,
 // v = L_cc^{-1} x_c (stored FP32 inverse, or substitution per right-hand side
@@ -466,7 +421,7 @@ struct SweepSmem {
 // its rows fall in. A tile only waits for tiles taken earlier (lower levels,
 // or its own chunk's first tile), so the sweep needs no co-residency.
 template <typename T, int RPT>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_fwd(const T *__restrict__ lnz, const ChunkDev *__restrict__ chunks,
+__global__ void __launch_bounds__(256, 3) k_fwd(const T *__restrict__ lnz, const ChunkDev *__restrict__ chunks,
                                              const TrsmTile *__restrict__ tiles, const SolveUnit *__restrict__ units,
                                              int total, const int32_t *__restrict__ dep_ptr,
                                              const int32_t *__restrict__ dep, const int32_t *__restrict__ need,
@@ -479,7 +434,6 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_fwd(const T *__
     extern __shared__ __align__(16) unsigned char smem_fwd[];
     const int ldv = rhs_ld(min(nrhs, kRhsBlk));
     SweepSmem<T> sm(smem_fwd, ldv);
-    __shared__ T rinv[kMaxChunk];
     __shared__ int s_t, s_ok;
     const int nblk = (nrhs + kRhsBlk - 1) / kRhsBlk;
     for (;;) {
@@ -555,15 +509,14 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_fwd(const T *__
         // loads that need no other tile: the tile's rows of L (and the diagonal block)
         stage_block(sm.lr, lnz + ch.off + (int64_t)tl.r0 * ch.ld + ch.c0, ch.ld, rows, w);
         if (first) {
-            if constexpr (sizeof(T) == 4) stage_block(sm.l, (const T *)(inv + ch.inv), w, w, w);
-            else load_diag(sm.l, rinv, lnz, ch, true);
+            stage_block(sm.l, inv + ch.inv, w, w, w);
             if (threadIdx.x == 0)
                 s_ok = wait_flag(arrive + (int64_t)tl.chunk * kSyncStride, need[tl.chunk], err, spin_limit, 5);
             __syncthreads();
             if (!s_ok) break;
             stage_rhs(sm.xin, ldv, x, nb, w, [&](int r) { return ch.col0 + r; });
             __syncthreads();
-            if constexpr (sizeof(T) == 4) {
+            {
                 // y_c = inv(L_cc) x_c: the block's stored inverse (zero above its diagonal)
                 const Map m;
                 if (m.row(0) < w && m.r0 < nb) {
@@ -578,21 +531,6 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_fwd(const T *__
                                 sm.v[k * ldv + m.r0 + j] = o[h][j];
                                 y[(int64_t)(ch.col0 + k) * nb + m.r0 + j] = o[h][j];
                             }
-                    }
-                }
-            } else {
-                const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
-                for (int r = warp; r < nb; r += blockDim.x / 32) {
-                    T u0 = lane < w ? sm.xin[lane * ldv + r] : T(0);
-                    T u1 = lane + 32 < w ? sm.xin[(lane + 32) * ldv + r] : T(0);
-                    warp_lower_solve(sm.l, rinv, w, u0, u1);
-                    if (lane < w) {
-                        sm.v[lane * ldv + r] = u0;
-                        y[(int64_t)(ch.col0 + lane) * nb + r] = u0;
-                    }
-                    if (lane + 32 < w) {
-                        sm.v[(lane + 32) * ldv + r] = u1;
-                        y[(int64_t)(ch.col0 + lane + 32) * nb + r] = u1;
                     }
                 }
             }
@@ -641,7 +579,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_fwd(const T *__
 // and marks the chunk done. Narrow chunks' warp tiles add and count, and the
 // last to finish solves.
 template <typename T, int RPT>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_bwd(const T *__restrict__ lnz, const ChunkDev *__restrict__ chunks,
+__global__ void __launch_bounds__(256, 3) k_bwd(const T *__restrict__ lnz, const ChunkDev *__restrict__ chunks,
                                              const TrsmTile *__restrict__ tiles, const SolveUnit *__restrict__ units,
                                              int total, const int32_t *__restrict__ dep_ptr,
                                              const int32_t *__restrict__ dep, const int32_t *__restrict__ ntiles,
@@ -654,7 +592,6 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_bwd(const T *__
     extern __shared__ __align__(16) unsigned char smem_bwd[];
     const int ldv = rhs_ld(min(nrhs, kRhsBlk));
     SweepSmem<T> sm(smem_bwd, ldv);
-    __shared__ T rinv[kMaxChunk];
     __shared__ int32_t grow[kSolveRows];
     __shared__ int s_t, s_ok;
     const int nblk = (nrhs + kRhsBlk - 1) / kRhsBlk;
@@ -739,8 +676,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_bwd(const T *__
 #pragma unroll
             for (int j = 0; j < Map::R; j++) o[h][j] = T(0);
         if (first) {
-            if constexpr (sizeof(T) == 4) stage_block(sm.l, (const T *)(inv + ch.inv), w, w, w);
-            else load_diag(sm.l, rinv, lnz, ch, false);
+            stage_block(sm.l, inv + ch.inv, w, w, w);
         }
         if (rows > 0) {
             if (threadIdx.x < rows) grow[threadIdx.x] = glbind[ch.gl + tl.r0 + threadIdx.x];
@@ -795,7 +731,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_bwd(const T *__
             }
         }
         __syncthreads();
-        if constexpr (sizeof(T) == 4) {
+        {
             // z_c = inv(L_cc)^T (y_c - acc_c) with the block's stored inverse
             if (m.row(0) < w && m.r0 < nb) {
                 T zo[Map::NR][Map::R];
@@ -808,20 +744,232 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_bwd(const T *__
                         if (k < w && m.r0 + j < nb) z[(int64_t)(ch.col0 + k) * nb + m.r0 + j] = zo[h][j];
                 }
             }
-        } else {
-            const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
-            for (int r = warp; r < nb; r += blockDim.x / 32) {
-                T u0 = lane < w ? sm.xin[lane * ldv + r] : T(0);
-                T u1 = lane + 32 < w ? sm.xin[(lane + 32) * ldv + r] : T(0);
-                warp_upper_solve(sm.l, rinv, w, u0, u1);
-                if (lane < w) z[(int64_t)(ch.col0 + lane) * nb + r] = u0;
-                if (lane + 32 < w) z[(int64_t)(ch.col0 + lane + 32) * nb + r] = u1;
-            }
         }
         __syncthreads();
         if (threadIdx.x == 0) {
             __threadfence();
             atomicExch(done + (int64_t)tl.chunk * kSyncStride, 1);
+        }
+    }
+}
+
+// ---- the sweeps of an FP64 factor: the same units, waits and releases as k_fwd
+// and k_bwd, products from digits (sweep64.cuh). NB: 8-column blocks of
+// right-hand sides per warp (1, 2, 4 for up to 16, 32, 64).
+struct Sweep64Args {
+    const double *lnz;
+    const ChunkDev *chunks;
+    const TrsmTile *tiles;
+    const SolveUnit *units;
+    int total;
+    const int32_t *dep_ptr, *dep;
+    const int32_t *count;  // forward: expected arrivals; backward: tiles per chunk
+    const int32_t *glbind;
+    double *x, *y, *z, *acc;
+    int nrhs;
+    int64_t vstride;
+    const double *inv;
+    int32_t *f0, *f1;  // forward: arrivals, ready; backward: tile counts, done
+    int64_t sstride;
+    int32_t *work, *err;
+    long long spin_limit;
+};
+
+template <int NB>
+__global__ void __launch_bounds__(256, 2) k_fwd64(Sweep64Args a) {
+    using Fr = fx::Frag<NB>;
+    extern __shared__ __align__(16) unsigned char smem_fwd64[];
+    uint64_t *tl_l = reinterpret_cast<uint64_t *>(smem_fwd64), *tl_w = tl_l + 64 * fx::kLd, *vec = tl_w + 64 * fx::kLd;
+    __shared__ int32_t e_l[64], e_w[64];
+    __shared__ int key[2][kRhsBlk];
+    __shared__ int s_t, s_ok;
+    const int ldv = rhs_ld(min(a.nrhs, kRhsBlk));
+    const int nblk = (a.nrhs + kRhsBlk - 1) / kRhsBlk;
+    for (;;) {
+        const int ug = grab_tile(a.work, a.total, a.err, &s_t);
+        if (ug >= a.total) break;
+        const int bk = ug % nblk;
+        const SolveUnit su = a.units[ug / nblk];
+        const int nb = min(kRhsBlk, a.nrhs - bk * kRhsBlk);
+        double *x = a.x + bk * a.vstride, *y = a.y + bk * a.vstride;
+        int32_t *arrive = a.f0 + bk * a.sstride, *ready = a.f1 + bk * a.sstride;
+        if (su.cnt > 0) {  // narrow tiles, one per warp
+            const int wp = threadIdx.x / 32;
+            if (wp < su.cnt) {
+                const int t = su.t0 + wp;
+                const TrsmTile tl = a.tiles[t];
+                const ChunkDev ch = a.chunks[tl.chunk];
+                fwd_tile_warp(a.lnz, ch, tl, t, a.dep_ptr, a.dep, a.count, a.glbind, x, y, nb, (const float *)nullptr,
+                              arrive, a.err, a.spin_limit, (double *)smem_fwd64 + wp * kSmallW * ldv, ldv);
+            }
+            __syncthreads();
+            continue;
+        }
+        // the tiles of one wide chunk: its first tile alone (cnt 0), or a run of further ones
+        const int c = a.tiles[su.t0].chunk;
+        const ChunkDev ch = a.chunks[c];
+        const int w = ch.w, g = su.cnt < 0 ? -su.cnt : 1;
+        auto stage = [&](int q) {
+            const int r0 = a.tiles[su.t0 + q].r0;
+            fx::stage_tile(tl_l, e_l, a.lnz + ch.off + (int64_t)r0 * ch.ld + ch.c0, ch.ld,
+                           max(0, min(kSolveRows, ch.m - r0)), w);
+        };
+        Fr v;
+        stage(0);
+        if (threadIdx.x < 2 * kRhsBlk) key[threadIdx.x / kRhsBlk][threadIdx.x % kRhsBlk] = fx::kKeyNone;
+        if (su.cnt == 0) {
+            fx::stage_tile(tl_w, e_w, a.inv + ch.inv, w, w, w);
+            if (threadIdx.x == 0)
+                s_ok = wait_flag(arrive + (int64_t)c * kSyncStride, a.count[c], a.err, a.spin_limit, 5);
+            __syncthreads();
+            if (!s_ok) break;
+            v.load(w, nb, [&](int r, int n) { return __ldcg(x + (int64_t)(ch.col0 + r) * nb + n); });
+            v.keys(nb, nullptr, key[1]);
+            __syncthreads();
+            v.put(nb, nullptr, key[1], vec);
+            __syncthreads();
+            v.template mul<false, false>(tl_w, e_w, vec, key[1], w, w, nb);  // y_c
+            v.each(w, nb, [&](int r, int n, double d) { y[(int64_t)(ch.col0 + r) * nb + n] = d; });
+        } else {
+            if (threadIdx.x == 0) s_ok = wait_flag(ready + (int64_t)c * kSyncStride, 1, a.err, a.spin_limit, 7);
+            __syncthreads();
+            if (!s_ok) break;
+            v.load(w, nb, [&](int r, int n) { return __ldcg(y + (int64_t)(ch.col0 + r) * nb + n); });
+        }
+        v.keys(nb, nullptr, key[0]);
+        __syncthreads();  // also: every warp is done with vec, and y_c is written
+        if (su.cnt == 0 && threadIdx.x == 0) {
+            // published as soon as it is written: the chunk's other tiles start
+            __threadfence();
+            atomicExch(ready + (int64_t)c * kSyncStride, 1);
+        }
+        v.put(nb, nullptr, key[0], vec);
+        __syncthreads();
+        for (int q = 0; q < g; q++) {
+            const int t = su.t0 + q, r0 = a.tiles[t].r0, rows = max(0, min(kSolveRows, ch.m - r0));
+            if (q > 0) {
+                stage(q);
+                __syncthreads();
+            }
+            Fr o;
+            o.template mul<false, false>(tl_l, e_l, vec, key[0], w, rows, nb);
+            o.each(rows, nb, [&](int r, int n, double d) { red_add(x + (int64_t)a.glbind[ch.gl + r0 + r] * nb + n, -d); });
+            // release: the barrier orders every thread's updates before thread 0's fence
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                __threadfence();
+                for (int p = a.dep_ptr[t]; p < a.dep_ptr[t + 1]; p++)
+                    atomicAdd(arrive + (int64_t)a.dep[p] * kSyncStride, 1);
+            }
+        }
+    }
+}
+
+template <int NB>
+__global__ void __launch_bounds__(256, 2) k_bwd64(Sweep64Args a) {
+    using Fr = fx::Frag<NB>;
+    extern __shared__ __align__(16) unsigned char smem_bwd64[];
+    uint64_t *tl_l = reinterpret_cast<uint64_t *>(smem_bwd64), *tl_w = tl_l + 64 * fx::kLd, *vec = tl_w + 64 * fx::kLd;
+    __shared__ int32_t e_l[64], e_w[64], grow[kSolveRows];
+    __shared__ int key[2][kRhsBlk];
+    __shared__ int s_t, s_ok;
+    const int ldv = rhs_ld(min(a.nrhs, kRhsBlk));
+    const int nblk = (a.nrhs + kRhsBlk - 1) / kRhsBlk;
+    for (;;) {
+        const int tr = grab_tile(a.work, a.total, a.err, &s_t);
+        if (tr >= a.total) break;
+        const int ug = a.total - 1 - tr;
+        const int bk = ug % nblk;
+        const SolveUnit su = a.units[ug / nblk];
+        const int nb = min(kRhsBlk, a.nrhs - bk * kRhsBlk);
+        const double *y = a.y + bk * a.vstride;
+        double *z = a.z + bk * a.vstride, *acc = a.acc + bk * a.vstride;
+        int32_t *cnt = a.f0 + bk * a.sstride, *done = a.f1 + bk * a.sstride;
+        if (su.cnt > 0) {  // narrow tiles, one per warp
+            const int wp = threadIdx.x / 32;
+            if (wp < su.cnt) {
+                const int t = su.t0 + wp;
+                const TrsmTile tl = a.tiles[t];
+                const ChunkDev ch = a.chunks[tl.chunk];
+                bwd_tile_warp(a.lnz, ch, tl, t, a.dep_ptr, a.dep, a.count, a.glbind, y, z, acc, nb,
+                              (const float *)nullptr, cnt, done, a.err, a.spin_limit,
+                              (double *)smem_bwd64 + wp * kSmallW * ldv, ldv);
+            }
+            __syncthreads();
+            continue;
+        }
+        // the chunk's first tile (cnt 0; it solves for z_c) or a run of further ones
+        const bool first = su.cnt == 0;
+        const int c = a.tiles[su.t0].chunk;
+        const ChunkDev ch = a.chunks[c];
+        const int w = ch.w, g = first ? 1 : -su.cnt;
+        if (first) fx::stage_tile(tl_w, e_w, a.inv + ch.inv, w, w, w);
+        if (threadIdx.x < 2 * kRhsBlk) key[threadIdx.x / kRhsBlk][threadIdx.x % kRhsBlk] = fx::kKeyNone;
+        Fr o;
+#pragma unroll
+        for (int b = 0; b < NB; b++)
+#pragma unroll
+            for (int e = 0; e < 4; e++) o.v[b][e] = 0.0;
+        bool ok = true;
+        for (int q = 0; q < g; q++) {
+            const int t = su.t0 + q, r0 = a.tiles[t].r0, rows = max(0, min(kSolveRows, ch.m - r0));
+            if (rows == 0) break;  // the last chunk of a root: nothing below
+            if (q > 0) __syncthreads();  // the previous tile and its vector are no longer read
+            if (threadIdx.x < rows) grow[threadIdx.x] = a.glbind[ch.gl + r0 + threadIdx.x];
+            fx::stage_tile(tl_l, e_l, a.lnz + ch.off + (int64_t)r0 * ch.ld + ch.c0, ch.ld, rows, w);
+            if (threadIdx.x == 0) {
+                bool k = true;
+                for (int p = a.dep_ptr[t]; p < a.dep_ptr[t + 1] && k; p++)
+                    k = wait_flag(done + (int64_t)a.dep[p] * kSyncStride, 1, a.err, a.spin_limit, 6);
+                s_ok = k;
+            }
+            __syncthreads();
+            if (!(ok = s_ok)) break;
+            Fr v;
+            v.load(rows, nb, [&](int r, int n) { return __ldcg(z + (int64_t)grow[r] * nb + n); });
+            v.keys(nb, e_l, key[q & 1]);
+            __syncthreads();
+            if (threadIdx.x < kRhsBlk) key[(q & 1) ^ 1][threadIdx.x] = fx::kKeyNone;  // the next tile's
+            v.put(nb, e_l, key[q & 1], vec);
+            __syncthreads();
+            o.template mul<true, true>(tl_l, nullptr, vec, key[q & 1], rows, w, nb);  // L_{rows,c}^T z_rows
+        }
+        if (!ok) break;
+        if (!first) {
+            o.each(w, nb, [&](int r, int n, double d) { red_add(acc + (int64_t)(ch.col0 + r) * nb + n, d); });
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                __threadfence();  // release this unit's contributions
+                atomicAdd(cnt + (int64_t)c * kSyncStride, g);
+            }
+            continue;
+        }
+        // the chunk's other tiles have added theirs into acc_c
+        if (threadIdx.x == 0)
+            s_ok = a.count[c] <= 1 || wait_flag(cnt + (int64_t)c * kSyncStride, a.count[c] - 1, a.err, a.spin_limit, 8);
+        __syncthreads();
+        if (!s_ok) break;
+        // z_c = L_cc^{-T} (y_c - acc_c - own part)
+        Fr v;
+        v.load(w, nb, [&](int r, int n) {
+            const int64_t i = (int64_t)(ch.col0 + r) * nb + n;
+            return __ldcg(y + i) - __ldcg(acc + i);
+        });
+#pragma unroll
+        for (int b = 0; b < NB; b++)
+#pragma unroll
+            for (int e = 0; e < 4; e++)
+                if (Fr::row(e) < w && Fr::col(b, e) < nb) v.v[b][e] -= o.v[b][e];
+        v.keys(nb, e_w, key[1]);  // key[1] is untouched since its reset (one tile at most came before)
+        __syncthreads();
+        v.put(nb, e_w, key[1], vec);
+        __syncthreads();
+        v.template mul<true, false>(tl_w, nullptr, vec, key[1], w, w, nb);
+        v.each(w, nb, [&](int r, int n, double d) { z[(int64_t)(ch.col0 + r) * nb + n] = d; });
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            atomicExch(done + (int64_t)c * kSyncStride, 1);
         }
     }
 }
@@ -988,7 +1136,6 @@ dim3 vec_grid(const sc_numeric *h, int64_t n, int64_t ncols) {
     return dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, per_col)), (unsigned)ncols);
 }
 
-template <typename T>
 int set_sweep_attrs();
 
 int ensure_solve(sc_numeric *h, int64_t nrhs) {
@@ -1126,7 +1273,7 @@ int ensure_solve(sc_numeric *h, int64_t nrhs) {
         // the two work counters
         if (cudaMalloc((void **)&h->d_serr, sizeof(int32_t)) != cudaSuccess) return SC_ERR_OOM;
         if (cudaMalloc((void **)&h->d_red, 4096 * sizeof(double)) != cudaSuccess) return SC_ERR_OOM;
-        if (set_sweep_attrs<double>() || set_sweep_attrs<float>()) return SC_ERR_CUDA;
+        if (set_sweep_attrs()) return SC_ERR_CUDA;
         h->solve_ready = true;
     }
     if (nrhs > h->solve_cap) {
@@ -1185,18 +1332,41 @@ void launch_sweeps(sc_numeric *h, int nrhs, int64_t vs, int64_t ss, T *xw, T *y,
                                            (const float *)h->d_inv, cnt, done, ss, work + 1, h->d_serr, spin);
 }
 
-template <typename T>
+template <int NB>
+void launch_sweeps64(sc_numeric *h, int nrhs, int64_t vs, int64_t ss, double *xw, double *y, double *z, double *acc,
+                     int32_t *sync, int nblk, cudaStream_t st) {
+    const size_t nch = h->sym->chunks.size();
+    const size_t smem = fx::sweep64_smem(std::min(nrhs, kRhsBlk));
+    int p = 1, q = 1;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, k_fwd64<NB>, 256, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, k_bwd64<NB>, 256, smem);
+    const int total = h->solve_tiles * nblk;
+    const int grid = std::max(1, std::min(total, std::max(1, std::min(p, q)) * h->num_sms));
+    Sweep64Args a{(const double *)h->d_lnz, h->d_chunks, h->d_solve_tiles, h->d_solve_units, total, h->d_dep_ptr,
+                  h->d_dep, h->d_counters + nch, h->d_glbind, xw, y, z, acc, nrhs, vs, (const double *)h->d_inv, sync,
+                  sync + nch * kSyncStride, ss, sync + nblk * ss, h->d_serr, (long long)h->sym->opt.spin_limit};
+    k_fwd64<NB><<<grid, 256, smem, st>>>(a);
+    a.count = h->d_counters;
+    a.f0 = sync + 2 * nch * kSyncStride;
+    a.f1 = sync + 3 * nch * kSyncStride;
+    a.work++;
+    k_bwd64<NB><<<grid, 256, smem, st>>>(a);
+}
+
 int set_sweep_attrs() {
-    const int smem = (int)solve_smem<T>(kRhsBlk);
     cudaError_t e = cudaSuccess;
-    auto set = [&](const void *k) {
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    auto set = [&](const void *k, size_t smem) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     };
-    set((const void *)k_fwd<T, 1>), set((const void *)k_bwd<T, 1>);
-    set((const void *)k_fwd<T, 2>), set((const void *)k_bwd<T, 2>);
-    set((const void *)k_fwd<T, 4>), set((const void *)k_bwd<T, 4>);
-    set((const void *)k_fwd<T, 8>), set((const void *)k_bwd<T, 8>);
-    set((const void *)k_fwd<T, 16>), set((const void *)k_bwd<T, 16>);
+    const size_t s32 = solve_smem<float>(kRhsBlk), s64 = fx::sweep64_smem(kRhsBlk);
+    set((const void *)k_fwd<float, 1>, s32), set((const void *)k_bwd<float, 1>, s32);
+    set((const void *)k_fwd<float, 2>, s32), set((const void *)k_bwd<float, 2>, s32);
+    set((const void *)k_fwd<float, 4>, s32), set((const void *)k_bwd<float, 4>, s32);
+    set((const void *)k_fwd<float, 8>, s32), set((const void *)k_bwd<float, 8>, s32);
+    set((const void *)k_fwd<float, 16>, s32), set((const void *)k_bwd<float, 16>, s32);
+    set((const void *)k_fwd64<1>, s64), set((const void *)k_bwd64<1>, s64);
+    set((const void *)k_fwd64<2>, s64), set((const void *)k_bwd64<2>, s64);
+    set((const void *)k_fwd64<4>, s64), set((const void *)k_bwd64<4>, s64);
     return e == cudaSuccess ? 0 : 1;
 }
 
@@ -1219,12 +1389,19 @@ int tri_solve(sc_numeric *h, int64_t nrhs, const double *B, int64_t ldb, double 
     }
     SC_CUDA(cudaMemsetAsync(h->d_sync, 0, (nblk * ss + 2) * sizeof(int32_t), st));
     SC_CUDA(cudaMemsetAsync(acc, 0, (size_t)nblk * vs * sizeof(T), st));
-    switch (rhs_per_thread((int)std::min<int64_t>(nrhs, kRhsBlk))) {
-        case 1: launch_sweeps<T, 1>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st); break;
-        case 2: launch_sweeps<T, 2>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st); break;
-        case 4: launch_sweeps<T, 4>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st); break;
-        case 8: launch_sweeps<T, 8>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st); break;
-        default: launch_sweeps<T, 16>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st); break;
+    if constexpr (sizeof(T) == 8) {
+        const int64_t nbm = std::min<int64_t>(nrhs, kRhsBlk);
+        if (nbm <= 16) launch_sweeps64<1>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st);
+        else if (nbm <= 32) launch_sweeps64<2>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st);
+        else launch_sweeps64<4>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st);
+    } else {
+        switch (rhs_per_thread((int)std::min<int64_t>(nrhs, kRhsBlk))) {
+            case 1: launch_sweeps<float, 1>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st); break;
+            case 2: launch_sweeps<float, 2>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st); break;
+            case 4: launch_sweeps<float, 4>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st); break;
+            case 8: launch_sweeps<float, 8>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st); break;
+            default: launch_sweeps<float, 16>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st); break;
+        }
     }
     launches += 2;
     for (int bk = 0; bk < nblk; bk++) {

@@ -35,13 +35,14 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include "fx.cuh"
 #include "kernels.cuh"
 #include "tc_gemm.cuh"
 
 namespace sc {
 namespace sp {
+using namespace fx;
 
-constexpr int S = 8;                   // slices
 constexpr int BM = 128, BN = 64;       // tile
 constexpr int BK = 32;                 // columns of a stage: 64 bytes of FP16, one swizzle row
 constexpr int kDrain = 4;              // stages between two drains of the accumulators (128 columns)
@@ -55,7 +56,6 @@ constexpr int kEpiWarps = 16;                   // four per TMEM lane quarter, e
 constexpr int kThreads = 32 * (4 + kEpiWarps);  // producer warp, MMA warp, two idle warps, epilogue warps
 // 96 registers a thread. Eight epilogue warps with twice the entries spilled their
 // accumulators, and a spill goes to L2 here: the stages leave L1 some 30 KB.
-constexpr int32_t kBadExp = 1 << 20;            // exponent of a row that holds an infinity or a NaN
 
 // instruction descriptor: kind::f16, D = F32, A = B = F16, both K-major, M = 128, N = n
 __device__ __forceinline__ uint32_t idesc_f16(int n) {
@@ -88,23 +88,6 @@ __device__ __forceinline__ void tmem_ld_16x8(uint32_t taddr, uint32_t (&r)[4]) {
 }
 
 // --------------------------------------------------------------------- splitting
-// X = round(x 2^(62 - E)) + 0x8080808080808080 for a finite |x| < 2^E: its bytes,
-// the highest first, are the digits d_1 .. d_8 plus 128.
-__device__ __forceinline__ uint64_t split_bytes(double x, int E) {
-    const uint64_t b = (uint64_t)__double_as_longlong(x);
-    const int ex = (int)(b >> 52) & 0x7ff;
-    uint64_t m = b & 0xFFFFFFFFFFFFFull;
-    if (ex) m |= 1ull << 52;
-    // x = m 2^(max(ex, 1) - 1075)
-    const int sh = max(ex, 1) - 1075 + 62 - E;  // <= 10
-    uint64_t X;
-    if (sh >= 0) X = m << sh;
-    else if (sh > -55) X = ((m >> (-sh - 1)) + 1) >> 1;  // to nearest
-    else X = 0;
-    if (b >> 63) X = 0 - X;
-    return X + 0x8080808080808080ull;
-}
-
 // One CTA of 256 threads splits 64 rows of a source block, four lanes per row
 // (8 columns of a 32-column piece each). Piece (kb, slice i, row r) is row
 // piece0 + (kb * S + i) * rows + r of the slice pool (32 FP16 values each).
@@ -173,54 +156,6 @@ __global__ void __launch_bounds__(256) k_split(const double *__restrict__ lnz, c
 // --------------------------------------------------------------------- product tiles
 __device__ __forceinline__ void red_sub(double *p, double a) {
     asm volatile("red.relaxed.gpu.global.add.f64 [%0], %1;" ::"l"(p), "d"(-a) : "memory");
-}
-
-// 96-bit accumulator (t: upper 64 bits, r: lower 32) of an entry, in units of 2^-68
-struct Acc96 {
-    int64_t t;
-    uint32_t r;
-};
-__device__ __forceinline__ int as_int(uint32_t v) { return __float2int_rn(__uint_as_float(v)); }
-// groups 1..4 of an entry: |g_1| <= 2^20, |g_2| <= 2^22, |g_3|, |g_4| <= 2^23, so
-// both pairs fit in 32 bits
-__device__ __forceinline__ void acc_add_high(Acc96 &a, uint32_t g1, uint32_t g2, uint32_t g3, uint32_t g4) {
-    const int p12 = as_int(g1) * 256 + as_int(g2), p34 = as_int(g3) * 256 + as_int(g4);
-    a.t += (int64_t)p12 * 65536 + p34;
-}
-// groups 5..8
-__device__ __forceinline__ void acc_add_low(Acc96 &a, uint32_t g5, uint32_t g6, uint32_t g7, uint32_t g8) {
-    const int64_t L =
-        (int64_t)as_int(g5) * (1 << 24) + ((int64_t)as_int(g6) * (1 << 16) + ((int64_t)as_int(g7) * 256 + as_int(g8)));
-    const uint32_t lo = (uint32_t)L, r = a.r + lo;
-    a.t += (L >> 32) + (r < lo ? 1 : 0);
-    a.r = r;
-}
-// the accumulator times 2^(e - 68), rounded to FP64, in integer operations (the
-// conversion of a 64-bit whole number and a scaling would go through the FP64 pipe)
-__device__ __forceinline__ double acc_value(const Acc96 &a, int e) {
-    // magnitude (m, r), then normalised: the highest bit of m at bit 62
-    const bool neg = a.t < 0;
-    uint64_t m = neg ? ~(uint64_t)a.t : (uint64_t)a.t;
-    uint32_t r = neg ? 0u - a.r : a.r;
-    if (neg && r == 0) m++;
-    int sc = e - 68 + 32;
-    if ((m >> 31) == 0) {  // 96 bits down to the lower 64
-        m = (m << 32) | r;
-        r = 0;
-        sc -= 32;
-    }
-    const int z = __clzll((long long)m) - 1;  // m < 2^63; at most 31 here unless r is 0
-    if (z == 63) return 0.0;
-    m = (m << z) | (z < 32 ? (uint64_t)(r >> 1) >> (31 - z) : 0ull);
-    if (z < 32 && (r << z)) m |= 1;  // whatever is below the last bit
-    // round to nearest even at bit 10: 53 bits from bit 62
-    m += 0x1ff + ((m >> 10) & 1);
-    m >>= 10;  // 2^52 <= m <= 2^53
-    sc += 62 - z;  // exponent of the highest bit
-    if (sc >= -1021 && sc <= 1022)
-        return __longlong_as_double((long long)((((uint64_t)(neg ? 2048 : 0) + (uint64_t)(sc + 1022)) << 52) + m));
-    const double d = scalbn((double)m, sc - 52);  // outside the normal range
-    return neg ? -d : d;
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
