@@ -69,6 +69,15 @@ SC_HD inline int block_rows(int rows, int nb, int ni_min, bool lower) {
 constexpr int kMaxChunk = 64;
 constexpr int kNarrowChunk = 16;  // solve tiles of chunks up to this width take a warp, wider ones a CTA
 
+// Is a chunk of w columns and `rows` rows below factored by one warp (k_narrow)?
+// FP32: up to 16 columns and 128 rows. FP64, where a warp's multiply-add takes 64 clocks:
+// while it has at most 200 of them in line (7 us; the CTA-wide POTRF and TRSM
+// take some 32 us in two launches) -- w^2 / 2 + 6 w for the pivots and w^2 / 2 for 32 rows.
+SC_HD inline bool narrow_chunk(int w, int rows, bool fp64) {
+    if (w > kNarrowChunk || rows > 128) return false;
+    return !fp64 || w * w / 2 * (1 + (rows + 31) / 32) + 6 * w <= 200;
+}
+
 // Supernode descriptor for the device-side RLB loops.
 struct SnDev {
     int64_t off;  // offset of Lnz(J)

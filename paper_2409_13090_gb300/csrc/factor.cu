@@ -8,6 +8,7 @@
 #include "kernels.cuh"
 #include "numeric.h"
 #include "split_gemm.cuh"
+#include "sweep64.cuh"
 #include "tc_gemm.cuh"
 
 namespace sc {
@@ -83,22 +84,32 @@ __global__ void __launch_bounds__(256) k_inverse(const float *__restrict__ lnz, 
 }
 
 
-// FP64 inverses of the factored diagonal blocks of the chunks wider than
-// kNarrowChunk, for the solve sweeps of FP64 factors: L_cc in 16 x 16 blocks; the
-// diagonal ones by substitution (a warp each, a lane per column), then block
-// diagonal by block diagonal W_ij = -W_ii sum_{j <= k < i} L_ik W_kj. Bound by the
-// FP64 pipe (some 41,000 clocks a block and SM).
-constexpr int kInv64Smem = 2 * kMaxChunk * (kMaxChunk + 1) * 8;
+// Inverses of the factored diagonal blocks of the chunks wider than kNarrowChunk, for
+// the solve sweeps of FP64 factors: L_cc in 16 x 16 blocks; the diagonal ones by
+// substitution (a warp each, a lane per column), then block diagonal by block
+// diagonal W_ij = -W_ii sum_{j <= k < i} L_ik W_kj, and one step W + W (I - L W) whose
+// products are formed from digits. Stored as the digits of W's rows (62 bits: the sum
+// before it is rounded to FP64) and the rows' exponents, so a product with W is
+// no further off than the substitution it stands for: with W in FP64 the solutions'
+// errors grew by up to a fifth. Bound by the FP64 pipe (some 41,000 clocks a block
+// and SM before the correction).
+constexpr int kInv64Smem = 8 * (2 * kMaxChunk * (kMaxChunk + 1) + 3 * kMaxChunk * fx::kLd);
 __global__ void __launch_bounds__(256) k_inverse64(const double *__restrict__ lnz, const ChunkDev *__restrict__ chunks,
-                                                   const int32_t *__restrict__ list, double *__restrict__ inv) {
+                                                   const int32_t *__restrict__ list, uint64_t *__restrict__ inv,
+                                                   int32_t *__restrict__ inv_exp) {
     extern __shared__ double smem_potrf[];
     __shared__ double rinv[kMaxChunk];
+    __shared__ int32_t e_l[kMaxChunk], e_w[kMaxChunk];
+    __shared__ int key[2][kMaxChunk];
     const ChunkDev ch = chunks[list[blockIdx.x]];
     const int w = ch.w;
-    if (w <= kNarrowChunk) return;
     auto l = reinterpret_cast<double (*)[kMaxChunk + 1]>(smem_potrf);
     auto v = l + kMaxChunk;
+    uint64_t *tl = reinterpret_cast<uint64_t *>(v + kMaxChunk), *tw = tl + kMaxChunk * fx::kLd,
+             *vec = tw + kMaxChunk * fx::kLd;
     load_block(l, lnz + ch.off + (int64_t)ch.c0 * ch.ld + ch.c0, ch.ld, w);
+    if (threadIdx.x < 2 * kMaxChunk) key[0][threadIdx.x] = fx::kKeyNone;
+    for (int e = threadIdx.x; e < kMaxChunk * (kMaxChunk + 1); e += 256) v[0][e] = 0.0;
     __syncthreads();
     if (threadIdx.x < kMaxChunk) rinv[threadIdx.x] = threadIdx.x < w ? 1.0 / l[threadIdx.x][threadIdx.x] : 0.0;
     __syncthreads();
@@ -119,7 +130,7 @@ __global__ void __launch_bounds__(256) k_inverse64(const double *__restrict__ ln
     __syncthreads();
     for (int d = 1; d < nbk; d++) {
         const int total = (nbk - d) * 256;
-        // the sums, in the (unused) transposed place
+        // the sums, in the transposed place
         for (int e = threadIdx.x; e < total; e += 256) {
             const int bj = e / 256, bi = bj + d, r = e / 16 % 16, c = e % 16;
             double s = 0.0;
@@ -136,11 +147,61 @@ __global__ void __launch_bounds__(256) k_inverse64(const double *__restrict__ ln
         }
         __syncthreads();
     }
-    double *out = inv + ch.inv;
-    for (int e = threadIdx.x; e < w * w; e += 256) {
-        const int r = e / w, c = e % w;
-        out[e] = r >= c ? v[r][c] : 0.0;
+    for (int e = threadIdx.x; e < kMaxChunk * kMaxChunk; e += 256)
+        if (e / kMaxChunk < e % kMaxChunk) v[e / kMaxChunk][e % kMaxChunk] = 0.0;
+    __syncthreads();
+    // W's columns as 64 right-hand sides: R = I - L W (the subtraction before the
+    // rounding), then the digits of W + W R
+    fx::stage_tile(tl, e_l, &l[0][0], kMaxChunk + 1, kMaxChunk, kMaxChunk);
+    fx::stage_tile(tw, e_w, &v[0][0], kMaxChunk + 1, kMaxChunk, kMaxChunk);
+    using Fr = fx::Frag<4>;
+    Fr f;
+    f.load(kMaxChunk, kMaxChunk, [&](int r, int c) { return v[r][c]; });
+    f.keys(kMaxChunk, nullptr, key[0]);
+    __syncthreads();
+    f.put(kMaxChunk, nullptr, key[0], vec);
+    __syncthreads();
+    const int mb = threadIdx.x / 32 % 4, ksteps = nbk;
+#pragma unroll
+    for (int b = 0; b < 4; b++) {
+        float acc[fx::S][4];
+        fx::product<false>(tl, vec, mb, Fr::n0(b), ksteps, acc);
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+            const int r = Fr::row(e), c = Fr::col(b, e), k = key[0][c], ex = e_l[r] + k - 1022;
+            fx::Acc96 a = fx::block_acc(acc, e);
+            // one, in units of 2^(ex - 68)
+            const int one = 68 - ex;
+            const bool fits = one >= 0 && one < 94;
+            if (r == c && fits) {
+                if (one >= 32) {
+                    a.t -= 1ll << (one - 32);
+                } else {
+                    const uint32_t d = 1u << one;
+                    a.t -= a.r < d ? 1 : 0;
+                    a.r -= d;
+                }
+            }
+            f.v[b][e] = r < w && c < w && fits && e_l[r] != fx::kBadExp && k != fx::kKeyBad ? -fx::acc_value(a, ex) : 0.0;
+        }
     }
+    f.keys(kMaxChunk, nullptr, key[1]);
+    __syncthreads();
+    f.put(kMaxChunk, nullptr, key[1], vec);
+    __syncthreads();
+    f.template mul<false, false>(tw, e_w, vec, key[1], w, w, kMaxChunk);
+    f.each(w, w, [&](int r, int c, double lo) {
+        const int E = e_w[r];
+        uint64_t X = 0x8080808080808080ull;
+        if (E != fx::kBadExp) {
+            X = fx::split_bytes(v[r][c], E);
+            // the correction only where it is one (far below W; not for a block whose
+            // condition is beyond FP64)
+            if (fabs(lo) < 0x1p-20 * scalbn(1.0, E)) X += fx::split_bytes(lo, E) - 0x8080808080808080ull;
+        }
+        inv[ch.inv + r * w + c] = X;
+    });
+    if ((int)threadIdx.x < w) inv_exp[ch.col0 + threadIdx.x] = e_w[threadIdx.x];
 }
 
 // ---- one persistent launch per level (SIMT precisions, RLB)
@@ -301,15 +362,17 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
     E();
     launches += 2;
     const double tau = s->opt.pivot_tau;
-    // diagonal-block inverses for the solve, all chunks in one launch
+    // diagonal-block inverses for the solve, all chunks but k_narrow's in one launch
     auto launch_inverses = [&]() {
-        const int32_t nch = (int32_t)s->chunks.size();
+        const int32_t nch = h->inv_cnt;
+        const int32_t *list = h->d_potrf + h->inv_off;
         if (!nch) return;
         B(kProfPotrf);
         if constexpr (sizeof(T) == 4)
-            k_inverse<<<nch, 256, kPotrfSmem, st>>>((const float *)lnz, h->d_chunks, h->d_potrf, (float *)h->d_inv);
+            k_inverse<<<nch, 256, kPotrfSmem, st>>>((const float *)lnz, h->d_chunks, list, (float *)h->d_inv);
         else
-            k_inverse64<<<nch, 256, kInv64Smem, st>>>((const double *)lnz, h->d_chunks, h->d_potrf, (double *)h->d_inv);
+            k_inverse64<<<nch, 256, kInv64Smem, st>>>((const double *)lnz, h->d_chunks, list, (uint64_t *)h->d_inv,
+                                                      h->d_inv_exp);
         E();
         launches++;
     };
@@ -394,6 +457,14 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
     const size_t nlev = h->plans.size();
     for (size_t lv = 0; lv < nlev; lv++) {
         const LevelPlan &p = h->plans[lv];
+        if (p.narrow_cnt) {
+            B(kProfPotrf);
+            k_narrow<T><<<(p.narrow_cnt + 7) / 8, 256, 0, st>>>(lnz, h->d_chunks, h->d_potrf + p.narrow_off,
+                                                                p.narrow_cnt, h->d_adiag, h->d_info, h->d_info + 1, tau,
+                                                                h->d_hi, h->d_lo, (T *)h->d_inv);
+            E();
+            launches++;
+        }
         if (p.potrf_cnt) {
             B(kProfPotrf);
             k_potrf<T><<<p.potrf_cnt, 256, kPotrfSmem, st>>>(lnz, h->d_chunks, h->d_potrf + p.potrf_off, h->d_adiag,
@@ -541,7 +612,9 @@ struct Plan {
     std::vector<RLSlab> rlslabs;
     std::vector<LoopItem> loops;
     std::vector<LevelPlan> levels;
+    bool fused = false;    // for the per-level kernel: no k_narrow chunks (set before build_plan)
     int64_t inv_size = 0;  // elements of the diagonal-block inverses
+    int32_t inv_off = 0, inv_cnt = 0;  // chunks of the inverse launch (in potrf)
     // FP64 products on the tensor cores (empty without them)
     std::vector<SplitBlk> splits;
     std::vector<SplitUnit> split_units;
@@ -617,16 +690,27 @@ void build_plan(const sc_symbolic *s, int precision, Plan &P, bool lookahead, bo
     for (size_t lv = 0; lv < s->levels.size(); lv++) {
         const Level &L = s->levels[lv];
         LevelPlan &p = P.levels[lv];
-        p.potrf_off = (int32_t)P.potrf.size();
+        // chunks narrow and short enough for one warp, then the others; the per-level
+        // kernel of a fused plan takes them all as the others
+        auto by_warp = [&](int32_t c) {
+            const ChunkDev &ch = P.cd[c];
+            return !P.fused && narrow_chunk(ch.w, ch.m - ch.c0 - ch.w, precision == SC_FP64);
+        };
+        p.narrow_off = (int32_t)P.potrf.size();
         for (int32_t c : L.chunks) {
-            P.potrf.push_back(c);
+            if (by_warp(c)) P.potrf.push_back(c);
             double w = P.cd[c].w;
             P.class_flops[kProfPotrf] += w * w * w / 3.0;
             P.class_flops[kProfTrsm] += (double)(P.cd[c].m - P.cd[c].c0 - P.cd[c].w) * w * w;
         }
+        p.narrow_cnt = (int32_t)P.potrf.size() - p.narrow_off;
+        p.potrf_off = (int32_t)P.potrf.size();
+        for (int32_t c : L.chunks)
+            if (!by_warp(c)) P.potrf.push_back(c);
         p.potrf_cnt = (int32_t)P.potrf.size() - p.potrf_off;
         p.trsm_off = (int32_t)P.trsm.size();
         for (int32_t c : L.chunks) {
+            if (by_warp(c)) continue;
             const ChunkDev &ch = P.cd[c];
             const int32_t rows = precision == SC_FP64 ? trsm_rows<double>() : trsm_rows<float>();
             for (int32_t r0 = ch.c0 + ch.w; r0 < ch.m; r0 += rows) P.trsm.push_back(TrsmTile{c, r0});
@@ -805,6 +889,15 @@ void build_plan(const sc_symbolic *s, int precision, Plan &P, bool lookahead, bo
             }
         }
     }
+    // the chunks that the inverse launch takes: all but k_narrow's (FP64: the sweeps
+    // substitute in the chunks up to kNarrowChunk)
+    P.inv_off = (int32_t)P.potrf.size();
+    for (const LevelPlan &p : P.levels)
+        for (int32_t i = 0; i < p.potrf_cnt; i++) {
+            const int32_t c = P.potrf[p.potrf_off + i];
+            if (precision != SC_FP64 || P.cd[c].w > kNarrowChunk) P.potrf.push_back(c);
+        }
+    P.inv_cnt = (int32_t)P.potrf.size() - P.inv_off;
     for (SplitBlk &bk : P.splits)
         if (bk.pad) {
             bk.piece0 += half_pieces[0];
@@ -941,6 +1034,7 @@ int split_plan_check(const sc_symbolic *s, int64_t *bad_level) {
 
 int plan_stats(const sc_symbolic *s, int precision, int64_t *out, int nout) {
     Plan P;
+    P.fused = true;  // every chunk counted with its TRSM tiles
     build_plan(s, precision, P, false, false);  // FP64: the products as the SIMT tiles they cover
     int64_t small_tasks = 0, tile_tasks = 0;
     for (const LevelPlan &l : P.levels) small_tasks += l.small_cnt + l.rls_cnt;
@@ -1022,12 +1116,16 @@ int numeric_create(sc_symbolic *s, int precision, sc_numeric **out) {
     }
     Plan P;
     const Knobs kn = knobs_of(s->tune);
-    h->fused = fused_plan(s, precision);
+    h->fused = P.fused = fused_plan(s, precision);
     // lookahead needs concurrent work: the captured graph's branches, or the fused launches
     h->lookahead = (h->use_graph || h->fused) && s->opt.variant == SC_RLB && kn.lookahead;
     build_plan(s, precision, P, h->lookahead, !h->fused);
     if (cudaMalloc(&h->d_inv, (size_t)std::max<int64_t>(1, P.inv_size) * h->elt) != cudaSuccess) return fail(SC_ERR_OOM);
     bytes += P.inv_size * (int64_t)h->elt;
+    if (precision == SC_FP64) {
+        if (cudaMalloc((void **)&h->d_inv_exp, (size_t)s->n * sizeof(int32_t)) != cudaSuccess) return fail(SC_ERR_OOM);
+        bytes += s->n * (int64_t)sizeof(int32_t);
+    }
     if (!P.splits.empty()) {
         // the slice pool; without room for it (or with more rows than a tensor map's
         // coordinate reaches) every FP64 product stays on the SIMT tiles
@@ -1071,6 +1169,8 @@ int numeric_create(sc_symbolic *s, int precision, sc_numeric **out) {
     }
     std::copy(P.class_flops, P.class_flops + kProfClasses, h->class_flops);
     h->plans = P.levels;
+    h->inv_off = P.inv_off;
+    h->inv_cnt = P.inv_cnt;
     h->ntasks = (int32_t)P.tasks.size();
     if ((rc = upload(h->d_chunks, P.cd, bytes))) return fail(rc);
     if ((rc = upload(h->d_potrf, P.potrf, bytes))) return fail(rc);
@@ -1258,7 +1358,7 @@ void numeric_free(sc_numeric *h) {
                     h->d_dep_ptr, h->d_dep, h->d_sync, h->d_serr, h->d_hi, h->d_lo, h->d_thin,
                     h->d_cgz, h->d_cgp, h->d_cgq, h->d_cgs, h->d_solve_units, h->d_flow, h->d_flow_ctr,
                     h->d_flow_need, h->d_task_chunk, h->d_sn_chunk, h->d_splits, h->d_split_units, h->d_split_of_task,
-                    h->d_slices, h->d_exps, h->d_slice_maps};
+                    h->d_slices, h->d_exps, h->d_slice_maps, h->d_inv_exp};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (h->sym) h->sym->refs--;

@@ -2,7 +2,7 @@
 // of digit products back to FP64: the arithmetic of the FP64 products on the tensor
 // cores (split_gemm.cuh: tcgen05 tiles; sweep64.cuh: warp-level MMAs of the solve).
 //
-// x with |x| < 2^E is the whole number X = round(x 2^(62 - E)), |X| <= 2^62,
+// x with |x| < 2^E is the whole number X = trunc(x 2^(62 - E)), |X| < 2^62,
 //   X = sum_{i = 1..8} d_i 256^(8 - i),  d_i in [-128, 127],  |d_1| <= 65.
 // A sum of products is
 //   sum_k x_k y_k = 2^(E_x + E_y) sum_{g = 1..8} 2^(-4 - 8 g) G_g,
@@ -20,21 +20,18 @@ namespace fx {
 constexpr int S = 8;  // digits
 constexpr int32_t kBadExp = 1 << 20; // exponent of a row or column that holds an infinity or a NaN
 
-// X = round(x 2^(62 - E)) + 0x8080808080808080 for a finite |x| < 2^E: its bytes,
-// the highest first, are the digits d_1 .. d_8 plus 128.
+// X + 0x8080808080808080 for a finite |x| < 2^E: its bytes, the highest first, are the
+// digits d_1 .. d_8 plus 128.
 __device__ __forceinline__ uint64_t split_bytes(double x, int E) {
-    const uint64_t b = (uint64_t)__double_as_longlong(x);
-    const int ex = (int)(b >> 52) & 0x7ff;
-    uint64_t m = b & 0xFFFFFFFFFFFFFull;
-    if (ex) m |= 1ull << 52;
-    // x = m 2^(max(ex, 1) - 1075)
-    const int sh = max(ex, 1) - 1075 + 62 - E;  // <= 10
-    uint64_t X;
-    if (sh >= 0) X = m << sh;
-    else if (sh > -55) X = ((m >> (-sh - 1)) + 1) >> 1;  // to nearest
-    else X = 0;
-    if (b >> 63) X = 0 - X;
-    return X + 0x8080808080808080ull;
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const int ex = (int)(hi >> 20) & 0x7ff;
+    // |x| = M 2^(max(ex, 1) - 1085), M < 2^63; X = M >> n (towards zero)
+    const uint32_t mh = (hi & 0xfffffu) | (ex ? 0x100000u : 0u);
+    const uint64_t M = ((uint64_t)mh << 42) | ((uint64_t)lo << 10);
+    const int n = E + 1023 - max(ex, 1);  // >= 1
+    const uint64_t X = n < 64 ? M >> n : 0;
+    const uint64_t s = (uint64_t)((int64_t)(int32_t)hi >> 31);  // all ones for a negative x
+    return (X ^ s) + (0x8080808080808080ull - s);
 }
 
 // 96-bit accumulator (t: upper 64 bits, r: lower 32) of an entry, in units of 2^-68
@@ -57,32 +54,39 @@ __device__ __forceinline__ void acc_add_low(Acc96 &a, uint32_t g5, uint32_t g6, 
     a.t += (L >> 32) + (r < lo ? 1 : 0);
     a.r = r;
 }
-// the accumulator times 2^(e - 68), rounded to FP64, in integer operations (the
-// conversion of a 64-bit whole number and a scaling would go through the FP64 pipe)
+// the accumulator times 2^(e - 68) when that is outside FP64's normal range
+static __device__ __noinline__ double acc_value_slow(int64_t t, uint32_t r, int e) {
+    return scalbn(scalbn((double)t, 32) + (double)r, e - 68);
+}
+// the accumulator times 2^(e - 68), rounded to FP64, in integer operations without
+// branches (a conversion of a 64-bit whole number and a scaling take the FP64 pipe 64
+// clocks each)
 __device__ __forceinline__ double acc_value(const Acc96 &a, int e) {
-    // magnitude (m, r), then normalised: the highest bit of m at bit 62
-    const bool neg = a.t < 0;
-    uint64_t m = neg ? ~(uint64_t)a.t : (uint64_t)a.t;
-    uint32_t r = neg ? 0u - a.r : a.r;
-    if (neg && r == 0) m++;
-    int sc = e - 68 + 32;
-    if ((m >> 31) == 0) {  // 96 bits down to the lower 64
-        m = (m << 32) | r;
-        r = 0;
-        sc -= 32;
+    // magnitude (one's complement: off by at most the last of the 96 bits)
+    const uint32_t s = (uint32_t)(a.t >> 63);
+    uint32_t w2 = (uint32_t)(a.t >> 32) ^ s, w1 = (uint32_t)a.t ^ s, w0 = a.r ^ s;
+    int sc = e - 68 + 32 + 62;
+    // whole words of leading zeros (up to bit 62 of the upper two words)
+#pragma unroll
+    for (int i = 0; i < 2; i++) {
+        const bool up = w2 == 0 && (w1 >> 31) == 0;
+        w2 = up ? w1 : w2;
+        w1 = up ? w0 : w1;
+        w0 = up ? 0u : w0;
+        sc -= up ? 32 : 0;
     }
-    const int z = __clzll((long long)m) - 1;  // m < 2^63; at most 31 here unless r is 0
-    if (z == 63) return 0.0;
-    m = (m << z) | (z < 32 ? (uint64_t)(r >> 1) >> (31 - z) : 0ull);
-    if (z < 32 && (r << z)) m |= 1;  // whatever is below the last bit
-    // round to nearest even at bit 10: 53 bits from bit 62
-    m += 0x1ff + ((m >> 10) & 1);
-    m >>= 10;  // 2^52 <= m <= 2^53
-    sc += 62 - z;  // exponent of the highest bit
-    if (sc >= -1021 && sc <= 1022)
-        return __longlong_as_double((long long)((((uint64_t)(neg ? 2048 : 0) + (uint64_t)(sc + 1022)) << 52) + m));
-    const double d = scalbn((double)m, sc - 52);  // outside the normal range
-    return neg ? -d : d;
+    const bool zero = (w2 | w1) == 0;
+    // w2 == 0 here means that bit 31 of w1 is set
+    const int z = w2 ? __clz((int)w2) - 1 : 31;
+    uint32_t hi = __funnelshift_l(w1, w2, z), lo = __funnelshift_l(w0, w1, z);
+    sc -= z;
+    // to nearest at bit 10: 53 bits from bit 62
+    const uint32_t l2 = lo + 0x200u;
+    hi += l2 < lo ? 1u : 0u;
+    const uint32_t mh = hi >> 10, ml = __funnelshift_r(l2, hi, 10);  // 2^52 <= (mh, ml) <= 2^53
+    if (zero) return 0.0;
+    if ((unsigned)(sc + 1021) > 2043u) return acc_value_slow(a.t, a.r, e);
+    return __hiloint2double((int)((mh + ((uint32_t)(sc + 1022) << 20)) | (s & 0x80000000u)), (int)ml);
 }
 
 }  // namespace fx

@@ -27,6 +27,7 @@ struct ProdLists {
 // `rest` the others, which may run concurrently with the next level.
 struct LevelPlan {
     int32_t potrf_off = 0, potrf_cnt = 0;   // chunk ids
+    int32_t narrow_off = 0, narrow_cnt = 0; // chunk ids (k_narrow: POTRF, rows below and inverse by one warp)
     int32_t trsm_off = 0, trsm_cnt = 0;     // TrsmTile
     ProdLists crit, rest;
     int32_t small_off = 0, small_cnt = 0;   // task ids (warp kernel)
@@ -82,7 +83,8 @@ struct sc_numeric {
     CUtensorMap *d_tmaps = nullptr;   // one per panel of width >= 16 (SC_TF32)
     int32_t *d_tmap_of_sn = nullptr;
     int32_t *d_err = nullptr;         // nonzero after a bounded device wait gave up
-    void *d_inv = nullptr;            // inverses of the chunks' diagonal blocks, in the factor's precision (FP64: the wide ones)
+    void *d_inv = nullptr;            // inverses of the chunks' diagonal blocks (FP64: the wide ones, as digits)
+    int32_t *d_inv_exp = nullptr;     // FP64: exponents of the inverses' rows, by column of the matrix
     float *d_hi = nullptr;            // SC_TF32X3: tf32(x) of every final factor entry (same layout as Lnz)
     float *d_lo = nullptr;            // SC_TF32X3: tf32(x - hi)
     int32_t nmaps = 0;                // panels with tensor maps (lo maps follow hi maps for SC_TF32X3)
@@ -130,6 +132,7 @@ struct sc_numeric {
     int64_t device_bytes = 0;
     // plan
     std::vector<sc::LevelPlan> plans;
+    int32_t inv_off = 0, inv_cnt = 0;    // chunk ids of the inverse launch after the last level (in d_potrf)
     int32_t ntasks = 0;
     int32_t kernel_launches = 0;
     double class_flops[sc::kProfClasses] = {};

@@ -274,8 +274,7 @@ __device__ __forceinline__ int grab_tile(int32_t *work, int total, int32_t *err,
 constexpr int kSmallW = kNarrowChunk;
 
 // Forward step of one narrow tile by one warp: wait for the chunk's arrivals,
-// v = L_cc^{-1} x_c (stored FP32 inverse, or substitution per right-hand side
-// in FP64), subtract L_{rows,c} v from x, count the arrivals. false when a wait
+// v = L_cc^{-1} x_c (stored FP32 inverse, or FP64 substitution), subtract L_{rows,c} v from x, count the arrivals. false when a wait
 // gave up.
 template <typename T>
 __device__ bool fwd_tile_warp(const T *__restrict__ lnz, const ChunkDev &ch, const TrsmTile &tl, int t,
@@ -286,10 +285,18 @@ __device__ bool fwd_tile_warp(const T *__restrict__ lnz, const ChunkDev &ch, con
     const int lane = threadIdx.x % 32, w = ch.w;
     const bool first = tl.r0 == ch.c0 + w;
     const int rows = max(0, min(kSolveRows, ch.m - tl.r0));
+    // FP64: lane j % 16 holds row j of L_cc below the diagonal and its reciprocal pivot
+    T lj[sizeof(T) == 8 ? kSmallW : 1], rj = T(0);
+    const T *dg = lnz + ch.off + (int64_t)ch.c0 * ch.ld + ch.c0;
+    if constexpr (sizeof(T) == 8) {
+        const int j = lane % 16;
+#pragma unroll
+        for (int k = 0; k < kSmallW; k++) lj[k] = j < w && k < j ? dg[(int64_t)j * ch.ld + k] : T(0);
+        if (j < w) rj = T(1) / dg[(int64_t)j * ch.ld + j];
+    }
     int ok = 1;
     if (lane == 0) ok = wait_flag(arrive + (int64_t)tl.chunk * kSyncStride, need[tl.chunk], err, spin_limit, 5);
     if (!__shfl_sync(0xffffffffu, ok, 0)) return false;
-    const T *dg = lnz + ch.off + (int64_t)ch.c0 * ch.ld + ch.c0;
     if constexpr (sizeof(T) == 4) {
         const float *iv = inv + ch.inv;
         for (int e = lane; e < w * nb; e += 32) {
@@ -299,13 +306,34 @@ __device__ bool fwd_tile_warp(const T *__restrict__ lnz, const ChunkDev &ch, con
             vw[k * ldv + r] = acc;
             if (first) y[(int64_t)(ch.col0 + k) * nb + r] = acc;
         }
-    } else {
-        for (int r = lane; r < nb; r += 32) {
+    } else if (nb > 8) {
+        // a right-hand side per lane
+        for (int r0 = 0; r0 < nb; r0 += 32) {
+            const int r = r0 + lane;
             for (int k = 0; k < w; k++) {
+                const T rk = __shfl_sync(0xffffffffu, rj, k);
+                if (r >= nb) continue;
                 T sum = __ldcg(x + (int64_t)(ch.col0 + k) * nb + r);
                 for (int q = 0; q < k; q++) sum -= dg[(int64_t)k * ch.ld + q] * vw[q * ldv + r];
-                vw[k * ldv + r] = sum / dg[(int64_t)k * ch.ld + k];
-                if (first) y[(int64_t)(ch.col0 + k) * nb + r] = vw[k * ldv + r];
+                vw[k * ldv + r] = sum * rk;
+                if (first) y[(int64_t)(ch.col0 + k) * nb + r] = sum * rk;
+            }
+        }
+    } else {
+        // a row per lane, two right-hand sides at a time
+        const int j = lane % 16;
+        for (int r0 = 0; r0 < nb; r0 += 2) {
+            const int r = r0 + lane / 16;
+            T s = j < w && r < nb ? __ldcg(x + (int64_t)(ch.col0 + j) * nb + r) : T(0);
+#pragma unroll
+            for (int k = 0; k < kSmallW; k++) {
+                if (k >= w) break;
+                const T yk = __shfl_sync(0xffffffffu, s * rj, (lane & 16) | k);
+                s = j == k ? yk : s - lj[k] * yk;
+            }
+            if (j < w && r < nb) {
+                vw[j * ldv + r] = s;
+                if (first) y[(int64_t)(ch.col0 + j) * nb + r] = s;
             }
         }
     }
@@ -361,7 +389,6 @@ __device__ bool bwd_tile_warp(const T *__restrict__ lnz, const ChunkDev &ch, con
         if (last) __threadfence();
     }
     if (!__shfl_sync(0xffffffffu, last, 0)) return true;
-    const T *dg = lnz + ch.off + (int64_t)ch.c0 * ch.ld + ch.c0;
     for (int e = lane; e < w * nb; e += 32) {
         const int k = e / nb, r = e % nb;
         const int64_t g = (int64_t)(ch.col0 + k) * nb + r;
@@ -377,13 +404,34 @@ __device__ bool bwd_tile_warp(const T *__restrict__ lnz, const ChunkDev &ch, con
             z[(int64_t)(ch.col0 + k) * nb + r] = sum;
         }
     } else {
-        for (int r = lane; r < nb; r += 32) {
+        // a column per lane, two right-hand sides at a time
+        const T *dg = lnz + ch.off + (int64_t)ch.c0 * ch.ld + ch.c0;
+        const int j = lane % 16;
+        T lj[kSmallW];
+#pragma unroll
+        for (int k = 0; k < kSmallW; k++) lj[k] = k < w && k > j ? dg[(int64_t)k * ch.ld + j] : T(0);
+        const T rj = j < w ? T(1) / dg[(int64_t)j * ch.ld + j] : T(0);
+        for (int r0 = 0; nb > 8 && r0 < nb; r0 += 32) {  // a right-hand side per lane
+            const int r = r0 + lane;
             for (int k = w - 1; k >= 0; k--) {
+                const T rk = __shfl_sync(0xffffffffu, rj, k);
+                if (r >= nb) continue;
                 T sum = vw[k * ldv + r];
                 for (int q = k + 1; q < w; q++) sum -= dg[(int64_t)q * ch.ld + k] * vw[q * ldv + r];
-                vw[k * ldv + r] = sum / dg[(int64_t)k * ch.ld + k];
-                z[(int64_t)(ch.col0 + k) * nb + r] = vw[k * ldv + r];
+                vw[k * ldv + r] = sum * rk;
+                z[(int64_t)(ch.col0 + k) * nb + r] = sum * rk;
             }
+        }
+        for (int r0 = 0; nb <= 8 && r0 < nb; r0 += 2) {
+            const int r = r0 + lane / 16;
+            T s = j < w && r < nb ? vw[j * ldv + r] : T(0);
+#pragma unroll
+            for (int k = kSmallW - 1; k >= 0; k--) {
+                if (k >= w) continue;
+                const T zk = __shfl_sync(0xffffffffu, s * rj, (lane & 16) | k);
+                s = j == k ? zk : s - lj[k] * zk;
+            }
+            if (j < w && r < nb) z[(int64_t)(ch.col0 + j) * nb + r] = s;
         }
     }
     __syncwarp();
@@ -768,7 +816,8 @@ struct Sweep64Args {
     double *x, *y, *z, *acc;
     int nrhs;
     int64_t vstride;
-    const double *inv;
+    const uint64_t *inv;  // digits of the inverses (k_inverse64)
+    const int32_t *inv_exp;
     int32_t *f0, *f1;  // forward: arrivals, ready; backward: tile counts, done
     int64_t sstride;
     int32_t *work, *err;
@@ -818,7 +867,7 @@ __global__ void __launch_bounds__(256, 2) k_fwd64(Sweep64Args a) {
         stage(0);
         if (threadIdx.x < 2 * kRhsBlk) key[threadIdx.x / kRhsBlk][threadIdx.x % kRhsBlk] = fx::kKeyNone;
         if (su.cnt == 0) {
-            fx::stage_tile(tl_w, e_w, a.inv + ch.inv, w, w, w);
+            fx::stage_inverse(tl_w, e_w, a.inv + ch.inv, a.inv_exp + ch.col0, w);
             if (threadIdx.x == 0)
                 s_ok = wait_flag(arrive + (int64_t)c * kSyncStride, a.count[c], a.err, a.spin_limit, 5);
             __syncthreads();
@@ -903,7 +952,7 @@ __global__ void __launch_bounds__(256, 2) k_bwd64(Sweep64Args a) {
         const int c = a.tiles[su.t0].chunk;
         const ChunkDev ch = a.chunks[c];
         const int w = ch.w, g = first ? 1 : -su.cnt;
-        if (first) fx::stage_tile(tl_w, e_w, a.inv + ch.inv, w, w, w);
+        if (first) fx::stage_inverse(tl_w, e_w, a.inv + ch.inv, a.inv_exp + ch.col0, w);
         if (threadIdx.x < 2 * kRhsBlk) key[threadIdx.x / kRhsBlk][threadIdx.x % kRhsBlk] = fx::kKeyNone;
         Fr o;
 #pragma unroll
@@ -1343,7 +1392,7 @@ void launch_sweeps64(sc_numeric *h, int nrhs, int64_t vs, int64_t ss, double *xw
     const int total = h->solve_tiles * nblk;
     const int grid = std::max(1, std::min(total, std::max(1, std::min(p, q)) * h->num_sms));
     Sweep64Args a{(const double *)h->d_lnz, h->d_chunks, h->d_solve_tiles, h->d_solve_units, total, h->d_dep_ptr,
-                  h->d_dep, h->d_counters + nch, h->d_glbind, xw, y, z, acc, nrhs, vs, (const double *)h->d_inv, sync,
+                  h->d_dep, h->d_counters + nch, h->d_glbind, xw, y, z, acc, nrhs, vs, (const uint64_t *)h->d_inv, h->d_inv_exp, sync,
                   sync + nch * kSyncStride, ss, sync + nblk * ss, h->d_serr, (long long)h->sym->opt.spin_limit};
     k_fwd64<NB><<<grid, 256, smem, st>>>(a);
     a.count = h->d_counters;

@@ -68,6 +68,24 @@ __device__ __forceinline__ void stage_tile(uint64_t *T, int32_t *rowE, const dou
                 : make_ulonglong2(split_bytes(v[2 * j], E), split_bytes(v[2 * j + 1], E));
 }
 
+// Stages the digits of a chunk's inverse (k_inverse64) and their row exponents.
+__device__ __forceinline__ void stage_inverse(uint64_t *T, int32_t *rowE, const uint64_t *__restrict__ inv,
+                                              const int32_t *__restrict__ exps, int w) {
+    constexpr int kIt = 64 * 64 / 256;
+    uint64_t v[kIt];
+#pragma unroll
+    for (int i = 0; i < kIt; i++) {
+        const int e = threadIdx.x + i * 256, r = e / 64, c = e % 64;
+        v[i] = r < w && c < w ? inv[r * w + c] : 0x8080808080808080ull;
+    }
+#pragma unroll
+    for (int i = 0; i < kIt; i++) {
+        const int e = threadIdx.x + i * 256;
+        T[e / 64 * kLd + e % 64] = v[i];
+    }
+    if (threadIdx.x < 64) rowE[threadIdx.x] = (int)threadIdx.x < w ? exps[threadIdx.x] : -1021;
+}
+
 // Digit s (0: the highest) of two staged values as FP16: 1024 + byte, less 1152.
 template <int s>
 __device__ __forceinline__ uint32_t digits(const ulonglong2 &x) {
@@ -135,15 +153,17 @@ __device__ __forceinline__ void product(const uint64_t *T, const uint64_t *V, in
         digit_row<7>(acc, x, b);
     }
 }
-// value of register e of a block's group sums, times 2^(er + ec)
+// register e of a block's group sums as one whole number
+__device__ __forceinline__ Acc96 block_acc(const float (&acc)[S][4], int e) {
+    // at most 64 terms: every pair of groups fits in 32 bits (|g_7| < 2^22.6)
+    auto pair = [&](int s) { return __float2int_rn(acc[s][e]) * 256 + __float2int_rn(acc[s + 1][e]); };
+    const int64_t H = ((int64_t)pair(0) << 16) + pair(2), L = ((int64_t)pair(4) << 16) + pair(6);
+    return Acc96{H + (L >> 32), (uint32_t)L};
+}
+// its value times 2^(er + ec)
 __device__ __forceinline__ double block_value(const float (&acc)[S][4], int e, int er, int ec) {
     if (er == kBadExp || ec == kBadExp) return __longlong_as_double(0x7ff8000000000000ll);
-    Acc96 a{0, 0};
-    acc_add_high(a, __float_as_uint(acc[0][e]), __float_as_uint(acc[1][e]), __float_as_uint(acc[2][e]),
-                 __float_as_uint(acc[3][e]));
-    acc_add_low(a, __float_as_uint(acc[4][e]), __float_as_uint(acc[5][e]), __float_as_uint(acc[6][e]),
-                __float_as_uint(acc[7][e]));
-    return acc_value(a, er + ec);
+    return acc_value(block_acc(acc, e), er + ec);
 }
 
 // A warp's part of a 64 x nb block of values, in the layout of the products: rows
