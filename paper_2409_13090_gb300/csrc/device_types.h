@@ -16,7 +16,7 @@ struct ChunkDev {
     int32_t c0;    // first local column of the chunk
     int32_t w;     // chunk width
     int32_t col0;  // global column of the chunk's first column
-    int32_t pad;
+    int32_t slot;  // FP64: offset of the chunk's digits (chunk64.cuh)
 };
 
 // One tile of the row-wise TRSM: rows [r0, min(r0+rows, m)) of chunk c.
@@ -67,6 +67,13 @@ SC_HD inline int block_rows(int rows, int nb, int ni_min, bool lower) {
 }
 
 constexpr int kMaxChunk = 64;
+// FP64 POTRF to TRSM: 256-word units of a chunk's digits -- L_cc, the inverses of its
+// 16 x 16 diagonal blocks, exponents.
+SC_HD inline int chunk64_units(int w) {
+    const int nb = (w + 15) / 16;
+    return nb * nb + nb + 1;
+}
+constexpr int kTrsm64Rows = 64;
 constexpr int kNarrowChunk = 16;  // solve tiles of chunks up to this width take a warp, wider ones a CTA
 
 // Is a chunk of w columns and `rows` rows below factored by one warp (k_narrow)?

@@ -8,6 +8,7 @@
 #include "kernels.cuh"
 #include "numeric.h"
 #include "split_gemm.cuh"
+#include "chunk64.cuh"
 #include "sweep64.cuh"
 #include "tc_gemm.cuh"
 
@@ -89,17 +90,17 @@ __global__ void __launch_bounds__(256) k_inverse(const float *__restrict__ lnz, 
 // substitution (a warp each, a lane per column), then block diagonal by block
 // diagonal W_ij = -W_ii sum_{j <= k < i} L_ik W_kj, and one step W + W (I - L W) whose
 // products are formed from digits. Stored as the digits of W's rows (62 bits: the sum
-// before it is rounded to FP64) and the rows' exponents, so a product with W is
-// no further off than the substitution it stands for: with W in FP64 the solutions'
+// before it is rounded to FP64), columns scaled, with the rows' exponents and minus the
+// columns', so a product with W is no further off than the substitution it stands for: with W in FP64 the solutions'
 // errors grew by up to a fifth. Bound by the FP64 pipe (some 41,000 clocks a block
 // and SM before the correction).
 constexpr int kInv64Smem = 8 * (2 * kMaxChunk * (kMaxChunk + 1) + 3 * kMaxChunk * fx::kLd);
 __global__ void __launch_bounds__(256) k_inverse64(const double *__restrict__ lnz, const ChunkDev *__restrict__ chunks,
                                                    const int32_t *__restrict__ list, uint64_t *__restrict__ inv,
-                                                   int32_t *__restrict__ inv_exp) {
+                                                   int32_t *__restrict__ inv_exp, int32_t *__restrict__ inv_cexp) {
     extern __shared__ double smem_potrf[];
     __shared__ double rinv[kMaxChunk];
-    __shared__ int32_t e_l[kMaxChunk], e_w[kMaxChunk];
+    __shared__ int32_t e_l[kMaxChunk], e_w[kMaxChunk], e_c[kMaxChunk], e_n[kMaxChunk];
     __shared__ int key[2][kMaxChunk];
     const ChunkDev ch = chunks[list[blockIdx.x]];
     const int w = ch.w;
@@ -111,7 +112,13 @@ __global__ void __launch_bounds__(256) k_inverse64(const double *__restrict__ ln
     if (threadIdx.x < 2 * kMaxChunk) key[0][threadIdx.x] = fx::kKeyNone;
     for (int e = threadIdx.x; e < kMaxChunk * (kMaxChunk + 1); e += 256) v[0][e] = 0.0;
     __syncthreads();
-    if (threadIdx.x < kMaxChunk) rinv[threadIdx.x] = threadIdx.x < w ? 1.0 / l[threadIdx.x][threadIdx.x] : 0.0;
+    if (threadIdx.x < kMaxChunk) {
+        const double lk = l[threadIdx.x][threadIdx.x];
+        rinv[threadIdx.x] = threadIdx.x < w ? 1.0 / lk : 0.0;
+        const int c = (int)threadIdx.x < w ? ((__double2hiint(lk) >> 20) & 0x7ff) - 1023 : 0;
+        e_c[threadIdx.x] = max(-1000, min(1000, c));
+        e_n[threadIdx.x] = -e_c[threadIdx.x];
+    }
     __syncthreads();
     const int nbk = (w + 15) / 16;
     if ((int)threadIdx.x / 32 < nbk && threadIdx.x % 32 < 16) {
@@ -153,19 +160,23 @@ __global__ void __launch_bounds__(256) k_inverse64(const double *__restrict__ ln
     // W's columns as 64 right-hand sides: R = I - L W (the subtraction before the
     // rounding), then the digits of W + W R
     fx::stage_tile(tl, e_l, &l[0][0], kMaxChunk + 1, kMaxChunk, kMaxChunk);
-    fx::stage_tile(tw, e_w, &v[0][0], kMaxChunk + 1, kMaxChunk, kMaxChunk);
     using Fr = fx::Frag<4>;
     Fr f;
     f.load(kMaxChunk, kMaxChunk, [&](int r, int c) { return v[r][c]; });
     f.keys(kMaxChunk, nullptr, key[0]);
     __syncthreads();
     f.put(kMaxChunk, nullptr, key[0], vec);
+    // from here on W's columns times 2^{c_k}, 2^{c_k} the size of L_kk: where W is multiplied, its
+    // columns' scales cancel against those of the other operand (D A D)
+    for (int e = threadIdx.x; e < kMaxChunk * kMaxChunk; e += 256)
+        v[e / kMaxChunk][e % kMaxChunk] *= scalbn(1.0, e_c[e % kMaxChunk]);
     __syncthreads();
+    fx::stage_tile(tw, e_w, &v[0][0], kMaxChunk + 1, kMaxChunk, kMaxChunk);
     const int mb = threadIdx.x / 32 % 4, ksteps = nbk;
 #pragma unroll
     for (int b = 0; b < 4; b++) {
         float acc[fx::S][4];
-        fx::product<false>(tl, vec, mb, Fr::n0(b), ksteps, acc);
+        fx::product<false>(tl, vec, mb, Fr::n0(b), 0, ksteps, acc);
 #pragma unroll
         for (int e = 0; e < 4; e++) {
             const int r = Fr::row(e), c = Fr::col(b, e), k = key[0][c], ex = e_l[r] + k - 1022;
@@ -185,13 +196,14 @@ __global__ void __launch_bounds__(256) k_inverse64(const double *__restrict__ ln
             f.v[b][e] = r < w && c < w && fits && e_l[r] != fx::kBadExp && k != fx::kKeyBad ? -fx::acc_value(a, ex) : 0.0;
         }
     }
-    f.keys(kMaxChunk, nullptr, key[1]);
+    f.keys(kMaxChunk, e_n, key[1]);
     __syncthreads();
-    f.put(kMaxChunk, nullptr, key[1], vec);
+    f.put(kMaxChunk, e_n, key[1], vec);
     __syncthreads();
     f.template mul<false, false>(tw, e_w, vec, key[1], w, w, kMaxChunk);
     f.each(w, w, [&](int r, int c, double lo) {
         const int E = e_w[r];
+        lo *= scalbn(1.0, e_c[c]);
         uint64_t X = 0x8080808080808080ull;
         if (E != fx::kBadExp) {
             X = fx::split_bytes(v[r][c], E);
@@ -201,7 +213,10 @@ __global__ void __launch_bounds__(256) k_inverse64(const double *__restrict__ ln
         }
         inv[ch.inv + r * w + c] = X;
     });
-    if ((int)threadIdx.x < w) inv_exp[ch.col0 + threadIdx.x] = e_w[threadIdx.x];
+    if ((int)threadIdx.x < w) {
+        inv_exp[ch.col0 + threadIdx.x] = e_w[threadIdx.x];
+        inv_cexp[ch.col0 + threadIdx.x] = e_n[threadIdx.x];
+    }
 }
 
 // ---- one persistent launch per level (SIMT precisions, RLB)
@@ -372,7 +387,7 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
             k_inverse<<<nch, 256, kPotrfSmem, st>>>((const float *)lnz, h->d_chunks, list, (float *)h->d_inv);
         else
             k_inverse64<<<nch, 256, kInv64Smem, st>>>((const double *)lnz, h->d_chunks, list, (uint64_t *)h->d_inv,
-                                                      h->d_inv_exp);
+                                                      h->d_inv_exp, h->d_inv_exp + s->n);
         E();
         launches++;
     };
@@ -467,15 +482,23 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
         }
         if (p.potrf_cnt) {
             B(kProfPotrf);
-            k_potrf<T><<<p.potrf_cnt, 256, kPotrfSmem, st>>>(lnz, h->d_chunks, h->d_potrf + p.potrf_off, h->d_adiag,
-                                                              h->d_info, h->d_info + 1, tau, h->d_hi, h->d_lo);
+            if constexpr (sizeof(T) == 8)
+                k_potrf64<<<p.potrf_cnt, 256, kChunk64Smem, st>>>((double *)lnz, h->d_chunks, h->d_potrf + p.potrf_off,
+                                                                  h->d_info, h->d_chunk64);
+            else
+                k_potrf<T><<<p.potrf_cnt, 256, kPotrfSmem, st>>>(lnz, h->d_chunks, h->d_potrf + p.potrf_off, h->d_adiag,
+                                                                  h->d_info, h->d_info + 1, tau, h->d_hi, h->d_lo);
             E();
             launches++;
         }
         if (p.trsm_cnt) {
             B(kProfTrsm);
-            k_trsm<T><<<p.trsm_cnt, trsm_rows<T>() * 4, 0, st>>>(lnz, h->d_chunks, h->d_trsm + p.trsm_off, h->d_hi,
-                                                           h->d_lo);
+            if constexpr (sizeof(T) == 8)
+                k_trsm64<<<p.trsm_cnt, 256, kChunk64Smem, st>>>((double *)lnz, h->d_chunks, h->d_trsm + p.trsm_off,
+                                                                h->d_chunk64);
+            else
+                k_trsm<T><<<p.trsm_cnt, trsm_rows<T>() * 4, 0, st>>>(lnz, h->d_chunks, h->d_trsm + p.trsm_off, h->d_hi,
+                                                               h->d_lo);
             E();
             launches++;
         }
@@ -588,8 +611,9 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
 int set_smem_attrs() {
     static bool done = false;
     if (done) return SC_OK;
-    SC_CUDA(cudaFuncSetAttribute(k_potrf<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPotrfSmem));
     SC_CUDA(cudaFuncSetAttribute(k_potrf<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPotrfSmem));
+    SC_CUDA(cudaFuncSetAttribute(k_potrf64, cudaFuncAttributeMaxDynamicSharedMemorySize, kChunk64Smem));
+    SC_CUDA(cudaFuncSetAttribute(k_trsm64, cudaFuncAttributeMaxDynamicSharedMemorySize, kChunk64Smem));
     SC_CUDA(cudaFuncSetAttribute(k_inverse64, cudaFuncAttributeMaxDynamicSharedMemorySize, kInv64Smem));
     SC_CUDA(cudaFuncSetAttribute(k_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, kPotrfSmem));
     SC_CUDA(cudaFuncSetAttribute(k_level<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPotrfSmem));
@@ -615,6 +639,7 @@ struct Plan {
     bool fused = false;    // for the per-level kernel: no k_narrow chunks (set before build_plan)
     int64_t inv_size = 0;  // elements of the diagonal-block inverses
     int32_t inv_off = 0, inv_cnt = 0;  // chunks of the inverse launch (in potrf)
+    int32_t chunk64_units = 0;         // digits of a level's chunks (FP64), in 256-word units
     // FP64 products on the tensor cores (empty without them)
     std::vector<SplitBlk> splits;
     std::vector<SplitUnit> split_units;
@@ -708,11 +733,20 @@ void build_plan(const sc_symbolic *s, int precision, Plan &P, bool lookahead, bo
         for (int32_t c : L.chunks)
             if (!by_warp(c)) P.potrf.push_back(c);
         p.potrf_cnt = (int32_t)P.potrf.size() - p.potrf_off;
+        // FP64: where the POTRF leaves the chunk's digits for the TRSM (256-word units,
+        // used again by the next level)
+        int32_t slot = 0;
+        for (int32_t i = 0; i < p.potrf_cnt; i++) {
+            ChunkDev &ch = P.cd[P.potrf[p.potrf_off + i]];
+            ch.slot = slot;
+            slot += chunk64_units(ch.w);
+        }
+        P.chunk64_units = std::max(P.chunk64_units, slot);
         p.trsm_off = (int32_t)P.trsm.size();
         for (int32_t c : L.chunks) {
             if (by_warp(c)) continue;
             const ChunkDev &ch = P.cd[c];
-            const int32_t rows = precision == SC_FP64 ? trsm_rows<double>() : trsm_rows<float>();
+            const int32_t rows = precision != SC_FP64 ? trsm_rows<float>() : P.fused ? trsm_rows<double>() : kTrsm64Rows;
             for (int32_t r0 = ch.c0 + ch.w; r0 < ch.m; r0 += rows) P.trsm.push_back(TrsmTile{c, r0});
         }
         p.trsm_cnt = (int32_t)P.trsm.size() - p.trsm_off;
@@ -1122,9 +1156,14 @@ int numeric_create(sc_symbolic *s, int precision, sc_numeric **out) {
     build_plan(s, precision, P, h->lookahead, !h->fused);
     if (cudaMalloc(&h->d_inv, (size_t)std::max<int64_t>(1, P.inv_size) * h->elt) != cudaSuccess) return fail(SC_ERR_OOM);
     bytes += P.inv_size * (int64_t)h->elt;
+    if (precision == SC_FP64 && !h->fused) {
+        const size_t b = (size_t)std::max(1, P.chunk64_units) * 256 * sizeof(uint64_t);
+        if (cudaMalloc((void **)&h->d_chunk64, b) != cudaSuccess) return fail(SC_ERR_OOM);
+        bytes += (int64_t)b;
+    }
     if (precision == SC_FP64) {
-        if (cudaMalloc((void **)&h->d_inv_exp, (size_t)s->n * sizeof(int32_t)) != cudaSuccess) return fail(SC_ERR_OOM);
-        bytes += s->n * (int64_t)sizeof(int32_t);
+        if (cudaMalloc((void **)&h->d_inv_exp, (size_t)s->n * 2 * sizeof(int32_t)) != cudaSuccess) return fail(SC_ERR_OOM);
+        bytes += s->n * 2 * (int64_t)sizeof(int32_t);
     }
     if (!P.splits.empty()) {
         // the slice pool; without room for it (or with more rows than a tensor map's
@@ -1358,7 +1397,7 @@ void numeric_free(sc_numeric *h) {
                     h->d_dep_ptr, h->d_dep, h->d_sync, h->d_serr, h->d_hi, h->d_lo, h->d_thin,
                     h->d_cgz, h->d_cgp, h->d_cgq, h->d_cgs, h->d_solve_units, h->d_flow, h->d_flow_ctr,
                     h->d_flow_need, h->d_task_chunk, h->d_sn_chunk, h->d_splits, h->d_split_units, h->d_split_of_task,
-                    h->d_slices, h->d_exps, h->d_slice_maps, h->d_inv_exp};
+                    h->d_slices, h->d_exps, h->d_slice_maps, h->d_inv_exp, h->d_chunk64};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (h->sym) h->sym->refs--;

@@ -370,7 +370,8 @@ __global__ void __launch_bounds__(trsm_rows<T>() * 4) k_trsm(T *__restrict__ lnz
 // is below 2^-58). FP64 outside the approximation's range, and FP32: the
 // library's function. Five multiply-adds of 64 clocks instead of some 440 clocks.
 __device__ __forceinline__ double fast_rsqrt(double d) {
-    if (!(d > 1e-300 && d < 1e300)) return rsqrt(d);
+    // (on the high word: a comparison in FP64 takes the pipe 64 clocks too)
+    if ((unsigned)(__double2hiint(d) - 0x02000000) >= 0x7c000000u) return rsqrt(d);
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
     const double e = fma(-d * y, y, 1.0);

@@ -817,7 +817,7 @@ struct Sweep64Args {
     int nrhs;
     int64_t vstride;
     const uint64_t *inv;  // digits of the inverses (k_inverse64)
-    const int32_t *inv_exp;
+    const int32_t *inv_exp, *inv_cexp;
     int32_t *f0, *f1;  // forward: arrivals, ready; backward: tile counts, done
     int64_t sstride;
     int32_t *work, *err;
@@ -829,7 +829,7 @@ __global__ void __launch_bounds__(256, 2) k_fwd64(Sweep64Args a) {
     using Fr = fx::Frag<NB>;
     extern __shared__ __align__(16) unsigned char smem_fwd64[];
     uint64_t *tl_l = reinterpret_cast<uint64_t *>(smem_fwd64), *tl_w = tl_l + 64 * fx::kLd, *vec = tl_w + 64 * fx::kLd;
-    __shared__ int32_t e_l[64], e_w[64];
+    __shared__ int32_t e_l[64], e_w[64], e_c[64];
     __shared__ int key[2][kRhsBlk];
     __shared__ int s_t, s_ok;
     const int ldv = rhs_ld(min(a.nrhs, kRhsBlk));
@@ -867,15 +867,15 @@ __global__ void __launch_bounds__(256, 2) k_fwd64(Sweep64Args a) {
         stage(0);
         if (threadIdx.x < 2 * kRhsBlk) key[threadIdx.x / kRhsBlk][threadIdx.x % kRhsBlk] = fx::kKeyNone;
         if (su.cnt == 0) {
-            fx::stage_inverse(tl_w, e_w, a.inv + ch.inv, a.inv_exp + ch.col0, w);
+            fx::stage_inverse(tl_w, e_w, e_c, a.inv + ch.inv, a.inv_exp + ch.col0, a.inv_cexp + ch.col0, w);
             if (threadIdx.x == 0)
                 s_ok = wait_flag(arrive + (int64_t)c * kSyncStride, a.count[c], a.err, a.spin_limit, 5);
             __syncthreads();
             if (!s_ok) break;
             v.load(w, nb, [&](int r, int n) { return __ldcg(x + (int64_t)(ch.col0 + r) * nb + n); });
-            v.keys(nb, nullptr, key[1]);
+            v.keys(nb, e_c, key[1]);
             __syncthreads();
-            v.put(nb, nullptr, key[1], vec);
+            v.put(nb, e_c, key[1], vec);
             __syncthreads();
             v.template mul<false, false>(tl_w, e_w, vec, key[1], w, w, nb);  // y_c
             v.each(w, nb, [&](int r, int n, double d) { y[(int64_t)(ch.col0 + r) * nb + n] = d; });
@@ -919,7 +919,7 @@ __global__ void __launch_bounds__(256, 2) k_bwd64(Sweep64Args a) {
     using Fr = fx::Frag<NB>;
     extern __shared__ __align__(16) unsigned char smem_bwd64[];
     uint64_t *tl_l = reinterpret_cast<uint64_t *>(smem_bwd64), *tl_w = tl_l + 64 * fx::kLd, *vec = tl_w + 64 * fx::kLd;
-    __shared__ int32_t e_l[64], e_w[64], grow[kSolveRows];
+    __shared__ int32_t e_l[64], e_w[64], e_c[64], grow[kSolveRows];
     __shared__ int key[2][kRhsBlk];
     __shared__ int s_t, s_ok;
     const int ldv = rhs_ld(min(a.nrhs, kRhsBlk));
@@ -952,7 +952,7 @@ __global__ void __launch_bounds__(256, 2) k_bwd64(Sweep64Args a) {
         const int c = a.tiles[su.t0].chunk;
         const ChunkDev ch = a.chunks[c];
         const int w = ch.w, g = first ? 1 : -su.cnt;
-        if (first) fx::stage_inverse(tl_w, e_w, a.inv + ch.inv, a.inv_exp + ch.col0, w);
+        if (first) fx::stage_inverse(tl_w, e_w, e_c, a.inv + ch.inv, a.inv_exp + ch.col0, a.inv_cexp + ch.col0, w);
         if (threadIdx.x < 2 * kRhsBlk) key[threadIdx.x / kRhsBlk][threadIdx.x % kRhsBlk] = fx::kKeyNone;
         Fr o;
 #pragma unroll
@@ -1013,7 +1013,7 @@ __global__ void __launch_bounds__(256, 2) k_bwd64(Sweep64Args a) {
         __syncthreads();
         v.put(nb, e_w, key[1], vec);
         __syncthreads();
-        v.template mul<true, false>(tl_w, nullptr, vec, key[1], w, w, nb);
+        v.template mul<true, false>(tl_w, e_c, vec, key[1], w, w, nb);
         v.each(w, nb, [&](int r, int n, double d) { z[(int64_t)(ch.col0 + r) * nb + n] = d; });
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -1392,7 +1392,7 @@ void launch_sweeps64(sc_numeric *h, int nrhs, int64_t vs, int64_t ss, double *xw
     const int total = h->solve_tiles * nblk;
     const int grid = std::max(1, std::min(total, std::max(1, std::min(p, q)) * h->num_sms));
     Sweep64Args a{(const double *)h->d_lnz, h->d_chunks, h->d_solve_tiles, h->d_solve_units, total, h->d_dep_ptr,
-                  h->d_dep, h->d_counters + nch, h->d_glbind, xw, y, z, acc, nrhs, vs, (const uint64_t *)h->d_inv, h->d_inv_exp, sync,
+                  h->d_dep, h->d_counters + nch, h->d_glbind, xw, y, z, acc, nrhs, vs, (const uint64_t *)h->d_inv, h->d_inv_exp, h->d_inv_exp + h->sym->n, sync,
                   sync + nch * kSyncStride, ss, sync + nblk * ss, h->d_serr, (long long)h->sym->opt.spin_limit};
     k_fwd64<NB><<<grid, 256, smem, st>>>(a);
     a.count = h->d_counters;

@@ -14,7 +14,10 @@
 // Operands in shared memory as whole numbers (fx::split_bytes): a tile has a
 // scale per row; a vector block [right-hand side][64 entries] a scale per
 // right-hand side. Where the rows of a tile are the inner dimension (backward), the
-// row scales go into the vector: L_ic z_i = X_ic (2^{E_i} z_i).
+// row scales go into the vector: L_ic z_i = X_ic (2^{E_i} z_i). An inverse also has a
+// scale per column, 2^{-c_k} with 2^{c_k} the size of L_kk, which goes into the other factor or
+// the result: the terms of a product then are of the size of their digits, also for
+// D A D with any diagonal D.
 #pragma once
 #include "fx.cuh"
 #include "kernels.cuh"
@@ -68,9 +71,11 @@ __device__ __forceinline__ void stage_tile(uint64_t *T, int32_t *rowE, const dou
                 : make_ulonglong2(split_bytes(v[2 * j], E), split_bytes(v[2 * j + 1], E));
 }
 
-// Stages the digits of a chunk's inverse (k_inverse64) and their row exponents.
-__device__ __forceinline__ void stage_inverse(uint64_t *T, int32_t *rowE, const uint64_t *__restrict__ inv,
-                                              const int32_t *__restrict__ exps, int w) {
+// Stages the digits of a chunk's inverse (k_inverse64), their row exponents and minus
+// their column exponents: W_jk = X_jk 2^{rowE_j + colE_k}.
+__device__ __forceinline__ void stage_inverse(uint64_t *T, int32_t *rowE, int32_t *colE,
+                                              const uint64_t *__restrict__ inv, const int32_t *__restrict__ exps,
+                                              const int32_t *__restrict__ cexps, int w) {
     constexpr int kIt = 64 * 64 / 256;
     uint64_t v[kIt];
 #pragma unroll
@@ -83,7 +88,10 @@ __device__ __forceinline__ void stage_inverse(uint64_t *T, int32_t *rowE, const 
         const int e = threadIdx.x + i * 256;
         T[e / 64 * kLd + e % 64] = v[i];
     }
-    if (threadIdx.x < 64) rowE[threadIdx.x] = (int)threadIdx.x < w ? exps[threadIdx.x] : -1021;
+    if (threadIdx.x < 64) {
+        rowE[threadIdx.x] = (int)threadIdx.x < w ? exps[threadIdx.x] : -1021;
+        colE[threadIdx.x] = (int)threadIdx.x < w ? cexps[threadIdx.x] : 0;
+    }
 }
 
 // Digit s (0: the highest) of two staged values as FP16: 1024 + byte, less 1152.
@@ -110,10 +118,10 @@ __device__ __forceinline__ void digit_row(float (&acc)[S][4], const ulonglong2 (
 }
 
 // Group sums of a 16 x 8 block of T V (or T^T V): rows 16 mb .. + 15 of the result,
-// right-hand sides n0 .. n0 + 7, inner dimension 16 ksteps. Lane l holds rows l / 4
+// right-hand sides n0 .. n0 + 7, inner dimension 16 ks0 .. 16 ks1 - 1. Lane l holds rows l / 4
 // (registers 0, 1) and l / 4 + 8 (2, 3), columns 2 (l % 4) and + 1.
 template <bool kTrans>
-__device__ __forceinline__ void product(const uint64_t *T, const uint64_t *V, int mb, int n0, int ksteps,
+__device__ __forceinline__ void product(const uint64_t *T, const uint64_t *V, int mb, int n0, int ks0, int ks1,
                                         float (&acc)[S][4]) {
     const int lane = threadIdx.x % 32, g = lane / 4, t = lane % 4;
 #pragma unroll
@@ -121,7 +129,7 @@ __device__ __forceinline__ void product(const uint64_t *T, const uint64_t *V, in
 #pragma unroll
         for (int e = 0; e < 4; e++) acc[s][e] = 0.f;
 #pragma unroll 1
-    for (int ks = 0; ks < ksteps; ks++) {
+    for (int ks = ks0; ks < ks1; ks++) {
         const int k = 16 * ks + 2 * t, m = 16 * mb + g;
         ulonglong2 x[4];
         if constexpr (kTrans) {
@@ -233,7 +241,7 @@ struct Frag {
         for (int b = 0; b < NB; b++) {
             if (n0(b) >= nb || 16 * mb >= M) break;
             float acc[S][4];
-            product<kTrans>(T, V, mb, n0(b), (K + 15) / 16, acc);
+            product<kTrans>(T, V, mb, n0(b), 0, (K + 15) / 16, acc);
 #pragma unroll
             for (int e = 0; e < 4; e++) {
                 const int k = key[col(b, e)];

@@ -70,6 +70,26 @@ def test_rows_of_very_different_scale():
     assert (err <= TOL * _row_scale(A)).all()
 
 
+@pytest.mark.parametrize("scaled_rhs", [True, False])
+@pytest.mark.parametrize("nrhs", [1, 9, 33])
+def test_solve_with_rows_of_very_different_scale(nrhs, scaled_rhs):
+    """(D A D) x = b: with b = D b0 the solution is D^{-1} (A^{-1} b0), every entry to the
+    accuracy of its own scale (A is diagonally dominant; 2 n u rounded up to
+    1e-12 of the largest entry of A^{-1} b0). With b = b0 the right-hand side D^{-1} b0
+    has entries of very different size, and the comparison is by the largest."""
+    A = _dense(300, 5)
+    d = 2.0 ** np.random.default_rng(3).integers(-60, 61, size=A.n)
+    b0 = inputs.rhs(A.n, nrhs, 4) / (1.0 if scaled_rhs else d[:, None])
+    o = oracle.Oracle(A, None, pr=True)
+    assert o.factor() == 0
+    x0 = o.solve(b0)
+    cols = np.repeat(np.arange(A.n), np.diff(A.colptr))
+    A.values *= d[A.rowind] * d[cols]
+    num = sc.Symbolic(A, ordering="natural").factor(A.values, precision="fp64")
+    X, _ = num.solve(b0 * d[:, None])
+    assert np.abs(X * d[:, None] - x0).max() <= 1e-12 * np.abs(x0).max()
+
+
 def test_nan_reaches_the_pivot():
     """A NaN in A's first column at row 200 of 300: rows below row 200 and the
     pivot of column 201 (1-based) see it, the columns before do not."""
