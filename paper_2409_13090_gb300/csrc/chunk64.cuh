@@ -94,21 +94,24 @@ __device__ __forceinline__ void ldl16(const double (*a)[17], double (*u)[17], do
     double r = live ? a[i][j] : 0.0;
     if (t < 16) col[0][t] = a[t][0];
     asm volatile("bar.sync 1, 128;" ::: "memory");
+    w = min(w, 16);  // past the chunk: the identity
+    if (t < 16 && t >= w) d[t] = 1.0;
+    for (int e = t; e < 256; e += 128)
+        if (e % 16 >= w) u[e / 16][e % 16] = 0.0;
 #pragma unroll 1
-    for (int k = 0; k < 16; k++) {
+    for (int k = 0; k < w; k++) {
         const double *ck = col[k & 1];
         double dk = ck[k];
         const double aik = live ? ck[i] : 0.0, ajk = live ? ck[j] : 0.0;
-        double uk;
-        // (comparisons on the high word: one in FP64 takes the pipe 64 clocks too)
-        if ((unsigned)(__double2hiint(dk) - 0x02000000) < 0x7c000000u) {  // 2^-991 <= dk < 2^993
-            double y;
-            asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(dk));
-            const double e = fma(-dk, y, 1.0), x = ajk * y;
-            uk = fma(x, fma(e, e, e), x);
-        } else {
+        double y;
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(dk));
+        const double e = fma(-dk, y, 1.0), x = ajk * y;
+        double uk = fma(x, fma(e, e, e), x);
+        // outside 2^-991 <= dk < 2^993 (on the high word: a comparison in FP64 takes the
+        // pipe 64 clocks too)
+        if ((unsigned)(__double2hiint(dk) - 0x02000000) >= 0x7c000000u) {
             if (!(dk > 0.0)) {
-                if (t == 0 && k < w) atomicMin(info, col0 + k + 1);
+                if (t == 0) atomicMin(info, col0 + k + 1);
                 dk = 1.0;
             }
             uk = ajk / dk;
@@ -192,6 +195,7 @@ __global__ void __launch_bounds__(256) k_potrf64(double *__restrict__ lnz, const
             wv = i == j ? 1.0 : 0.0;
 #pragma unroll
             for (int k = 0; k < 15; k++) {
+                if (16 * p + k + 1 >= w) break;
                 const double wk = __shfl_sync(0xffffffffu, wv, k + (lane & 16));
                 if (i > k) wv -= ui[k] * wk;
             }

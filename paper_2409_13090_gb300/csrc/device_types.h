@@ -67,6 +67,9 @@ SC_HD inline int block_rows(int rows, int nb, int ni_min, bool lower) {
 }
 
 constexpr int kMaxChunk = 64;
+constexpr int kLoopMinWarps = 1216;  // loop items of narrow supernodes of a level from which a warp takes one
+constexpr int kNarrowMin64 = 1024;  // small chunks of a level from which FP64 takes them by warps
+
 // FP64 POTRF to TRSM: 256-word units of a chunk's digits -- L_cc, the inverses of its
 // 16 x 16 diagonal blocks, exponents.
 SC_HD inline int chunk64_units(int w) {

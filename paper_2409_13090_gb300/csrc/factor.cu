@@ -717,10 +717,15 @@ void build_plan(const sc_symbolic *s, int precision, Plan &P, bool lookahead, bo
         LevelPlan &p = P.levels[lv];
         // chunks narrow and short enough for one warp, then the others; the per-level
         // kernel of a fused plan takes them all as the others
-        auto by_warp = [&](int32_t c) {
+        auto small = [&](int32_t c) {
             const ChunkDev &ch = P.cd[c];
             return !P.fused && narrow_chunk(ch.w, ch.m - ch.c0 - ch.w, precision == SC_FP64);
         };
+        // FP64: a level of few chunks gains nothing (a CTA takes a small chunk in about
+        // the warp's time, and the level one launch less)
+        const bool use_warps =
+            precision != SC_FP64 || std::count_if(L.chunks.begin(), L.chunks.end(), small) >= kNarrowMin64;
+        auto by_warp = [&](int32_t c) { return use_warps && small(c); };
         p.narrow_off = (int32_t)P.potrf.size();
         for (int32_t c : L.chunks) {
             if (by_warp(c)) P.potrf.push_back(c);
@@ -832,13 +837,17 @@ void build_plan(const sc_symbolic *s, int precision, Plan &P, bool lookahead, bo
         p.small_cnt = (int32_t)ids_small.size();
         // device-side RLB loops
         // (items of supernodes narrower than 32 columns: one warp each)
+        // (while a level has few of them a CTA each: a warp's chain of products would be
+        // the level's time, 33 us a level of the 64 x 64 2D matrix)
+        auto narrow = [&](const LoopItem &it) { return s->sup_ptr[it.sn + 1] - s->sup_ptr[it.sn] < 32; };
+        const bool warp_items = std::count_if(L.loops.begin(), L.loops.end(), narrow) >= kLoopMinWarps;
         p.loop_off = (int32_t)P.loops.size();
         for (const LoopItem &it : L.loops)
-            if (s->sup_ptr[it.sn + 1] - s->sup_ptr[it.sn] >= 32) P.loops.push_back(it);
+            if (!warp_items || !narrow(it)) P.loops.push_back(it);
         p.loop_cnt = (int32_t)P.loops.size() - p.loop_off;
         p.loopw_off = (int32_t)P.loops.size();
         for (const LoopItem &it : L.loops)
-            if (s->sup_ptr[it.sn + 1] - s->sup_ptr[it.sn] < 32) P.loops.push_back(it);
+            if (warp_items && narrow(it)) P.loops.push_back(it);
         p.loopw_cnt = (int32_t)P.loops.size() - p.loopw_off;
         P.class_flops[kProfLoop] += L.loop_flops;
         // RL update matrices and assembly
