@@ -88,36 +88,29 @@ __global__ void __launch_bounds__(256) k_inverse(const float *__restrict__ lnz, 
 // Inverses of the factored diagonal blocks of the chunks wider than kNarrowChunk, for
 // the solve sweeps of FP64 factors: L_cc in 16 x 16 blocks; the diagonal ones by
 // substitution (a warp each, a lane per column), then block diagonal by block
-// diagonal W_ij = -W_ii sum_{j <= k < i} L_ik W_kj, and one step W + W (I - L W) whose
-// products are formed from digits. Stored as the digits of W's rows (62 bits: the sum
-// before it is rounded to FP64), columns scaled, with the rows' exponents and minus the
-// columns', so a product with W is no further off than the substitution it stands for: with W in FP64 the solutions'
-// errors grew by up to a fifth. Bound by the FP64 pipe (some 41,000 clocks a block
-// and SM before the correction).
-constexpr int kInv64Smem = 8 * (2 * kMaxChunk * (kMaxChunk + 1) + 3 * kMaxChunk * fx::kLd);
+// diagonal W_ij = -W_ii sum_{j <= k < i} L_ik W_kj. Stored as the digits of W's rows (columns
+// times 2^{c_k}, 2^{c_k} the size of L_kk: where W is multiplied, its columns' scales
+// cancel against those of the other operand, also for D A D), the rows' exponents
+// and minus the columns'. Bound by the FP64 pipe (some 41,000 clocks a block and
+// SM). A step W + W (I - L W) after it changed the solutions' errors by less than the
+// seeds differ (40 seeds of five matrices) and cost another 20,000 clocks.
+constexpr int kInv64Smem = 8 * (2 * kMaxChunk * (kMaxChunk + 1));
 __global__ void __launch_bounds__(256) k_inverse64(const double *__restrict__ lnz, const ChunkDev *__restrict__ chunks,
                                                    const int32_t *__restrict__ list, uint64_t *__restrict__ inv,
                                                    int32_t *__restrict__ inv_exp, int32_t *__restrict__ inv_cexp) {
     extern __shared__ double smem_potrf[];
     __shared__ double rinv[kMaxChunk];
-    __shared__ int32_t e_l[kMaxChunk], e_w[kMaxChunk], e_c[kMaxChunk], e_n[kMaxChunk];
-    __shared__ int key[2][kMaxChunk];
+    __shared__ int32_t e_c[kMaxChunk];
     const ChunkDev ch = chunks[list[blockIdx.x]];
     const int w = ch.w;
     auto l = reinterpret_cast<double (*)[kMaxChunk + 1]>(smem_potrf);
     auto v = l + kMaxChunk;
-    uint64_t *tl = reinterpret_cast<uint64_t *>(v + kMaxChunk), *tw = tl + kMaxChunk * fx::kLd,
-             *vec = tw + kMaxChunk * fx::kLd;
     load_block(l, lnz + ch.off + (int64_t)ch.c0 * ch.ld + ch.c0, ch.ld, w);
-    if (threadIdx.x < 2 * kMaxChunk) key[0][threadIdx.x] = fx::kKeyNone;
-    for (int e = threadIdx.x; e < kMaxChunk * (kMaxChunk + 1); e += 256) v[0][e] = 0.0;
     __syncthreads();
     if (threadIdx.x < kMaxChunk) {
         const double lk = l[threadIdx.x][threadIdx.x];
         rinv[threadIdx.x] = threadIdx.x < w ? 1.0 / lk : 0.0;
-        const int c = (int)threadIdx.x < w ? ((__double2hiint(lk) >> 20) & 0x7ff) - 1023 : 0;
-        e_c[threadIdx.x] = max(-1000, min(1000, c));
-        e_n[threadIdx.x] = -e_c[threadIdx.x];
+        e_c[threadIdx.x] = (int)threadIdx.x < w ? ((__double2hiint(lk) >> 20) & 0x7ff) - 1023 : 0;
     }
     __syncthreads();
     const int nbk = (w + 15) / 16;
@@ -154,68 +147,19 @@ __global__ void __launch_bounds__(256) k_inverse64(const double *__restrict__ ln
         }
         __syncthreads();
     }
-    for (int e = threadIdx.x; e < kMaxChunk * kMaxChunk; e += 256)
-        if (e / kMaxChunk < e % kMaxChunk) v[e / kMaxChunk][e % kMaxChunk] = 0.0;
-    __syncthreads();
-    // W's columns as 64 right-hand sides: R = I - L W (the subtraction before the
-    // rounding), then the digits of W + W R
-    fx::stage_tile(tl, e_l, &l[0][0], kMaxChunk + 1, kMaxChunk, kMaxChunk);
-    using Fr = fx::Frag<4>;
-    Fr f;
-    f.load(kMaxChunk, kMaxChunk, [&](int r, int c) { return v[r][c]; });
-    f.keys(kMaxChunk, nullptr, key[0]);
-    __syncthreads();
-    f.put(kMaxChunk, nullptr, key[0], vec);
-    // from here on W's columns times 2^{c_k}, 2^{c_k} the size of L_kk: where W is multiplied, its
-    // columns' scales cancel against those of the other operand (D A D)
-    for (int e = threadIdx.x; e < kMaxChunk * kMaxChunk; e += 256)
-        v[e / kMaxChunk][e % kMaxChunk] *= scalbn(1.0, e_c[e % kMaxChunk]);
-    __syncthreads();
-    fx::stage_tile(tw, e_w, &v[0][0], kMaxChunk + 1, kMaxChunk, kMaxChunk);
-    const int mb = threadIdx.x / 32 % 4, ksteps = nbk;
-#pragma unroll
-    for (int b = 0; b < 4; b++) {
-        float acc[fx::S][4];
-        fx::product<false>(tl, vec, mb, Fr::n0(b), 0, ksteps, acc);
-#pragma unroll
-        for (int e = 0; e < 4; e++) {
-            const int r = Fr::row(e), c = Fr::col(b, e), k = key[0][c], ex = e_l[r] + k - 1022;
-            fx::Acc96 a = fx::block_acc(acc, e);
-            // one, in units of 2^(ex - 68)
-            const int one = 68 - ex;
-            const bool fits = one >= 0 && one < 94;
-            if (r == c && fits) {
-                if (one >= 32) {
-                    a.t -= 1ll << (one - 32);
-                } else {
-                    const uint32_t d = 1u << one;
-                    a.t -= a.r < d ? 1 : 0;
-                    a.r -= d;
-                }
-            }
-            f.v[b][e] = r < w && c < w && fits && e_l[r] != fx::kBadExp && k != fx::kKeyBad ? -fx::acc_value(a, ex) : 0.0;
-        }
-    }
-    f.keys(kMaxChunk, e_n, key[1]);
-    __syncthreads();
-    f.put(kMaxChunk, e_n, key[1], vec);
-    __syncthreads();
-    f.template mul<false, false>(tw, e_w, vec, key[1], w, w, kMaxChunk);
-    f.each(w, w, [&](int r, int c, double lo) {
-        const int E = e_w[r];
-        lo *= scalbn(1.0, e_c[c]);
-        uint64_t X = 0x8080808080808080ull;
-        if (E != fx::kBadExp) {
-            X = fx::split_bytes(v[r][c], E);
-            // the correction only where it is one (far below W; not for a block whose
-            // condition is beyond FP64)
-            if (fabs(lo) < 0x1p-20 * scalbn(1.0, E)) X += fx::split_bytes(lo, E) - 0x8080808080808080ull;
-        }
-        inv[ch.inv + r * w + c] = X;
-    });
-    if ((int)threadIdx.x < w) {
-        inv_exp[ch.col0 + threadIdx.x] = e_w[threadIdx.x];
-        inv_cexp[ch.col0 + threadIdx.x] = e_n[threadIdx.x];
+    // digits: four threads per row, columns q, q + 4, ...
+    const int r = threadIdx.x / 4, q = threadIdx.x % 4;
+    int key = fx::kKeyNone;
+    for (int c = q; c <= r; c += 4) key = max(key, fx::exp_key(v[r][c], e_c[c]));
+    key = max(key, __shfl_xor_sync(0xffffffffu, key, 1));
+    key = max(key, __shfl_xor_sync(0xffffffffu, key, 2));
+    if (r >= w) return;
+    for (int c = q; c < w; c += 4)
+        inv[ch.inv + r * w + c] =
+            c > r || key == fx::kKeyBad ? 0x8080808080808080ull : fx::split_bytes(v[r][c], key - 1022 - e_c[c]);
+    if (q == 0) {
+        inv_exp[ch.col0 + r] = key == fx::kKeyBad ? fx::kBadExp : key - 1022;
+        inv_cexp[ch.col0 + r] = -e_c[r];
     }
 }
 

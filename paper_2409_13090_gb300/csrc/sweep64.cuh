@@ -161,17 +161,13 @@ __device__ __forceinline__ void product(const uint64_t *T, const uint64_t *V, in
         digit_row<7>(acc, x, b);
     }
 }
-// register e of a block's group sums as one whole number
-__device__ __forceinline__ Acc96 block_acc(const float (&acc)[S][4], int e) {
+// value of register e of a block's group sums, times 2^(er + ec)
+__device__ __forceinline__ double block_value(const float (&acc)[S][4], int e, int er, int ec) {
+    if (er == kBadExp || ec == kBadExp) return __longlong_as_double(0x7ff8000000000000ll);
     // at most 64 terms: every pair of groups fits in 32 bits (|g_7| < 2^22.6)
     auto pair = [&](int s) { return __float2int_rn(acc[s][e]) * 256 + __float2int_rn(acc[s + 1][e]); };
     const int64_t H = ((int64_t)pair(0) << 16) + pair(2), L = ((int64_t)pair(4) << 16) + pair(6);
-    return Acc96{H + (L >> 32), (uint32_t)L};
-}
-// its value times 2^(er + ec)
-__device__ __forceinline__ double block_value(const float (&acc)[S][4], int e, int er, int ec) {
-    if (er == kBadExp || ec == kBadExp) return __longlong_as_double(0x7ff8000000000000ll);
-    return acc_value(block_acc(acc, e), er + ec);
+    return acc_value(Acc96{H + (L >> 32), (uint32_t)L}, er + ec);
 }
 
 // A warp's part of a 64 x nb block of values, in the layout of the products: rows
