@@ -260,6 +260,34 @@ __device__ bool wait_flag(const int32_t *flag, int32_t target, int32_t *err, lon
     return false;
 }
 
+// ---- a tile's dependency list (the chunks its rows fall in), by one warp. Read as soon as the
+// tile is known, one entry per lane, so the arrivals after the tile's fence and the
+// waits before it do not add the lists' two dependent loads, or one wait after
+// another, to a chain step.
+struct Deps {
+    int p0, p1, c;  // range in the list; this lane's entry (of the first 32)
+    __device__ __forceinline__ Deps(const int32_t *__restrict__ dep_ptr, const int32_t *__restrict__ dep, int t, int cnt) {
+        const int lane = threadIdx.x % 32;
+        p0 = dep_ptr[t];
+        p1 = dep_ptr[t + cnt];
+        c = p0 + lane < p1 ? dep[p0 + lane] : -1;
+    }
+    // after the CTA's barrier: every lane's fence, then its arrivals
+    __device__ __forceinline__ void arrive(int32_t *words, const int32_t *__restrict__ dep) const {
+        __threadfence();
+        if (c >= 0) atomicAdd(words + (int64_t)c * kSyncStride, 1);
+        for (int p = p0 + 32 + (int)threadIdx.x % 32; p < p1; p += 32) atomicAdd(words + (int64_t)dep[p] * kSyncStride, 1);
+    }
+    // true in every lane when all the words have become 1
+    __device__ __forceinline__ bool wait(const int32_t *words, const int32_t *__restrict__ dep, int32_t *err,
+                                         long long spin_limit, int code) const {
+        bool ok = c < 0 || wait_flag(words + (int64_t)c * kSyncStride, 1, err, spin_limit, code);
+        for (int p = p0 + 32 + (int)threadIdx.x % 32; p < p1 && ok; p += 32)
+            ok = wait_flag(words + (int64_t)dep[p] * kSyncStride, 1, err, spin_limit, code);
+        return __all_sync(0xffffffffu, ok);
+    }
+};
+
 // next tile index of a sweep for this CTA (broadcast through shared memory);
 // `total` once the sweep is done or a wait has given up
 __device__ __forceinline__ int grab_tile(int32_t *work, int total, int32_t *err, int *slot) {
@@ -285,6 +313,7 @@ __device__ bool fwd_tile_warp(const T *__restrict__ lnz, const ChunkDev &ch, con
     const int lane = threadIdx.x % 32, w = ch.w;
     const bool first = tl.r0 == ch.c0 + w;
     const int rows = max(0, min(kSolveRows, ch.m - tl.r0));
+    const Deps deps(dep_ptr, dep, t, 1);
     // FP64: lane j % 16 holds row j of L_cc below the diagonal and its reciprocal pivot
     T lj[sizeof(T) == 8 ? kSmallW : 1], rj = T(0);
     const T *dg = lnz + ch.off + (int64_t)ch.c0 * ch.ld + ch.c0;
@@ -346,10 +375,7 @@ __device__ bool fwd_tile_warp(const T *__restrict__ lnz, const ChunkDev &ch, con
         red_add(x + (int64_t)glbind[ch.gl + tl.r0 + i] * nb + r, -acc);
     }
     __syncwarp();
-    if (lane == 0) {
-        __threadfence();
-        for (int p = dep_ptr[t]; p < dep_ptr[t + 1]; p++) atomicAdd(arrive + (int64_t)dep[p] * kSyncStride, 1);
-    }
+    deps.arrive(arrive, dep);
     __syncwarp();
     return true;
 }
@@ -367,11 +393,8 @@ __device__ bool bwd_tile_warp(const T *__restrict__ lnz, const ChunkDev &ch, con
     const int lane = threadIdx.x % 32, w = ch.w;
     const int rows = max(0, min(kSolveRows, ch.m - tl.r0));
     if (rows > 0) {
-        int ok = 1;
-        if (lane == 0)
-            for (int p = dep_ptr[t]; p < dep_ptr[t + 1] && ok; p++)
-                ok = wait_flag(done + (int64_t)dep[p] * kSyncStride, 1, err, spin_limit, 6);
-        if (!__shfl_sync(0xffffffffu, ok, 0)) return false;
+        if (!Deps(dep_ptr, dep, t, 1).wait(done, dep, err, spin_limit, 6)) return false;
+        __syncwarp();
         for (int e = lane; e < w * nb; e += 32) {
             const int k = e / nb, r = e % nb;
             T sum = T(0);
@@ -525,6 +548,7 @@ __global__ void __launch_bounds__(256, 3) k_fwd(const T *__restrict__ lnz, const
                 const int tq = su.t0 + q;
                 const TrsmTile tl = tiles[tq];
                 const int rows = max(0, min(kSolveRows, ch.m - tl.r0));
+                const Deps deps(dep_ptr, dep, tq, 1);
                 if (q > 0) {
                     stage_block(sm.lr, lnz + ch.off + (int64_t)tl.r0 * ch.ld + ch.c0, ch.ld, rows, w);
                     __syncthreads();
@@ -541,10 +565,7 @@ __global__ void __launch_bounds__(256, 3) k_fwd(const T *__restrict__ lnz, const
                 // each tile's arrivals go out as soon as its rows are updated: a later
                 // chunk's step must not wait for the rest of the unit
                 __syncthreads();
-                if (threadIdx.x == 0) {
-                    __threadfence();
-                    for (int p = dep_ptr[tq]; p < dep_ptr[tq + 1]; p++) atomicAdd(arrive + (int64_t)dep[p] * kSyncStride, 1);
-                }
+                if (threadIdx.x < 32) deps.arrive(arrive, dep);
             }
             continue;
         }
@@ -553,6 +574,7 @@ __global__ void __launch_bounds__(256, 3) k_fwd(const T *__restrict__ lnz, const
         const ChunkDev ch = chunks[tl.chunk];
         const int w = ch.w;
         const bool first = tl.r0 == ch.c0 + w;  // the chunk's first tile solves and publishes y_c
+        const Deps deps(dep_ptr, dep, t, 1);
         const int rows = max(0, min(kSolveRows, ch.m - tl.r0));
         // loads that need no other tile: the tile's rows of L (and the diagonal block)
         stage_block(sm.lr, lnz + ch.off + (int64_t)tl.r0 * ch.ld + ch.c0, ch.ld, rows, w);
@@ -609,12 +631,9 @@ __global__ void __launch_bounds__(256, 3) k_fwd(const T *__restrict__ lnz, const
                                            m.r0, nb);
             }
         }
-        // release: the barrier orders every thread's updates before thread 0's fence
+        // release: the barrier orders every thread's updates before warp 0's fence
         __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            for (int p = dep_ptr[t]; p < dep_ptr[t + 1]; p++) atomicAdd(arrive + (int64_t)dep[p] * kSyncStride, 1);
-        }
+        if (threadIdx.x < 32) deps.arrive(arrive, dep);
     }
 }
 
@@ -670,12 +689,7 @@ __global__ void __launch_bounds__(256, 3) k_bwd(const T *__restrict__ lnz, const
             const int c = tiles[su.t0].chunk;
             const ChunkDev ch = chunks[c];
             const int w = ch.w;
-            if (threadIdx.x == 0) {
-                bool ok = true;
-                for (int p = dep_ptr[su.t0]; p < dep_ptr[su.t0 + g] && ok; p++)
-                    ok = wait_flag(done + (int64_t)dep[p] * kSyncStride, 1, err, spin_limit, 6);
-                s_ok = ok;
-            }
+            if (threadIdx.x < 32) s_ok = Deps(dep_ptr, dep, su.t0, g).wait(done, dep, err, spin_limit, 6);
             __syncthreads();
             if (!s_ok) break;
             const Map m;
@@ -717,6 +731,7 @@ __global__ void __launch_bounds__(256, 3) k_bwd(const T *__restrict__ lnz, const
         // before it waits and keeps its own contribution in registers
         const bool first = tl.r0 == ch.c0 + w;
         const int rows = max(0, min(kSolveRows, ch.m - tl.r0));
+        const Deps deps(dep_ptr, dep, t, 1);
         const Map m;
         T o[Map::NR][Map::R];
 #pragma unroll
@@ -729,12 +744,7 @@ __global__ void __launch_bounds__(256, 3) k_bwd(const T *__restrict__ lnz, const
         if (rows > 0) {
             if (threadIdx.x < rows) grow[threadIdx.x] = glbind[ch.gl + tl.r0 + threadIdx.x];
             stage_block(sm.lr, lnz + ch.off + (int64_t)tl.r0 * ch.ld + ch.c0, ch.ld, rows, w);
-            if (threadIdx.x == 0) {
-                bool ok = true;
-                for (int p = dep_ptr[t]; p < dep_ptr[t + 1] && ok; p++)
-                    ok = wait_flag(done + (int64_t)dep[p] * kSyncStride, 1, err, spin_limit, 6);
-                s_ok = ok;
-            }
+            if (threadIdx.x < 32) s_ok = deps.wait(done, dep, err, spin_limit, 6);
             __syncthreads();
             if (!s_ok) break;
             stage_rhs(sm.v, ldv, (const T *)z, nb, rows, [&](int r) { return grow[r]; });
@@ -896,6 +906,7 @@ __global__ void __launch_bounds__(256, 2) k_fwd64(Sweep64Args a) {
         __syncthreads();
         for (int q = 0; q < g; q++) {
             const int t = su.t0 + q, r0 = a.tiles[t].r0, rows = max(0, min(kSolveRows, ch.m - r0));
+            const Deps deps(a.dep_ptr, a.dep, t, 1);
             if (q > 0) {
                 stage(q);
                 __syncthreads();
@@ -903,13 +914,9 @@ __global__ void __launch_bounds__(256, 2) k_fwd64(Sweep64Args a) {
             Fr o;
             o.template mul<false, false>(tl_l, e_l, vec, key[0], w, rows, nb);
             o.each(rows, nb, [&](int r, int n, double d) { red_add(x + (int64_t)a.glbind[ch.gl + r0 + r] * nb + n, -d); });
-            // release: the barrier orders every thread's updates before thread 0's fence
+            // release: the barrier orders every thread's updates before warp 0's fence
             __syncthreads();
-            if (threadIdx.x == 0) {
-                __threadfence();
-                for (int p = a.dep_ptr[t]; p < a.dep_ptr[t + 1]; p++)
-                    atomicAdd(arrive + (int64_t)a.dep[p] * kSyncStride, 1);
-            }
+            if (threadIdx.x < 32) deps.arrive(arrive, a.dep);
         }
     }
 }
@@ -965,13 +972,9 @@ __global__ void __launch_bounds__(256, 2) k_bwd64(Sweep64Args a) {
             if (rows == 0) break;  // the last chunk of a root: nothing below
             if (q > 0) __syncthreads();  // the previous tile and its vector are no longer read
             if (threadIdx.x < rows) grow[threadIdx.x] = a.glbind[ch.gl + r0 + threadIdx.x];
+            const Deps deps(a.dep_ptr, a.dep, t, 1);
             fx::stage_tile(tl_l, e_l, a.lnz + ch.off + (int64_t)r0 * ch.ld + ch.c0, ch.ld, rows, w);
-            if (threadIdx.x == 0) {
-                bool k = true;
-                for (int p = a.dep_ptr[t]; p < a.dep_ptr[t + 1] && k; p++)
-                    k = wait_flag(done + (int64_t)a.dep[p] * kSyncStride, 1, a.err, a.spin_limit, 6);
-                s_ok = k;
-            }
+            if (threadIdx.x < 32) s_ok = deps.wait(done, a.dep, a.err, a.spin_limit, 6);
             __syncthreads();
             if (!(ok = s_ok)) break;
             Fr v;
