@@ -301,6 +301,160 @@ __device__ __forceinline__ int grab_tile(int32_t *work, int total, int32_t *err,
 // per-warp shared-memory slice of kSmallW rows of ldv values.
 constexpr int kSmallW = kNarrowChunk;
 
+// Narrow tiles with up to kFewRhs right-hand sides, by one warp (FP32): a row (and the one 32
+// below it) per lane, everything that needs no other tile loaded before the wait, the diagonal
+// step's and the rows' vectors passed by shuffles. (The forms below, an output per lane
+// with its loads in the inner loop, took 18.2 ms for the solves of a batch of 256 2D
+// problems, these 14.9. In FP64 they would spill.)
+constexpr int kFewRhs = 4;
+struct NarrowTile {
+    float l0[kSmallW], l1[kSmallW];  // rows lane and lane + 32 of the tile
+    int g0, g1;                  // their global rows
+    float d[kSmallW];            // lane j % 16: row (forward) or column (backward) j of the chunk's inverse
+    int rows, lane, j;
+    template <bool kBackward>
+    __device__ __forceinline__ void load(const float *__restrict__ lnz, const ChunkDev &ch, const TrsmTile &tl,
+                                         const int32_t *__restrict__ glbind, const float *__restrict__ inv) {
+        const int w = ch.w;
+        lane = threadIdx.x % 32;
+        j = lane % 16;
+        rows = max(0, min(kSolveRows, ch.m - tl.r0));
+        const float *p = lnz + ch.off + (int64_t)(tl.r0 + lane) * ch.ld + ch.c0;
+        const bool a = lane < rows, b = lane + 32 < rows;
+#pragma unroll
+        for (int k = 0; k < kSmallW; k++) {
+            l0[k] = a && k < w ? p[k] : 0.f;
+            l1[k] = b && k < w ? p[32 * (int64_t)ch.ld + k] : 0.f;
+        }
+        g0 = a ? glbind[ch.gl + tl.r0 + lane] : 0;
+        g1 = b ? glbind[ch.gl + tl.r0 + lane + 32] : 0;
+        const float *iv = inv + ch.inv;
+#pragma unroll
+        for (int k = 0; k < kSmallW; k++) d[k] = j < w && k < w ? (kBackward ? iv[k * w + j] : iv[j * w + k]) : 0.f;
+    }
+    // the diagonal step for the vector whose entry j is v in lanes j and j + 16
+    __device__ __forceinline__ float diag(float v) const {
+        float s = 0.f;
+#pragma unroll
+        for (int k = 0; k < kSmallW; k++) s += d[k] * __shfl_sync(0xffffffffu, v, k);
+        return s;
+    }
+};
+
+__device__ bool fwd_tile_few(const float *__restrict__ lnz, const ChunkDev &ch, const TrsmTile &tl, int t,
+                             const int32_t *__restrict__ dep_ptr, const int32_t *__restrict__ dep,
+                             const int32_t *__restrict__ need, const int32_t *__restrict__ glbind, float *__restrict__ x,
+                             float *__restrict__ y, int nb, const float *__restrict__ inv, int32_t *__restrict__ arrive,
+                             int32_t *__restrict__ err, long long spin_limit) {
+    const int w = ch.w;
+    const Deps deps(dep_ptr, dep, t, 1);
+    const int want = need[tl.chunk];
+    NarrowTile n;
+    n.load<false>(lnz, ch, tl, glbind, inv);
+    int ok = 1;
+    if (n.lane == 0) ok = wait_flag(arrive + (int64_t)tl.chunk * kSyncStride, want, err, spin_limit, 5);
+    if (!__shfl_sync(0xffffffffu, ok, 0)) return false;
+    __syncwarp();
+    const bool first = tl.r0 == ch.c0 + w;
+    for (int r = 0; r < nb; r++) {
+        const float v = n.diag(n.j < w ? __ldcg(x + (int64_t)(ch.col0 + n.j) * nb + r) : 0.f);
+        if (first && n.lane < w) y[(int64_t)(ch.col0 + n.lane) * nb + r] = v;
+        float a = 0.f, b = 0.f;
+#pragma unroll
+        for (int k = 0; k < kSmallW; k++) {
+            if (k >= w) break;
+            const float yk = __shfl_sync(0xffffffffu, v, k);
+            a += n.l0[k] * yk;
+            if (n.rows > 32) b += n.l1[k] * yk;
+        }
+        if (n.lane < n.rows) red_add(x + (int64_t)n.g0 * nb + r, -a);
+        if (n.lane + 32 < n.rows) red_add(x + (int64_t)n.g1 * nb + r, -b);
+    }
+    __syncwarp();
+    deps.arrive(arrive, dep);
+    __syncwarp();
+    return true;
+}
+
+__device__ bool bwd_tile_few(const float *__restrict__ lnz, const ChunkDev &ch, const TrsmTile &tl, int t,
+                             const int32_t *__restrict__ dep_ptr, const int32_t *__restrict__ dep,
+                             const int32_t *__restrict__ ntiles, const int32_t *__restrict__ glbind,
+                             const float *__restrict__ y, float *__restrict__ z, float *__restrict__ acc, int nb,
+                             const float *__restrict__ inv, int32_t *__restrict__ cnt, int32_t *__restrict__ done,
+                             int32_t *__restrict__ err, long long spin_limit) {
+    const int w = ch.w;
+    const Deps deps(dep_ptr, dep, t, 1);
+    const int nt = ntiles[tl.chunk];
+    NarrowTile n;
+    n.load<true>(lnz, ch, tl, glbind, inv);
+    float own[kFewRhs], yv[kFewRhs];  // lane: entry lane / 2 of the tile's part; entry j of y_c
+#pragma unroll
+    for (int r = 0; r < kFewRhs; r++) {
+        own[r] = 0.f;
+        yv[r] = r < nb && n.j < w ? y[(int64_t)(ch.col0 + n.j) * nb + r] : 0.f;
+    }
+    if (n.rows > 0) {
+        if (!deps.wait(done, dep, err, spin_limit, 6)) return false;
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < kFewRhs; r++) {
+            if (r >= nb) break;
+            const float z0 = n.lane < n.rows ? __ldcg(z + (int64_t)n.g0 * nb + r) : 0.f;
+            const float z1 = n.lane + 32 < n.rows ? __ldcg(z + (int64_t)n.g1 * nb + r) : 0.f;
+            float v[kSmallW];
+#pragma unroll
+            for (int k = 0; k < kSmallW; k++) v[k] = k < w ? n.l0[k] * z0 : 0.f;
+            if (n.rows > 32) {
+#pragma unroll
+                for (int k = 0; k < kSmallW; k++)
+                    if (k < w) v[k] += n.l1[k] * z1;
+            }
+            // recursive halving: bit o / 2 of the entry's index goes with bit o of the lane
+#pragma unroll
+            for (int o = 16; o >= 2; o >>= 1) {
+                const bool up = n.lane & o;
+#pragma unroll
+                for (int q = 0; q < o / 2; q++) {
+                    const float send = up ? v[q] : v[q + o / 2], keep = up ? v[q + o / 2] : v[q];
+                    v[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                }
+            }
+            own[r] = v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+        }
+    }
+    const int k = n.lane / 2;
+    if (nt > 1) {
+        // other tiles of the chunk: the last to finish solves
+#pragma unroll
+        for (int r = 0; r < kFewRhs; r++)
+            if (r < nb && n.lane % 2 == 0 && k < w) red_add(acc + (int64_t)(ch.col0 + k) * nb + r, own[r]);
+        __syncwarp();
+        int last = 0;
+        if (n.lane == 0) {
+            __threadfence();
+            last = atomicAdd(cnt + (int64_t)tl.chunk * kSyncStride, 1) == nt - 1;
+            if (last) __threadfence();
+        }
+        if (!__shfl_sync(0xffffffffu, last, 0)) return true;
+        __syncwarp();
+    }
+#pragma unroll
+    for (int r = 0; r < kFewRhs; r++) {
+        if (r >= nb) break;
+        float part = __shfl_sync(0xffffffffu, own[r], 2 * n.j);  // entry j
+        if (nt > 1) part = n.j < w ? __ldcg(acc + (int64_t)(ch.col0 + n.j) * nb + r) : 0.f;
+        const float v = n.diag(yv[r] - part);
+        if (n.lane < w) z[(int64_t)(ch.col0 + n.lane) * nb + r] = v;
+    }
+    __syncwarp();
+    if (n.lane == 0) {
+        __threadfence();
+        atomicExch(done + (int64_t)tl.chunk * kSyncStride, 1);
+    }
+    __syncwarp();
+    return true;
+}
+
 // Forward step of one narrow tile by one warp: wait for the chunk's arrivals,
 // v = L_cc^{-1} x_c (stored FP32 inverse, or FP64 substitution), subtract L_{rows,c} v from x, count the arrivals. false when a wait
 // gave up.
@@ -522,8 +676,11 @@ __global__ void __launch_bounds__(256, 3) k_fwd(const T *__restrict__ lnz, const
                 const int t = su.t0 + wp;
                 const TrsmTile tl = tiles[t];
                 const ChunkDev ch = chunks[tl.chunk];
-                fwd_tile_warp(lnz, ch, tl, t, dep_ptr, dep, need, glbind, x, y, nb, inv, arrive, err, spin_limit,
-                              sm.v + wp * kSmallW * ldv, ldv);
+                if constexpr (RPT == 1)  // up to kFewRhs right-hand sides
+                    fwd_tile_few(lnz, ch, tl, t, dep_ptr, dep, need, glbind, x, y, nb, inv, arrive, err, spin_limit);
+                else
+                    fwd_tile_warp(lnz, ch, tl, t, dep_ptr, dep, need, glbind, x, y, nb, inv, arrive, err, spin_limit,
+                                  sm.v + wp * kSmallW * ldv, ldv);
             }
             __syncthreads();
             continue;
@@ -678,8 +835,12 @@ __global__ void __launch_bounds__(256, 3) k_bwd(const T *__restrict__ lnz, const
                 const int t = su.t0 + wp;
                 const TrsmTile tl = tiles[t];
                 const ChunkDev ch = chunks[tl.chunk];
-                bwd_tile_warp(lnz, ch, tl, t, dep_ptr, dep, ntiles, glbind, y, z, acc, nb, inv, cnt, done, err,
-                              spin_limit, sm.v + wp * kSmallW * ldv, ldv);
+                if constexpr (RPT == 1)  // up to kFewRhs right-hand sides
+                    bwd_tile_few(lnz, ch, tl, t, dep_ptr, dep, ntiles, glbind, y, z, acc, nb, inv, cnt, done, err,
+                                 spin_limit);
+                else
+                    bwd_tile_warp(lnz, ch, tl, t, dep_ptr, dep, ntiles, glbind, y, z, acc, nb, inv, cnt, done, err,
+                                  spin_limit, sm.v + wp * kSmallW * ldv, ldv);
             }
             __syncthreads();
             continue;
