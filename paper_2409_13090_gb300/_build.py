@@ -11,7 +11,7 @@ OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libsc.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["analyze.cpp", "schedule.cpp", "batch.cpp", "api.cpp", "factor.cu", "solve.cu", "probe.cu", "noalloc.cu", "tune.cpp", "check.cpp", "serialize.cpp"]
-HEADERS = ["sc_internal.h", "device_types.h", "kernels.cuh", "numeric.h", "tc_gemm.cuh", "split_gemm.cuh", "fx.cuh", "sweep64.cuh", "chunk64.cuh"]
+HEADERS = ["sc_internal.h", "device_types.h", "kernels.cuh", "numeric.h", "tc_gemm.cuh", "split_gemm.cuh", "fx.cuh", "sweep64.cuh", "chunk64.cuh", "loops64.cuh"]
 
 
 def _nvcc() -> str:

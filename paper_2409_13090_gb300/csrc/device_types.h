@@ -97,6 +97,7 @@ struct SnDev {
     int32_t n;    // |J|
     int32_t b1;   // one past J's last block
     int32_t pad;
+    int64_t gl;   // offset of glbind(J)
 };
 
 // Block descriptor (Sec. 1 / Alg. 5): rows pos..pos+size-1 of Lnz(J) hold the

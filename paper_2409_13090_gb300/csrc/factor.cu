@@ -9,6 +9,7 @@
 #include "numeric.h"
 #include "split_gemm.cuh"
 #include "chunk64.cuh"
+#include "loops64.cuh"
 #include "sweep64.cuh"
 #include "tc_gemm.cuh"
 
@@ -480,13 +481,22 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
                 join = true;
             }
             if (p.loop_cnt) {
-                k_rlb_loop<T><<<p.loop_cnt, 256, 0, ls>>>(lnz, h->d_loops + p.loop_off, h->d_sn, h->d_blk,
-                                                          h->d_rbval);
+                if constexpr (sizeof(T) == 8)
+                    k_rlb_loop64<<<p.loop_cnt, 256, 0, ls>>>((double *)lnz, h->d_loops + p.loop_off, h->d_sn, h->d_blk,
+                                                             h->d_rbval, h->d_row_blk);
+                else
+                    k_rlb_loop<T><<<p.loop_cnt, 256, 0, ls>>>(lnz, h->d_loops + p.loop_off, h->d_sn, h->d_blk,
+                                                              h->d_rbval);
                 launches++;
             }
             if (p.loopw_cnt) {
-                k_rlb_loop_warp<T><<<(p.loopw_cnt + 7) / 8, 256, 0, ls>>>(lnz, h->d_loops + p.loopw_off, p.loopw_cnt,
-                                                                          h->d_sn, h->d_blk, h->d_rbval);
+                if constexpr (sizeof(T) == 8)
+                    k_rlb_loop_warp64<<<(p.loopw_cnt + 7) / 8, 256, 0, ls>>>(
+                        (double *)lnz, h->d_loops + p.loopw_off, p.loopw_cnt, h->d_sn, h->d_blk, h->d_rbval,
+                        h->d_row_blk);
+                else
+                    k_rlb_loop_warp<T><<<(p.loopw_cnt + 7) / 8, 256, 0, ls>>>(
+                        lnz, h->d_loops + p.loopw_off, p.loopw_cnt, h->d_sn, h->d_blk, h->d_rbval);
                 launches++;
             }
             if (join) SC_CUDA(cudaEventRecord(h->ev_join, st2));
@@ -1179,7 +1189,7 @@ int numeric_create(sc_symbolic *s, int precision, sc_numeric **out) {
         std::vector<SnDev> snd(s->nsuper);
         for (int64_t J = 0; J < s->nsuper; J++)
             snd[J] = SnDev{s->lnz_off[J], s->lnz_ld[J], (int32_t)(s->gl_ptr[J + 1] - s->gl_ptr[J]), s->sup_ptr[J],
-                           s->sup_ptr[J + 1] - s->sup_ptr[J], (int32_t)s->blk_ptr[J + 1], 0};
+                           s->sup_ptr[J + 1] - s->sup_ptr[J], (int32_t)s->blk_ptr[J + 1], 0, s->gl_ptr[J]};
         std::vector<BlkDev> bd(s->blk_first.size());
         for (int64_t J = 0; J < s->nsuper; J++) {
             int64_t b0 = s->blk_ptr[J], b1 = s->blk_ptr[J + 1];
@@ -1200,6 +1210,15 @@ int numeric_create(sc_symbolic *s, int precision, sc_numeric **out) {
         if ((rc = upload(h->d_sn, snd, bytes))) return fail(rc);
         if ((rc = upload(h->d_blk, bd, bytes))) return fail(rc);
         if ((rc = upload(h->d_rbval, s->rb_val, bytes))) return fail(rc);
+        if (precision == SC_FP64 && !h->fused && !P.loops.empty()) {
+            std::vector<int32_t> rb(s->glbind.size(), 0);
+            for (int64_t J = 0; J < s->nsuper; J++) {
+                int64_t q = s->gl_ptr[J] + s->sup_ptr[J + 1] - s->sup_ptr[J];
+                for (int64_t b = s->blk_ptr[J]; b < s->blk_ptr[J + 1]; b++)
+                    for (int32_t i = 0; i < s->blk_size[b]; i++) rb[q++] = (int32_t)b;
+            }
+            if ((rc = upload(h->d_row_blk, rb, bytes))) return fail(rc);
+        }
     }
     *out = h;
     return SC_OK;
@@ -1350,7 +1369,7 @@ void numeric_free(sc_numeric *h) {
                     h->d_dep_ptr, h->d_dep, h->d_sync, h->d_serr, h->d_hi, h->d_lo, h->d_thin,
                     h->d_cgz, h->d_cgp, h->d_cgq, h->d_cgs, h->d_solve_units, h->d_flow, h->d_flow_ctr,
                     h->d_flow_need, h->d_task_chunk, h->d_sn_chunk, h->d_splits, h->d_split_units, h->d_split_of_task,
-                    h->d_slices, h->d_exps, h->d_slice_maps, h->d_inv_exp, h->d_chunk64};
+                    h->d_slices, h->d_exps, h->d_slice_maps, h->d_inv_exp, h->d_chunk64, h->d_row_blk};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (h->sym) h->sym->refs--;

@@ -79,6 +79,7 @@ struct sc_numeric {
     sc::SnDev *d_sn = nullptr;
     sc::BlkDev *d_blk = nullptr;
     int32_t *d_rbval = nullptr;
+    int32_t *d_row_blk = nullptr;  // FP64 RLB: the block of every row of glbind (rows below the diagonal blocks)
     sc::LoopItem *d_loops = nullptr;
     CUtensorMap *d_tmaps = nullptr;   // one per panel of width >= 16 (SC_TF32)
     int32_t *d_tmap_of_sn = nullptr;

@@ -117,6 +117,33 @@ __device__ __forceinline__ void digit_row(float (&acc)[S][4], const ulonglong2 (
     for (int j = 0; j < S - i; j++) mma_16816(acc[i + j], a, b[j]);
 }
 
+// The 36 MMAs of a 16 x 8 x 16 block: x the staged pairs of rows g, g + 8 at columns 2 t, and
+// at columns 2 t + 8; y0, y1 those of the other operand's row g.
+__device__ __forceinline__ void digit_product(float (&acc)[S][4], const ulonglong2 (&x)[4], const ulonglong2 &y0,
+                                              const ulonglong2 &y1) {
+    const uint32_t b[S][2] = {{digits<0>(y0), digits<0>(y1)}, {digits<1>(y0), digits<1>(y1)},
+                              {digits<2>(y0), digits<2>(y1)}, {digits<3>(y0), digits<3>(y1)},
+                              {digits<4>(y0), digits<4>(y1)}, {digits<5>(y0), digits<5>(y1)},
+                              {digits<6>(y0), digits<6>(y1)}, {digits<7>(y0), digits<7>(y1)}};
+    digit_row<0>(acc, x, b);
+    digit_row<1>(acc, x, b);
+    digit_row<2>(acc, x, b);
+    digit_row<3>(acc, x, b);
+    digit_row<4>(acc, x, b);
+    digit_row<5>(acc, x, b);
+    digit_row<6>(acc, x, b);
+    digit_row<7>(acc, x, b);
+}
+// a += register e of a block's group sums over at most 64 columns: every pair of groups
+// fits in 32 bits (|g_7| < 2^22.6)
+__device__ __forceinline__ void acc_add64(Acc96 &a, const float (&acc)[S][4], int e) {
+    auto pair = [&](int s) { return __float2int_rn(acc[s][e]) * 256 + __float2int_rn(acc[s + 1][e]); };
+    const int64_t H = ((int64_t)pair(0) << 16) + pair(2), L = ((int64_t)pair(4) << 16) + pair(6);
+    const uint32_t r = a.r + (uint32_t)L;
+    a.t += H + (L >> 32) + (r < (uint32_t)L ? 1 : 0);
+    a.r = r;
+}
+
 // Group sums of a 16 x 8 block of T V (or T^T V): rows 16 mb .. + 15 of the result,
 // right-hand sides n0 .. n0 + 7, inner dimension 16 ks0 .. 16 ks1 - 1. Lane l holds rows l / 4
 // (registers 0, 1) and l / 4 + 8 (2, 3), columns 2 (l % 4) and + 1.
@@ -147,27 +174,15 @@ __device__ __forceinline__ void product(const uint64_t *T, const uint64_t *V, in
         }
         const uint64_t *v = V + (n0 + g) * kLd + k;
         const ulonglong2 y0 = *reinterpret_cast<const ulonglong2 *>(v), y1 = *reinterpret_cast<const ulonglong2 *>(v + 8);
-        const uint32_t b[S][2] = {{digits<0>(y0), digits<0>(y1)}, {digits<1>(y0), digits<1>(y1)},
-                                  {digits<2>(y0), digits<2>(y1)}, {digits<3>(y0), digits<3>(y1)},
-                                  {digits<4>(y0), digits<4>(y1)}, {digits<5>(y0), digits<5>(y1)},
-                                  {digits<6>(y0), digits<6>(y1)}, {digits<7>(y0), digits<7>(y1)}};
-        digit_row<0>(acc, x, b);
-        digit_row<1>(acc, x, b);
-        digit_row<2>(acc, x, b);
-        digit_row<3>(acc, x, b);
-        digit_row<4>(acc, x, b);
-        digit_row<5>(acc, x, b);
-        digit_row<6>(acc, x, b);
-        digit_row<7>(acc, x, b);
+        digit_product(acc, x, y0, y1);
     }
 }
 // value of register e of a block's group sums, times 2^(er + ec)
 __device__ __forceinline__ double block_value(const float (&acc)[S][4], int e, int er, int ec) {
     if (er == kBadExp || ec == kBadExp) return __longlong_as_double(0x7ff8000000000000ll);
-    // at most 64 terms: every pair of groups fits in 32 bits (|g_7| < 2^22.6)
-    auto pair = [&](int s) { return __float2int_rn(acc[s][e]) * 256 + __float2int_rn(acc[s + 1][e]); };
-    const int64_t H = ((int64_t)pair(0) << 16) + pair(2), L = ((int64_t)pair(4) << 16) + pair(6);
-    return acc_value(Acc96{H + (L >> 32), (uint32_t)L}, er + ec);
+    Acc96 a{0, 0};
+    acc_add64(a, acc, e);
+    return acc_value(a, er + ec);
 }
 
 // A warp's part of a 64 x nb block of values, in the layout of the products: rows
