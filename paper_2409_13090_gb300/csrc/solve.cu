@@ -41,8 +41,11 @@ constexpr int kSyncStride = 32;
 constexpr int kSyncWords = 4;
 
 // row stride (elements) of the shared-memory right-hand-side tiles of a block
-// of nb right-hand sides: a multiple of 4, so 16-byte vector loads stay aligned
-__host__ __device__ constexpr int rhs_ld(int nb) { return (nb + 3) / 4 * 4; }
+// of nb right-hand sides: an odd multiple of 4, so 16-byte vector loads stay aligned
+// and the results of a product, a row per lane, go to different banks (with the stride 64 every lane
+// of a warp wrote to the same bank: y_c = inv(L_cc) x_c took 12,000 clocks for 64
+// right-hand sides, the same product without these stores 6,700)
+__host__ __device__ constexpr int rhs_ld(int nb) { return ((nb + 3) / 4 | 1) * 4; }
 
 // right-hand sides per thread in the block products (four thread groups share
 // the block's right-hand sides): 1, 2, 4, 8 or 16
@@ -243,6 +246,23 @@ __device__ __forceinline__ void add_rhs(T *dst, const T (&o)[RPT], T sign, int r
 #pragma unroll
     for (int j = 0; j < RPT; j++)
         if (r0 + j < nb) red_add(dst + j, sign * o[j]);
+}
+
+// dst[0..RPT) = o over the valid right-hand sides r0 + j < nb (FP32; 16-byte stores where
+// nb is a multiple of 4 and so dst is aligned)
+template <int RPT>
+__device__ __forceinline__ void put_rhs(float *dst, const float (&o)[RPT], int r0, int nb) {
+    if constexpr (RPT % 4 == 0) {
+        if ((nb & 3) == 0) {
+#pragma unroll
+            for (int j = 0; j < RPT; j += 4)
+                if (r0 + j < nb) *reinterpret_cast<float4 *>(dst + j) = make_float4(o[j], o[j + 1], o[j + 2], o[j + 3]);
+            return;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < RPT; j++)
+        if (r0 + j < nb) dst[j] = o[j];
 }
 
 // Bounded wait until *flag >= target (acquire at GPU scope). Gives up, setting
@@ -752,12 +772,10 @@ __global__ void __launch_bounds__(256, 3) k_fwd(const T *__restrict__ lnz, const
 #pragma unroll
                     for (int h = 0; h < Map::NR; h++) {
                         const int k = m.row(h);
-#pragma unroll
-                        for (int j = 0; j < Map::R; j++)
-                            if (k < w && m.r0 + j < nb) {
-                                sm.v[k * ldv + m.r0 + j] = o[h][j];
-                                y[(int64_t)(ch.col0 + k) * nb + m.r0 + j] = o[h][j];
-                            }
+                        if (k < w) {
+                            put_rhs<Map::R>(sm.v + k * ldv + m.r0, o[h], m.r0, nb);
+                            put_rhs<Map::R>(y + (int64_t)(ch.col0 + k) * nb + m.r0, o[h], m.r0, nb);
+                        }
                     }
                 }
             }
@@ -944,9 +962,26 @@ __global__ void __launch_bounds__(256, 3) k_bwd(const T *__restrict__ lnz, const
 #pragma unroll
             for (int h = 0; h < Map::NR; h++) {
                 const int k = m.row(h);
+                if (k >= w) continue;
+                T *xi = sm.xin + k * ldv + m.r0, *vi = sm.v + k * ldv + m.r0;
+                if constexpr (Map::R % 4 == 0) {
+                    // whole pieces also at a ragged end: the row's padding is never read
 #pragma unroll
-                for (int j = 0; j < Map::R; j++)
-                    if (k < w && m.r0 + j < nb) sm.xin[k * ldv + m.r0 + j] -= sm.v[k * ldv + m.r0 + j] + o[h][j];
+                    for (int j = 0; j < Map::R; j += 4) {
+                        if (m.r0 + j >= nb) break;
+                        float4 a = *reinterpret_cast<float4 *>(xi + j);
+                        const float4 b = *reinterpret_cast<const float4 *>(vi + j);
+                        a.x -= b.x + o[h][j];
+                        a.y -= b.y + o[h][j + 1];
+                        a.z -= b.z + o[h][j + 2];
+                        a.w -= b.w + o[h][j + 3];
+                        *reinterpret_cast<float4 *>(xi + j) = a;
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < Map::R; j++)
+                        if (m.r0 + j < nb) xi[j] -= vi[j] + o[h][j];
+                }
             }
         }
         __syncthreads();
@@ -958,9 +993,7 @@ __global__ void __launch_bounds__(256, 3) k_bwd(const T *__restrict__ lnz, const
 #pragma unroll
                 for (int h = 0; h < Map::NR; h++) {
                     const int k = m.row(h);
-#pragma unroll
-                    for (int j = 0; j < Map::R; j++)
-                        if (k < w && m.r0 + j < nb) z[(int64_t)(ch.col0 + k) * nb + m.r0 + j] = zo[h][j];
+                    if (k < w) put_rhs<Map::R>(z + (int64_t)(ch.col0 + k) * nb + m.r0, zo[h], m.r0, nb);
                 }
             }
         }
