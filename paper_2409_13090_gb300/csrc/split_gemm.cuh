@@ -25,12 +25,14 @@
 // smaller than the FMA chain's (K = 64 .. 512).
 //
 // Tile 128 x 64: the eight groups' accumulators fill the 512 TMEM columns, so the
-// next 128 columns wait for the drain. Measured at 10000 x 3000: 11.7 TFLOP/s
-// (FP64 operations) at K = 64, 17.3 at 128, 19.7 at 1024, against 1.2 for the SIMT
-// tiles; without the drains 27.7 (an M = 128, N = 64, K = 16 MMA takes some 70
-// clocks, about twice its share of the peak: 128 columns would need 1024 columns
-// of TMEM). Factorizations: 48^3 7-point 77.1 -> 22.8 ms, 80^3 27-point 1541 ->
-// 217 ms.
+// next 128 columns wait for the drain. A slice of A is multiplied by up to four slices
+// of B in one MMA (N = 256): they lie one after another in shared memory, and so do the
+// groups that the products go to. The 36 products one by one (N = 64, some 70 clocks
+// each, about twice their share of the peak: 128 rows of A are read for 64 of
+// B) reached 11.7 TFLOP/s (FP64 operations) at K = 64, 17.3 at 128, 19.7 at 1024 on
+// 10000 x 3000, against 1.2 for the SIMT tiles; by 12 MMAs the steps of 48^3
+// 7-point take 18.1 instead of 18.9 ms, 80^3 27-point 178 instead of 197, with the same bits.
+// Factorizations on the SIMT tiles: 77 and 1541 ms.
 #pragma once
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -231,8 +233,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const GemmTile tl = tiles[t];
                 const Task tk = tasks[tl.task];
                 const int nk = (tk.k + BK - 1) / BK;
-                const int nn = min(BN, (tk.n - tl.tn * BN + 15) / 16 * 16);
-                const uint32_t idesc = idesc_f16(nn);
                 for (int kb = 0; kb < nk; kb++, g++) {
                     const bool first = kb % kDrain == 0;
                     if (first && drains > 0 && !mbar_wait(smem_u32(acce), (drains - 1) & 1u, spin_limit, err, 12)) {
@@ -249,13 +249,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const int ksteps = min(BK / 16, (tk.k - kb * BK + 15) / 16);
                     for (int kk = 0; kk < ksteps; kk++) {  // 16 FP16 = 32 bytes along K inside the swizzle row
                         const uint64_t ad = umma_desc_sw64(a0 + kk * 32), bd = umma_desc_sw64(b0 + kk * 32);
-                        // group by group; within a group every pair of slices i + j = g (0-based)
+                        // slice i of A times the slices j .. j + 3 of B at once: B's slices lie one
+                        // after another, and so do the groups i + j that the products go to
 #pragma unroll
-                        for (int gr = 0; gr < S; gr++)
+                        for (int i = 0; i < S; i++)
 #pragma unroll
-                            for (int i = 0; i <= gr; i++)
-                                mma_f16(tmem + gr * BN, ad + (uint64_t)(i * (A_BYTES >> 4)),
-                                        bd + (uint64_t)((gr - i) * (B_BYTES >> 4)), idesc,
+                            for (int j = 0; j < S - i; j += 4)
+                                mma_f16(tmem + (i + j) * BN, ad + (uint64_t)(i * (A_BYTES >> 4)),
+                                        bd + (uint64_t)(j * (B_BYTES >> 4)), idesc_f16(BN * (S - i - j < 4 ? S - i - j : 4)),
                                         (first && kk == 0 && i == 0) ? 0u : 1u);
                     }
                     mma_commit(smem_u32(empty + s));
