@@ -1130,9 +1130,14 @@ int numeric_create(sc_symbolic *s, int precision, sc_numeric **out) {
     }
     if (!P.splits.empty()) {
         // the slice pool; without room for it (or with more rows than a tensor map's
-        // coordinate reaches) every FP64 product stays on the SIMT tiles
+        // coordinate reaches) every FP64 product stays on the SIMT tiles. It takes at most
+        // half of what is free: a matrix whose factor and solve vectors fit the device
+        // without the pool must not run out of memory because of it.
         const size_t pool = (size_t)P.slice_pieces * sp::BK * sizeof(uint16_t);
-        if (P.slice_pieces > INT32_MAX || cudaMalloc((void **)&h->d_slices, pool) != cudaSuccess ||
+        size_t free_bytes = 0, total_bytes = 0;
+        if (cudaMemGetInfo(&free_bytes, &total_bytes) != cudaSuccess) return fail(SC_ERR_CUDA);
+        if (P.slice_pieces > INT32_MAX || pool > free_bytes / 2 ||
+            cudaMalloc((void **)&h->d_slices, pool) != cudaSuccess ||
             cudaMalloc((void **)&h->d_exps, (size_t)P.exps * sizeof(int32_t)) != cudaSuccess) {
             cudaGetLastError();
             if (h->d_slices) cudaFree(h->d_slices);
