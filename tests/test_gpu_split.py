@@ -120,3 +120,33 @@ def test_irregular_updates_between_supernodes(variant):
         Lo = o.L_supernodal()
         num.refactor(A.values)
         assert np.abs(num.export_L() - Lo).max() <= TOL * np.abs(Lo).max()
+
+
+@pytest.mark.parametrize("blocks", [600, 3000])
+def test_pivot_roots_over_the_exponent_range(blocks):
+    """2 x 2 blocks [[d, a], [a, e]] with d from 2^-1000 to 2^1000 (both sides of where
+    the POTRFs' approximations give way to the library's functions), by the CTA-wide
+    POTRF (600 chunks on the level) and by warps (3000). With u = 2^-53: 1 / sqrt(d)
+    has one rounding in e's product d y (half of it counts) and one at the end, 1.5 u
+    and less than 2^-58 of the series; sqrt(d) = d rk one more: below 3 u (the
+    library's 1 / sqrt(d), 2 u: 3 u; 3.1 u with the reference's long double). L_10 is
+    a rk, 3 u, or (a / d) sqrt(d): 2 u, 3 u and one more product, 6 u; 6.2 u with the
+    products of these errors."""
+    rng = np.random.default_rng(blocks)
+    d = np.ldexp(rng.uniform(1.0, 2.0, blocks), rng.integers(-1000, 1001, blocks))
+    d[:6] = np.ldexp(1.0, [-1000, -991, -990, 991, 993, 1000])
+    a = d * rng.uniform(-0.5, 0.5, blocks)  # a^2 / d < d
+    n = 2 * blocks
+    values = np.stack([d, a, d], 1).ravel()
+    even = np.arange(0, n, 2)
+    colptr = np.append(np.stack([even // 2 * 3, even // 2 * 3 + 2], 1).ravel(), 3 * blocks)
+    A = inputs.SparseSym(n, colptr.astype(np.int64), np.stack([even, even + 1, even + 1], 1).ravel().astype(np.int32), values)
+    num = sc.Symbolic(A, ordering="natural").factor(A.values, precision="fp64")
+    assert num.rc == 0
+    L = num.export_L()
+    root = np.sqrt(d.astype(np.longdouble))
+    u = 2.0 ** -53
+    L = L.reshape(blocks, 2, 2)
+    assert (np.abs(L[:, 0, 0] - root) <= 3.1 * u * root).all()
+    ref = a / root
+    assert (np.abs(L[:, 1, 0] - ref) <= 6.2 * u * np.abs(ref)).all()
