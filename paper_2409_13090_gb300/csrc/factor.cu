@@ -87,25 +87,41 @@ __global__ void __launch_bounds__(256) k_inverse(const float *__restrict__ lnz, 
 
 
 // Inverses of the factored diagonal blocks of the chunks wider than kNarrowChunk, for
-// the solve sweeps of FP64 factors: L_cc in 16 x 16 blocks; the diagonal ones by
-// substitution (a warp each, a lane per column), then block diagonal by block
-// diagonal W_ij = -W_ii sum_{j <= k < i} L_ik W_kj. Stored as the digits of W's rows (columns
-// times 2^{c_k}, 2^{c_k} the size of L_kk: where W is multiplied, its columns' scales
+// the solve sweeps of FP64 factors: L_cc in 16 x 16 blocks; the diagonal ones W_ii by
+// substitution (a warp each, a lane per column), then W_ij = -W_ii sum_{j <= k < i} L_ik W_kj
+// by digits (fx.cuh) on mma.sync. A warp takes eight columns of W through all the block rows,
+// so nothing but the digits of L and the W_ii passes between warps. An operand has an
+// exponent per row or column of a 16-column panel; in W_ii S the inner index also carries
+// the scale 2^{c_k}, the size of L_kk, as in chunk64.cuh. Stored as the digits of W's rows (columns
+// times 2^{c_k}: where W is multiplied, its columns' scales
 // cancel against those of the other operand, also for D A D), the rows' exponents
-// and minus the columns'. Bound by the FP64 pipe (some 41,000 clocks a block and
-// SM). A step W + W (I - L W) after it changed the solutions' errors by less than the
-// seeds differ (40 seeds of five matrices) and cost another 20,000 clocks.
-constexpr int kInv64Smem = 8 * (2 * kMaxChunk * (kMaxChunk + 1));
-__global__ void __launch_bounds__(256) k_inverse64(const double *__restrict__ lnz, const ChunkDev *__restrict__ chunks,
-                                                   const int32_t *__restrict__ list, uint64_t *__restrict__ inv,
-                                                   int32_t *__restrict__ inv_exp, int32_t *__restrict__ inv_cexp) {
+// and minus the columns'. With the products on the FP64 pipe a block took an SM
+// some 41,000 clocks, 33,000 of them these products; by digits the 48^3 FP64 step takes 18.01
+// instead of 18.12 ms, the 83 x 71 RL factor 0.670 instead of 0.681. What is left is the
+// substitution (136 multiply-adds of a warp, 64 clocks each) and the launch. A step
+// W + W (I - L W) after it changed the solutions' errors by less than the
+// seeds differ (40 seeds of five matrices).
+constexpr int kInv64Smem = 8 * (2 * 64 * fx::kLd + kMaxChunk * (kMaxChunk + 1));
+__global__ void __launch_bounds__(256, 2) k_inverse64(const double *__restrict__ lnz, const ChunkDev *__restrict__ chunks,
+                                                      const int32_t *__restrict__ list, uint64_t *__restrict__ inv,
+                                                      int32_t *__restrict__ inv_exp, int32_t *__restrict__ inv_cexp) {
     extern __shared__ double smem_potrf[];
     __shared__ double rinv[kMaxChunk];
-    __shared__ int32_t e_c[kMaxChunk];
+    __shared__ int32_t e_c[kMaxChunk], e_l[kMaxChunk], e_d[kMaxChunk], e_v[4][kMaxChunk];
     const ChunkDev ch = chunks[list[blockIdx.x]];
-    const int w = ch.w;
-    auto l = reinterpret_cast<double (*)[kMaxChunk + 1]>(smem_potrf);
-    auto v = l + kMaxChunk;
+    const int w = ch.w, nbk = (w + 15) / 16;
+    // T: digits of L's rows left of the diagonal blocks, and of the W_ii there; V: digits of
+    // the columns of W (and of S), in the place of L's values, which are only read before
+    uint64_t *T = reinterpret_cast<uint64_t *>(smem_potrf), *V = T + 64 * fx::kLd;
+    auto l = reinterpret_cast<double (*)[kMaxChunk + 1]>(V);
+    auto v = reinterpret_cast<double (*)[kMaxChunk + 1]>(V + 64 * fx::kLd);
+    auto put = [](double x, int key, int e) {
+        return key == fx::kKeyBad ? 0x8080808080808080ull : fx::split_bytes(x, key - 1022 - e);
+    };
+    auto quad_max = [](int k) {
+        k = max(k, __shfl_xor_sync(0xffffffffu, k, 1));
+        return max(k, __shfl_xor_sync(0xffffffffu, k, 2));
+    };
     load_block(l, lnz + ch.off + (int64_t)ch.c0 * ch.ld + ch.c0, ch.ld, w);
     __syncthreads();
     if (threadIdx.x < kMaxChunk) {
@@ -113,8 +129,16 @@ __global__ void __launch_bounds__(256) k_inverse64(const double *__restrict__ ln
         rinv[threadIdx.x] = threadIdx.x < w ? 1.0 / lk : 0.0;
         e_c[threadIdx.x] = (int)threadIdx.x < w ? ((__double2hiint(lk) >> 20) & 0x7ff) - 1023 : 0;
     }
+    // four threads per row: columns q, q + 4, ...
+    const int r = threadIdx.x / 4, q = threadIdx.x % 4, ob = r / 16 * 16;
+    {
+        int key = fx::kKeyNone;
+        for (int c = q; c < ob; c += 4) key = max(key, fx::exp_key(l[r][c], 0));
+        key = quad_max(key);
+        for (int c = q; c < ob; c += 4) T[r * fx::kLd + c] = put(l[r][c], key, 0);
+        if (q == 0) e_l[r] = fx::key_exp(key);
+    }
     __syncthreads();
-    const int nbk = (w + 15) / 16;
     if ((int)threadIdx.x / 32 < nbk && threadIdx.x % 32 < 16) {
         const int o = threadIdx.x / 32 * 16, j = threadIdx.x % 32;
         double x[16];
@@ -129,37 +153,79 @@ __global__ void __launch_bounds__(256) k_inverse64(const double *__restrict__ ln
         for (int i = 0; i < 16; i++) v[o + i][o + j] = i >= j ? x[i] : 0.0;
     }
     __syncthreads();
-    for (int d = 1; d < nbk; d++) {
-        const int total = (nbk - d) * 256;
-        // the sums, in the transposed place
-        for (int e = threadIdx.x; e < total; e += 256) {
-            const int bj = e / 256, bi = bj + d, r = e / 16 % 16, c = e % 16;
-            double s = 0.0;
-            for (int k = 16 * bj; k < 16 * bi; k++) s += l[16 * bi + r][k] * v[k][16 * bj + c];
-            v[16 * bj + r][16 * bi + c] = s;
-        }
-        __syncthreads();
-        for (int e = threadIdx.x; e < total; e += 256) {
-            const int bj = e / 256, bi = bj + d, r = e / 16 % 16, c = e % 16;
-            double s = 0.0;
+    if (ob < 16 * nbk) {
+        // digits of the W_ii: rows (for W_ii S) and columns (for L_ki W_ii)
+        int kd = fx::kKeyNone, kv = fx::kKeyNone;
 #pragma unroll
-            for (int k = 0; k < 16; k++) s -= v[16 * bi + r][16 * bi + k] * v[16 * bj + k][16 * bi + c];
-            v[16 * bi + r][16 * bj + c] = s;
+        for (int t = ob + q; t < ob + 16; t += 4) {
+            kd = max(kd, fx::exp_key(v[r][t], e_c[t]));
+            kv = max(kv, fx::exp_key(v[t][r], 0));
         }
-        __syncthreads();
+        kd = quad_max(kd);
+        kv = quad_max(kv);
+#pragma unroll
+        for (int t = ob + q; t < ob + 16; t += 4) {
+            T[r * fx::kLd + t] = put(v[r][t], kd, e_c[t]);
+            V[r * fx::kLd + t] = put(v[t][r], kv, 0);
+        }
+        if (q == 0) {
+            e_d[r] = fx::key_exp(kd);
+            e_v[ob / 16][r] = fx::key_exp(kv);
+        }
     }
-    // digits: four threads per row, columns q, q + 4, ...
-    const int r = threadIdx.x / 4, q = threadIdx.x % 4;
+    __syncthreads();
+    // columns n0 .. n0 + 7 of W by this warp, block row by block row (lane: rows r0 and r0 + 8,
+    // columns nc and nc + 1 of a product)
+    const int lane = threadIdx.x % 32, n0 = threadIdx.x / 32 * 8, jb = n0 / 16, nc = n0 + 2 * (lane % 4);
+#pragma unroll 1
+    for (int i = jb + 1; i < nbk; i++) {
+        const int r0 = 16 * i + lane / 4;
+        float acc[fx::S][4];
+        double x[4] = {0.0, 0.0, 0.0, 0.0};
+        int k[2];  // exponent keys of the columns nc, nc + 1
+        // digits of x, its rows times 2^{f0}, 2^{f1}, as columns of V
+        auto put_columns = [&](int f0, int f1) {
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                k[h] = max(fx::exp_key(x[h], f0), fx::exp_key(x[2 + h], f1));
+#pragma unroll
+                for (int o = 4; o < 32; o *= 2) k[h] = max(k[h], __shfl_xor_sync(0xffffffffu, k[h], o));
+                V[(nc + h) * fx::kLd + r0] = put(x[h], k[h], f0);
+                V[(nc + h) * fx::kLd + r0 + 8] = put(x[2 + h], k[h], f1);
+            }
+            __syncwarp();
+        };
+        // S = sum_k L_ik W_kj
+#pragma unroll 1
+        for (int p = jb; p < i; p++) {
+            fx::product<false>(T, V, i, n0, p, p + 1, acc);
+#pragma unroll
+            for (int e = 0; e < 4; e++) x[e] += fx::block_value(acc, e, e_l[r0 + 8 * (e / 2)], e_v[p][nc + e % 2]);
+        }
+        put_columns(-e_c[r0], -e_c[r0 + 8]);
+        fx::product<false>(T, V, i, n0, i, i + 1, acc);
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+            x[e] = -fx::block_value(acc, e, e_d[r0 + 8 * (e / 2)], fx::key_exp(k[e % 2]));
+            v[r0 + 8 * (e / 2)][nc + e % 2] = x[e];
+        }
+        __syncwarp();  // S's digits have been read
+        put_columns(0, 0);
+        if (lane < 4) {
+            e_v[i][nc] = fx::key_exp(k[0]);
+            e_v[i][nc + 1] = fx::key_exp(k[1]);
+        }
+        __syncwarp();
+    }
+    __syncthreads();
+    // digits of the rows
     int key = fx::kKeyNone;
     for (int c = q; c <= r; c += 4) key = max(key, fx::exp_key(v[r][c], e_c[c]));
-    key = max(key, __shfl_xor_sync(0xffffffffu, key, 1));
-    key = max(key, __shfl_xor_sync(0xffffffffu, key, 2));
+    key = quad_max(key);
     if (r >= w) return;
-    for (int c = q; c < w; c += 4)
-        inv[ch.inv + r * w + c] =
-            c > r || key == fx::kKeyBad ? 0x8080808080808080ull : fx::split_bytes(v[r][c], key - 1022 - e_c[c]);
+    for (int c = q; c < w; c += 4) inv[ch.inv + r * w + c] = c > r ? 0x8080808080808080ull : put(v[r][c], key, e_c[c]);
     if (q == 0) {
-        inv_exp[ch.col0 + r] = key == fx::kKeyBad ? fx::kBadExp : key - 1022;
+        inv_exp[ch.col0 + r] = fx::key_exp(key);
         inv_cexp[ch.col0 + r] = -e_c[r];
     }
 }

@@ -150,3 +150,16 @@ def test_pivot_roots_over_the_exponent_range(blocks):
     assert (np.abs(L[:, 0, 0] - root) <= 3.1 * u * root).all()
     ref = a / root
     assert (np.abs(L[:, 1, 0] - ref) <= 6.2 * u * np.abs(ref)).all()
+
+
+@pytest.mark.parametrize("chunk", [17, 31, 32, 33, 48, 49, 63, 64])
+def test_solve_by_inverses_of_every_width(chunk):
+    """Diagonal blocks of one to four 16-column panels, whole and ragged, and a last chunk
+    of another width. Diagonally dominant, so 2 n u of the largest entry rounded up to 1e-12."""
+    A = _dense(170, chunk)
+    B = inputs.rhs(A.n, 9, chunk)
+    o = oracle.Oracle(A, None, pr=True)
+    assert o.factor() == 0
+    x0 = o.solve(B)
+    X, _ = sc.Symbolic(A, ordering="natural", chunk=chunk).factor(A.values, precision="fp64").solve(B)
+    assert np.abs(X - x0).max() <= 1e-12 * np.abs(x0).max()
