@@ -148,17 +148,25 @@ def _e2e(num, A, B, stream, steps, **solve_kw):
                                                "lib_copy_out_ms": sum(cout) / len(cout), **rates}
 
 
+# an FP64 product as products of 8-bit digits on the tensor cores, and the classes that use them
+DIGIT_PRODUCTS = 36
+DIGIT_CLASSES = ("gemm_tc", "trsm", "rlb_loop", "rl_update")
+
+
 def _class_rooflines(prof, peaks, fp_peak, precision, workload, scale, merge):
     """Per kernel class of one factorization: algorithmic flops / summed launch
     time against the class's peak (SIMT classes: the measured FMA rate of the
-    storage precision; tensor-core tiles: the TF32 peak)."""
+    storage precision; tensor-core tiles: the TF32 peak; FP64 where it runs as 36
+    products of 8-bit digits: a 36th of the FP16 peak)."""
     out = {}
     tf32 = peaks["bf16_tflops_sustained"] * (1.1 / 2.25)
     for k, v in prof.items():
         if not v["launches"]:
             continue
         ach = v["flops"] / (v["ms"] * 1e-3) / 1e12 if v["ms"] > 0 else 0.0
-        if k == "gemm_tc":
+        if precision == "fp64" and k in DIGIT_CLASSES:
+            pk, bound = peaks["bf16_tflops_sustained"] / DIGIT_PRODUCTS, "tensor"
+        elif k == "gemm_tc":
             pk, bound = tf32, "tensor"
         else:
             pk, bound = fp_peak["fp64" if precision == "fp64" else "fp32"], "alu"
@@ -176,7 +184,7 @@ def _class_rooflines(prof, peaks, fp_peak, precision, workload, scale, merge):
 def _solve_roofline(view, n, nrhs, s_l, ms, sweeps, peaks, peak_kind, fma_peak):
     """A triangular solve against both of its limits: HBM (per sweep nnz(L) x
     entry size + 2 n nrhs x entry size + |glbind| x 4 bytes) and the FMA rate of
-    the storage precision (2 nnz(L) nrhs flops per sweep); the larger of the
+    FP32 or the FP64 rate by digit products (2 nnz(L) nrhs flops per sweep); the larger of the
     two floors is the bound."""
     nnz_l, gl = int(view["nnzL"]), len(view["glbind"])
     byts = sweeps * (nnz_l * s_l + 2 * n * nrhs * s_l + gl * 4)
@@ -189,7 +197,7 @@ def _solve_roofline(view, n, nrhs, s_l, ms, sweeps, peaks, peak_kind, fma_peak):
             "achieved_gbs": byts / (ms * 1e-3) / 1e9, "peak_gbs": peaks["hbm_gbs"],
             "achieved_tflops": flops / (ms * 1e-3) / 1e12, "peak_tflops": fma_peak,
             "bytes": int(byts), "flops": flops, "sweeps": sweeps,
-            "peak_source": f"{peak_kind} HBM copy; measured FMA-tile probe",
+            "peak_source": f"{peak_kind} HBM copy; measured FMA-tile probe (FP64: bf16 sustained / {DIGIT_PRODUCTS})",
             "definition": "per sweep: nnz(L) x entry size + 2 n nrhs x entry size + |glbind| x 4 bytes and "
                           "2 nnz(L) nrhs flops; frac = the larger floor / the measured time"}
 
@@ -688,11 +696,13 @@ def main():
                                                      args.scale, args.merge)
         dom = max(prof, key=lambda k: prof[k]["ms"])
         d = rooflines[args.precision][dom]
-        best_seen = max(value / 1e3, d["achieved_tflops"]) if dom != "gemm_tc" else 0.0
+        best_seen = max(value / 1e3, d["achieved_tflops"]) if d["bound"] != "tensor" else 0.0
         peak = d["peak_tflops"]
-        peak_src = (f"TF32 = {peak_kind} bf16 sustained x 1.1/2.25 (nominal tf32/bf16)" if dom == "gemm_tc" else
+        peak_src = (f"{peak_kind} bf16 sustained / {DIGIT_PRODUCTS} digit products"
+                    if args.precision == "fp64" and dom in DIGIT_CLASSES else
+                    f"TF32 = {peak_kind} bf16 sustained x 1.1/2.25 (nominal tf32/bf16)" if dom == "gemm_tc" else
                     "measured FMA-tile probe (sc_probe_fma_peak)")
-        if dom != "gemm_tc" and peak is not None and best_seen > peak:
+        if d["bound"] != "tensor" and peak is not None and best_seen > peak:
             peak, peak_src = best_seen, "best rate observed in this run (above the probe)"
         roofline = {"bound": d["bound"], "achieved": d["achieved_tflops"], "peak": peak, "unit": "TFLOP/s",
                     "frac": d["achieved_tflops"] / peak if peak else None, "traffic": d["traffic_bytes"],
@@ -706,8 +716,8 @@ def main():
     s_l = 8 if args.precision == "fp64" else 4
     sweeps = 2 * (1 + (sum(iters) / len(iters) if iters else 0))
     rooflines["solve_" + args.precision] = _solve_roofline(
-        view, A.n, nrhs, s_l, sol_ms / K, sweeps, peaks, peak_kind, fp_peak["fp64" if args.precision == "fp64"
-                                                                          else "fp32"])
+        view, A.n, nrhs, s_l, sol_ms / K, sweeps, peaks, peak_kind,
+        peaks["bf16_tflops_sustained"] / DIGIT_PRODUCTS if args.precision == "fp64" else fp_peak["fp32"])
 
     # ---- the chosen form on the same matrix: TF32x3 factor + CG preconditioned by it to eta <= 1e-14
     chosen = None
