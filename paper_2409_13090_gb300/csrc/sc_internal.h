@@ -102,8 +102,9 @@ inline int tc_route_width(const Task &t, int src_width, int min_k, int wide_n, b
 // Does an FP64 product run on the tensor cores as products of FP16 slices
 // (split_gemm.cuh)? The source panel needs 16-byte aligned rows (|J| >= 16: row
 // stride a multiple of 4, panel 256-byte aligned; kx0 even), K >= 16, and enough
-// work: a tile of slice products takes some 6 us, the time in which an SM's FP64
-// pipe makes about 24,000 multiply-adds.
+// work: a tile of slice products took some 6 us when the line was set (its 36 MMAs
+// one by one; the drain and the write are most of a small one), the time in which an SM's
+// FP64 pipe makes about 24,000 multiply-adds.
 constexpr double kSplitMinWork = 32768;
 inline bool split_route(const Task &t, int src_width) {
     return src_width >= 16 && t.k >= 16 && t.kx0 % 2 == 0 && (double)t.m * t.n * t.k >= kSplitMinWork;
