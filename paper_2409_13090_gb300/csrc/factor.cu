@@ -481,6 +481,9 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
         return SC_OK;
     };
     const size_t nlev = h->plans.size();
+    // FP64 by digits, except for a fused handle (here in its profile): its plan has the
+    // FP64-pipe kernels' tiles, and it holds no digits
+    const bool digits = sizeof(T) == 8 && !h->fused;
     for (size_t lv = 0; lv < nlev; lv++) {
         const LevelPlan &p = h->plans[lv];
         if (p.narrow_cnt) {
@@ -493,7 +496,7 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
         }
         if (p.potrf_cnt) {
             B(kProfPotrf);
-            if constexpr (sizeof(T) == 8)
+            if (digits)
                 k_potrf64<<<p.potrf_cnt, 256, kChunk64Smem, st>>>((double *)lnz, h->d_chunks, h->d_potrf + p.potrf_off,
                                                                   h->d_info, h->d_chunk64);
             else
@@ -504,7 +507,7 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
         }
         if (p.trsm_cnt) {
             B(kProfTrsm);
-            if constexpr (sizeof(T) == 8)
+            if (digits)
                 k_trsm64<<<p.trsm_cnt, 256, kChunk64Smem, st>>>((double *)lnz, h->d_chunks, h->d_trsm + p.trsm_off,
                                                                 h->d_chunk64);
             else
@@ -547,7 +550,7 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
                 join = true;
             }
             if (p.loop_cnt) {
-                if constexpr (sizeof(T) == 8)
+                if (digits)
                     k_rlb_loop64<<<p.loop_cnt, 256, 0, ls>>>((double *)lnz, h->d_loops + p.loop_off, h->d_sn, h->d_blk,
                                                              h->d_rbval, h->d_row_blk);
                 else
@@ -556,7 +559,7 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
                 launches++;
             }
             if (p.loopw_cnt) {
-                if constexpr (sizeof(T) == 8)
+                if (digits)
                     k_rlb_loop_warp64<<<(p.loopw_cnt + 7) / 8, 256, 0, ls>>>(
                         (double *)lnz, h->d_loops + p.loopw_off, p.loopw_cnt, h->d_sn, h->d_blk, h->d_rbval,
                         h->d_row_blk);
@@ -631,6 +634,7 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
 int set_smem_attrs() {
     static bool done = false;
     if (done) return SC_OK;
+    SC_CUDA(cudaFuncSetAttribute(k_potrf<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPotrfSmem));
     SC_CUDA(cudaFuncSetAttribute(k_potrf<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPotrfSmem));
     SC_CUDA(cudaFuncSetAttribute(k_potrf64, cudaFuncAttributeMaxDynamicSharedMemorySize, kChunk64Smem));
     SC_CUDA(cudaFuncSetAttribute(k_trsm64, cudaFuncAttributeMaxDynamicSharedMemorySize, kChunk64Smem));

@@ -163,3 +163,20 @@ def test_solve_by_inverses_of_every_width(chunk):
     x0 = o.solve(B)
     X, _ = sc.Symbolic(A, ordering="natural", chunk=chunk).factor(A.values, precision="fp64").solve(B)
     assert np.abs(X - x0).max() <= 1e-12 * np.abs(x0).max()
+
+
+@pytest.mark.parametrize("lookahead", [1, -1])
+@pytest.mark.parametrize("matrix", ["st27", "lap2d"])
+def test_profile_of_a_fused_handle(matrix, lookahead):
+    """A handle with one launch per level holds no digits: its profile runs the FP64-pipe kernels
+    of its own plan, class by class, and leaves the factor. Bound: the module's."""
+    A = inputs.stencil_3d_27pt(13, 11, 12, seed=9) if matrix == "st27" else inputs.laplacian_2d(37, 29, 0.05)
+    sym = sc.Symbolic(A, ordering="grid_nd", grid=A.grid, merge=0.3, tune=dict(fused=1, lookahead=lookahead))
+    num = sym.factor(A.values, precision="fp64")
+    p = num.profile(A.values)
+    assert p["potrf"]["launches"] > 0 and p["trsm"]["launches"] > 0 and p["rlb_loop"]["launches"] > 0
+    assert p["gemm_tc"]["launches"] == 0
+    o = oracle.Oracle(A, oracle.nd_grid(*A.grid, 8), pr=True, merge=0.3)
+    assert o.factor() == 0
+    Lo = o.L_supernodal()
+    assert np.abs(num.export_L() - Lo).max() <= TOL * np.abs(Lo).max()
