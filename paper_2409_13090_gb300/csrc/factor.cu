@@ -105,14 +105,14 @@ constexpr int kInv64Smem = 8 * (2 * 64 * fx::kLd + kMaxChunk * (kMaxChunk + 1));
 __global__ void __launch_bounds__(256, 2) k_inverse64(const double *__restrict__ lnz, const ChunkDev *__restrict__ chunks,
                                                       const int32_t *__restrict__ list, uint64_t *__restrict__ inv,
                                                       int32_t *__restrict__ inv_exp, int32_t *__restrict__ inv_cexp) {
-    extern __shared__ double smem_potrf[];
+    extern __shared__ __align__(16) unsigned char smem_inv64[];  // read 16 bytes at a time
     __shared__ double rinv[kMaxChunk];
     __shared__ int32_t e_c[kMaxChunk], e_l[kMaxChunk], e_d[kMaxChunk], e_v[4][kMaxChunk];
     const ChunkDev ch = chunks[list[blockIdx.x]];
     const int w = ch.w, nbk = (w + 15) / 16;
     // T: digits of L's rows left of the diagonal blocks, and of the W_ii there; V: digits of
     // the columns of W (and of S), in the place of L's values, which are only read before
-    uint64_t *T = reinterpret_cast<uint64_t *>(smem_potrf), *V = T + 64 * fx::kLd;
+    uint64_t *T = reinterpret_cast<uint64_t *>(smem_inv64), *V = T + 64 * fx::kLd;
     auto l = reinterpret_cast<double (*)[kMaxChunk + 1]>(V);
     auto v = reinterpret_cast<double (*)[kMaxChunk + 1]>(V + 64 * fx::kLd);
     auto put = [](double x, int key, int e) {
