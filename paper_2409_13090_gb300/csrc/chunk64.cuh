@@ -12,6 +12,16 @@
 // columns whose scales may differ by any amount (S_ik ~ s_k, W_jk ~ 1 / s_k in D A D): S's
 // columns are taken times 2^{-c_k}, W's times 2^{c_k}, with 2^{c_k} the size of L_kk.
 //
+// The residual S_p - X_p L_pp^T of that product is of the size kappa u, kappa =
+// || |W| |L_pp| ||_inf, where substitution leaves u. Where kappa > kFixPanel one step
+//   X_p <- X_p + (S_p - X_p L_pp^T) W^T
+// follows, whose residual is (kappa u)^2 + u (kappa < 1e8: L_pp is the factor of a matrix
+// that FP64 can factor). Restated on the CPU (Gaussian kernels and chains, 192 points, kappa
+// from 5 to 1e6; residual over sqrt(a_ii a_jj)): FP64 operations 2e-16 to 1.7e-15; without the
+// step 2e-16 to 5e-16 up to kappa = 50, 7e-12 at 1e6, and pivots <= 0 in matrices that
+// can be factored; with it 2e-16 to 6e-16. Diffusion matrices have kappa 5 to 10, at most 40.
+// Forming kappa costs some 2 us a level (48^3 FP64 step 18.03 -> 18.33 ms, 64^2 0.761 -> 0.788).
+//
 // Measured, 64 columns: the FP64-pipe kernels took 70 us for the POTRF (64 pivots of some
 // 900 clocks, and a rank-8 update of 27 us in all) and 19 us for a TRSM tile of
 // 16 rows.
@@ -19,6 +29,8 @@
 #include "sweep64.cuh"
 
 namespace sc {
+
+constexpr float kFixPanel = 32.f;
 
 // dynamic shared memory: the L or X digits of 64 rows (two tiles in the TRSM) and the W digits
 constexpr int kChunk64Smem = 8 * fx::kLd * (64 + 64 + 16);
@@ -77,6 +89,30 @@ __device__ __forceinline__ void panel_mul(double (&v)[4], const uint64_t *T, con
                            key_exp(keyV[n0 + 2 * (lane % 4) + e % 2]));
 }
 
+// The second step for the rows of block mb, columns 8 nb .. + 7 of panel p (by every warp of
+// the CTA; `on`: this one has rows): s holds X_p = S_p W^T, whose keys are in keyX, r holds
+// S_p (its digits would not do: they are relative to the row's largest S_ik 2^{-c_k}, of any
+// size beside the others). L: the rows of L_pp's digits. keyX of the rows from row0 on is left reset.
+__device__ __forceinline__ void panel_fix(double (&s)[4], double (&r)[4], bool on, uint64_t *X, const uint64_t *W,
+                                          const uint64_t *L, int mb, int nb, int p, int *keyS, int *keyX,
+                                          const int *keyL, const int *keyW, int row0, int c0, int c1) {
+    if (on) row_put(s, mb, 16 * p + 8 * nb, keyX, X);
+    __syncthreads();
+    if (threadIdx.x < 64) keyS[threadIdx.x] = kKeyNone;
+    if (on) panel_sub(r, X, L, mb, 8 * nb, p, keyX, keyL);
+    __syncthreads();  // keyS reset; X's digits and keys have been read
+    if ((int)threadIdx.x >= row0 && threadIdx.x < 64) keyX[threadIdx.x] = kKeyNone;
+    if (on) row_keys(r, mb, keyS, -c0, -c1);
+    __syncthreads();
+    if (on) row_put(r, mb, 16 * p + 8 * nb, keyS, X, -c0, -c1);
+    __syncthreads();
+    if (on) {
+        panel_mul(r, X, W, mb, 8 * nb, p, keyS, keyW);
+#pragma unroll
+        for (int e = 0; e < 4; e++) s[e] += r[e];
+    }
+}
+
 // L D L^T of a 16 x 16 block a (lower triangle) by the first four warps: u = the unit
 // lower factor below the diagonal, d = the pivots. A thread holds one entry of the
 // columns 1 .. 15 (120 of them, so every FP64 unit takes five multiply-adds a
@@ -126,6 +162,28 @@ __device__ __forceinline__ void ldl16(const double (*a)[17], double (*u)[17], do
     }
 }
 
+// |x| 2^e as FP32, truncated (infinity from its range on)
+__device__ __forceinline__ float size_of(double x, int e) {
+    const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff, f = ex + e - 896;
+    if (ex == 0x7ff || f >= 255) return __int_as_float(0x7f800000);
+    return f <= 0 ? 0.f : __int_as_float(f << 23 | (hi & 0xfffff) << 3);
+}
+
+// || |W| |L| ||_inf of 16 x 16 blocks by one warp, sums in a fixed order
+__device__ __forceinline__ float condition16(const float (*W)[17], const float (*L)[17]) {
+    const int lane = threadIdx.x % 32, i = lane % 16, k0 = lane / 16 * 8;
+    float rho = 0.f, kap = 0.f;
+#pragma unroll
+    for (int k = 0; k < 8; k++) rho += L[i][k0 + k];
+    rho += __shfl_xor_sync(0xffffffffu, rho, 16);
+#pragma unroll
+    for (int k = 0; k < 8; k++) kap += W[i][k0 + k] * __shfl_sync(0xffffffffu, rho, k0 + k);
+    kap += __shfl_xor_sync(0xffffffffu, kap, 16);
+#pragma unroll
+    for (int o = 1; o < 16; o *= 2) kap = fmaxf(kap, __shfl_xor_sync(0xffffffffu, kap, o));
+    return kap;
+}
+
 // c with 2^c about sqrt(d)
 __device__ __forceinline__ int half_exp(double d) { return (((__double2hiint(d) >> 20) & 0x7ff) - 1023) >> 1; }
 
@@ -139,7 +197,8 @@ __global__ void __launch_bounds__(256) k_potrf64(double *__restrict__ lnz, const
     extern __shared__ __align__(16) unsigned char smem_chunk64[];
     uint64_t *X = reinterpret_cast<uint64_t *>(smem_chunk64), *W = X + 64 * fx::kLd;  // W: 16 rows
     __shared__ double blk[16][17], u[16][17], d[16], rs[16], col[2][16];
-    __shared__ int keyS[4][64], keyX[4][64], keyW[64], cexp[64];
+    __shared__ int keyS[4][64], keyX[4][64], keyW[64], cexp[64], fix[4];
+    __shared__ float sizeL[16][17], sizeW[16][17];
     const ChunkDev ch = chunks[list[blockIdx.x]];
     const int w = ch.w, np = (w + 15) / 16;
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, mb = warp % 4, nb = warp / 4;
@@ -200,6 +259,7 @@ __global__ void __launch_bounds__(256) k_potrf64(double *__restrict__ lnz, const
                 if (i > k) wv -= ui[k] * wk;
             }
             wv *= rs[i];
+            sizeW[i][j] = fx::size_of(wv, cexp[16 * p + j]);
             atomicMax(&keyW[16 * p + i], fx::exp_key(wv, cexp[16 * p + j]));
         }
         double lv[4] = {0.0, 0.0, 0.0, 0.0};
@@ -209,6 +269,7 @@ __global__ void __launch_bounds__(256) k_potrf64(double *__restrict__ lnz, const
                 const int i = lane / 4 + 8 * (e / 2), j = colx + e % 2;
                 const double sq = d[j] * rs[j];
                 lv[e] = i == j ? sq : i > j ? u[i][j] * sq : 0.0;
+                sizeL[i][j] = fx::size_of(lv[e], -cexp[16 * p + i]);
                 const int r = 16 * p + i, c = 16 * p + j;
                 if (r < w && i >= j) base[(int64_t)r * ch.ld + c] = lv[e];
             }
@@ -223,17 +284,30 @@ __global__ void __launch_bounds__(256) k_potrf64(double *__restrict__ lnz, const
         if (mb == p) fx::row_put(lv, mb, 16 * p + 8 * nb, keyX[p], X);
         else if (mb > p && mb < np) fx::row_put(sp, mb, 16 * p + 8 * nb, keyS[p], X, -c0, -c1);
         __syncthreads();
-        if (mb > p && mb < np) {
+        const bool on = mb > p && mb < np;
+        double S[4] = {sp[0], sp[1], sp[2], sp[3]};
+        if (on) {
             fx::panel_mul(sp, X, W, mb, 8 * nb, p, keyS[p], keyW + 16 * p);
+            fx::row_keys(sp, mb, keyX[p]);
+        } else if (warp == 0) {  // (never among these: it has the rows of panel 0)
+            const float kap = fx::condition16(sizeW, sizeL);
+            if (lane == 0) fix[p] = !(kap <= kFixPanel);
+        }
+        __syncthreads();
+        if (fix[p] && p + 1 < np) {
+            fx::panel_fix(sp, S, on, X, W, X + 16 * p * fx::kLd, mb, nb, p, keyS[p], keyX[p], keyX[p] + 16 * p,
+                          keyW + 16 * p, 16 * p + 16, c0, c1);
+            if (on) fx::row_keys(sp, mb, keyX[p]);
+            __syncthreads();
+        }
+        if (on) {
 #pragma unroll
             for (int e = 0; e < 4; e++) {
                 const int r = row0 + 8 * (e / 2), c = 16 * p + colx + e % 2;
                 if (r < w && c < w) base[(int64_t)r * ch.ld + c] = sp[e];
             }
-            fx::row_keys(sp, mb, keyX[p]);
+            fx::row_put(sp, mb, 16 * p + 8 * nb, keyX[p], X);
         }
-        __syncthreads();
-        if (mb > p && mb < np) fx::row_put(sp, mb, 16 * p + 8 * nb, keyX[p], X);
         __syncthreads();
 #pragma unroll
         for (int q = 0; q < 3; q++)
@@ -241,7 +315,7 @@ __global__ void __launch_bounds__(256) k_potrf64(double *__restrict__ lnz, const
             for (int e = 0; e < 4; e++) s[q][e] = s[q + 1][e];
     }
     // to the slot: L digits [16 np][16 np], W digits [np][16][16], keys of L [4][64], of W
-    // [64], the columns' exponents [64]
+    // [64], the columns' exponents [64], which panels take the second step [4]
     uint64_t *out = slots + (int64_t)ch.slot * 256;
     const int n = 16 * np;
     for (int e = threadIdx.x; e < n * n; e += 256) {
@@ -255,6 +329,7 @@ __global__ void __launch_bounds__(256) k_potrf64(double *__restrict__ lnz, const
     if (threadIdx.x < 64) {
         ko[256 + threadIdx.x] = keyW[threadIdx.x];
         ko[320 + threadIdx.x] = (int)threadIdx.x < n ? cexp[threadIdx.x] : 0;
+        if (threadIdx.x < 4) ko[384 + threadIdx.x] = (int)threadIdx.x < np ? fix[threadIdx.x] : 0;
     }
 }
 
@@ -264,7 +339,8 @@ __global__ void __launch_bounds__(256, 2) k_trsm64(double *__restrict__ lnz, con
                                                    const uint64_t *__restrict__ slots) {
     extern __shared__ __align__(16) unsigned char smem_chunk64[];
     uint64_t *X = reinterpret_cast<uint64_t *>(smem_chunk64), *L = X + 64 * fx::kLd, *W = L + 64 * fx::kLd;
-    __shared__ int keyS[4][64], keyX[4][64], keyL[4][64], keyW[64], cexp[64];
+    __shared__ int keyS[4][64], keyX[4][64], keyL[4][64], keyW[64], cexp[64], fix[4];
+    __shared__ double keep[256][5];  // a thread's S_p (in registers it would spill)
     const TrsmTile tl = tiles[blockIdx.x];
     const ChunkDev ch = chunks[tl.chunk];
     const int w = ch.w, np = (w + 15) / 16, n = 16 * np, rows = min(kTrsm64Rows, ch.m - tl.r0);
@@ -290,6 +366,7 @@ __global__ void __launch_bounds__(256, 2) k_trsm64(double *__restrict__ lnz, con
     if (threadIdx.x < 64) {
         keyW[threadIdx.x] = ki[256 + threadIdx.x];
         cexp[threadIdx.x] = ki[320 + threadIdx.x];
+        if (threadIdx.x < 4) fix[threadIdx.x] = ki[384 + threadIdx.x];
     }
     __syncthreads();
 #pragma unroll 1
@@ -306,13 +383,28 @@ __global__ void __launch_bounds__(256, 2) k_trsm64(double *__restrict__ lnz, con
         if (on) fx::row_put(sp, mb, 16 * p + 8 * nb, keyS[p], X, -c0, -c1);
         __syncthreads();
         if (on) {
+            if (fix[p]) {
+#pragma unroll
+                for (int e = 0; e < 4; e++) keep[threadIdx.x][e] = sp[e];
+            }
             fx::panel_mul(sp, X, W, mb, 8 * nb, p, keyS[p], keyW + 16 * p);
+            if (p + 1 < np || fix[p]) fx::row_keys(sp, mb, keyX[p]);
+        }
+        if (fix[p]) {
+            __syncthreads();
+            double S[4];
+#pragma unroll
+            for (int e = 0; e < 4; e++) S[e] = on ? keep[threadIdx.x][e] : 0.0;
+            fx::panel_fix(sp, S, on, X, W, L + 16 * p * fx::kLd, mb, nb, p, keyS[p], keyX[p], keyL[p] + 16 * p,
+                          keyW + 16 * p, 0, c0, c1);
+            if (on) fx::row_keys(sp, mb, keyX[p]);
+        }
+        if (on) {
 #pragma unroll
             for (int e = 0; e < 4; e++) {
                 const int r = row0 + 8 * (e / 2), c = 16 * p + colx + e % 2;
                 if (r < rows && c < w) base[(int64_t)r * ch.ld + c] = sp[e];
             }
-            if (p + 1 < np) fx::row_keys(sp, mb, keyX[p]);
         }
         if (p + 1 >= np) break;
         __syncthreads();

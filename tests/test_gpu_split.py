@@ -180,3 +180,41 @@ def test_profile_of_a_fused_handle(matrix, lookahead):
     assert o.factor() == 0
     Lo = o.L_supernodal()
     assert np.abs(num.export_L() - Lo).max() <= TOL * np.abs(Lo).max()
+
+
+def _dense_sym(M):
+    n = len(M)
+    cols = np.concatenate([[0], np.cumsum(np.arange(n, 0, -1))]).astype(np.int64)
+    rows = np.concatenate([np.arange(j, n) for j in range(n)]).astype(np.int32)
+    return inputs.SparseSym(n, cols, rows, np.concatenate([M[j:, j] for j in range(n)]))
+
+
+def _kernel_matrix(n, length, nugget):
+    """Gaussian kernel on n equally spaced points of [0, 1]: its leading blocks are
+    as ill-conditioned as the nugget allows (2-norm condition about n / nugget)."""
+    t = np.linspace(0.0, 1.0, n)
+    return np.exp(-0.5 * ((t[:, None] - t) / length) ** 2) + nugget * np.eye(n)
+
+
+@pytest.mark.parametrize("n,chunk", [(192, 64), (150, 64), (192, 24), (131, 33)])
+@pytest.mark.parametrize("nugget", [1e-2, 1e-5, 1e-8, 1e-11, 1e-13])
+@pytest.mark.parametrize("length", [0.02, 0.1])
+def test_factor_of_ill_conditioned_blocks(length, nugget, n, chunk):
+    """|A - L L^T| <= (n + 1) u sqrt(a_ii a_jj): the bound of Cholesky in FP64 (Higham, "Accuracy and
+    Stability of Numerical Algorithms", 10.3, with |L| |L|^T <= sqrt(a_ii a_jj)), whatever
+    the condition; and no pivot <= 0 where the oracle finds none."""
+    M = _kernel_matrix(n, length, nugget)
+    A = _dense_sym(M)
+    o = oracle.Oracle(A, None, pr=True)
+    assert o.factor() == 0
+    sym = sc.Symbolic(A, ordering="natural", chunk=chunk)
+    num = sym.factor(A.values, precision="fp64")
+    assert num.rc == 0
+    v = sym.view()
+    perm = np.asarray(v["perm"], dtype=np.int64)
+    assert v["nsuper"] == 1
+    L = np.tril(num.export_L().reshape(n, n)).astype(np.longdouble)
+    P = M[np.ix_(perm, perm)]
+    d = np.sqrt(np.diag(P))
+    res = np.abs(P.astype(np.longdouble) - L @ L.T) / np.outer(d, d)
+    assert res.max() <= (n + 1) * 2.0 ** -53
