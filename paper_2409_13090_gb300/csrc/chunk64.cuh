@@ -162,13 +162,6 @@ __device__ __forceinline__ void ldl16(const double (*a)[17], double (*u)[17], do
     }
 }
 
-// |x| 2^e as FP32, truncated (infinity from its range on)
-__device__ __forceinline__ float size_of(double x, int e) {
-    const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff, f = ex + e - 896;
-    if (ex == 0x7ff || f >= 255) return __int_as_float(0x7f800000);
-    return f <= 0 ? 0.f : __int_as_float(f << 23 | (hi & 0xfffff) << 3);
-}
-
 // || |W| |L| ||_inf of 16 x 16 blocks by one warp, sums in a fixed order
 __device__ __forceinline__ float condition16(const float (*W)[17], const float (*L)[17]) {
     const int lane = threadIdx.x % 32, i = lane % 16, k0 = lane / 16 * 8;

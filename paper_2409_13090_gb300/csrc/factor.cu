@@ -98,16 +98,23 @@ __global__ void __launch_bounds__(256) k_inverse(const float *__restrict__ lnz, 
 // and minus the columns'. With the products on the FP64 pipe a block took an SM
 // some 41,000 clocks, 33,000 of them these products; by digits the 48^3 FP64 step takes 18.01
 // instead of 18.12 ms, the 83 x 71 RL factor 0.670 instead of 0.681. What is left is the
-// substitution (136 multiply-adds of a warp, 64 clocks each) and the launch. A step
-// W + W (I - L W) after it changed the solutions' errors by less than the
-// seeds differ (40 seeds of five matrices).
+// substitution (136 multiply-adds of a warp, 64 clocks each) and the launch.
+//
+// W rounded to FP64 would cost the sweeps' y = W x a residual of || |W| |L| || u = kappa u. The digits
+// have nine bits more: R = I - L W is formed by digits (exact sums, the identity subtracted
+// from the whole numbers), and W R in FP32 is added to the digits of W. The solution's backward
+// error then is that of substitution up to kappa of some 2000 (sweep64.cuh); chunks above kFixChunk
+// are marked in fix.
 constexpr int kInv64Smem = 8 * (2 * 64 * fx::kLd + kMaxChunk * (kMaxChunk + 1));
 __global__ void __launch_bounds__(256, 2) k_inverse64(const double *__restrict__ lnz, const ChunkDev *__restrict__ chunks,
                                                       const int32_t *__restrict__ list, uint64_t *__restrict__ inv,
-                                                      int32_t *__restrict__ inv_exp, int32_t *__restrict__ inv_cexp) {
+                                                      int32_t *__restrict__ inv_exp, int32_t *__restrict__ inv_cexp,
+                                                      int32_t *__restrict__ fix) {
     extern __shared__ __align__(16) unsigned char smem_inv64[];  // read 16 bytes at a time
     __shared__ double rinv[kMaxChunk];
     __shared__ int32_t e_c[kMaxChunk], e_l[kMaxChunk], e_d[kMaxChunk], e_v[4][kMaxChunk];
+    __shared__ float size_l[kMaxChunk];  // row sums of |L| over the rows' sizes
+    __shared__ int kappa;                // as FP32 bits (not negative, so they compare as whole numbers)
     const ChunkDev ch = chunks[list[blockIdx.x]];
     const int w = ch.w, nbk = (w + 15) / 16;
     // T: digits of L's rows left of the diagonal blocks, and of the W_ii there; V: digits of
@@ -121,6 +128,10 @@ __global__ void __launch_bounds__(256, 2) k_inverse64(const double *__restrict__
     auto quad_max = [](int k) {
         k = max(k, __shfl_xor_sync(0xffffffffu, k, 1));
         return max(k, __shfl_xor_sync(0xffffffffu, k, 2));
+    };
+    auto quad_sum = [](float x) {
+        x += __shfl_xor_sync(0xffffffffu, x, 1);
+        return x + __shfl_xor_sync(0xffffffffu, x, 2);
     };
     load_block(l, lnz + ch.off + (int64_t)ch.c0 * ch.ld + ch.c0, ch.ld, w);
     __syncthreads();
@@ -136,7 +147,15 @@ __global__ void __launch_bounds__(256, 2) k_inverse64(const double *__restrict__
         for (int c = q; c < ob; c += 4) key = max(key, fx::exp_key(l[r][c], 0));
         key = quad_max(key);
         for (int c = q; c < ob; c += 4) T[r * fx::kLd + c] = put(l[r][c], key, 0);
-        if (q == 0) e_l[r] = fx::key_exp(key);
+        const int er = r < w ? 1023 - ((__double2hiint(l[r][r]) >> 20) & 0x7ff) : 0;
+        float sum = 0.f;
+        for (int c = q; c <= r; c += 4) sum += fx::size_of(l[r][c], er);
+        sum = quad_sum(sum);
+        if (q == 0) {
+            e_l[r] = fx::key_exp(key);
+            size_l[r] = sum;
+        }
+        if (threadIdx.x == 0) kappa = 0;
     }
     __syncthreads();
     if ((int)threadIdx.x / 32 < nbk && threadIdx.x % 32 < 16) {
@@ -218,12 +237,86 @@ __global__ void __launch_bounds__(256, 2) k_inverse64(const double *__restrict__
         __syncwarp();
     }
     __syncthreads();
-    // digits of the rows
+    // R = I - L W, columns as above: L's rows and W's columns with one exponent each, so the
+    // sums over all of the inner index are exact
+    fx::stage_tile<true>(T, e_l, lnz + ch.off + (int64_t)ch.c0 * ch.ld + ch.c0, ch.ld, w, w);
+    {
+        int key = fx::kKeyNone;
+        for (int t = r + q; t < w; t += 4) key = max(key, fx::exp_key(v[t][r], 0));
+        key = quad_max(key);
+        for (int t = q; t < kMaxChunk; t += 4)
+            V[r * fx::kLd + t] = t >= r && t < w ? put(v[t][r], key, 0) : 0x8080808080808080ull;
+        if (q == 0) e_v[0][r] = fx::key_exp(key);
+    }
+    __syncthreads();
+    {
+        float res[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            if (i < jb || i >= nbk) continue;
+            float acc[fx::S][4];
+            fx::product<false>(T, V, i, n0, jb, i + 1, acc);
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+                const int row = 16 * i + lane / 4 + 8 * (e / 2), col = nc + e % 2, E = e_l[row] + e_v[0][col];
+                fx::Acc96 a{0, 0};
+                fx::acc_add64(a, acc, e);
+                if (row == col && row < w) fx::acc_sub_one(a, E);
+                res[i][e] = -(float)fx::acc_value(a, E - e_c[row] + e_c[col]);
+            }
+        }
+        __syncwarp();  // V's rows n0 .. + 7 are this warp's alone: R's columns take their place
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            if (i < jb || i >= nbk) continue;
+#pragma unroll
+            for (int e = 0; e < 4; e++)
+                reinterpret_cast<float *>(V + (nc + e % 2) * fx::kLd)[16 * i + lane / 4 + 8 * (e / 2)] = res[i][e];
+        }
+    }
+    __syncthreads();
+    // W, columns times 2^{c_k}, in the place of L's digits; kappa
+    float *wf = reinterpret_cast<float *>(T) + r * (kMaxChunk + 1);
     int key = fx::kKeyNone;
-    for (int c = q; c <= r; c += 4) key = max(key, fx::exp_key(v[r][c], e_c[c]));
+    float sum = 0.f;
+    for (int c = q; c < kMaxChunk; c += 4) {
+        const double x = c <= r && r < w ? v[r][c] : 0.0;
+        const float f = fx::size_of(x, e_c[c]);
+        wf[c] = __double2hiint(x) < 0 ? -f : f;
+        sum += f * size_l[c];
+        if (c <= r) key = max(key, fx::exp_key(x, e_c[c]));
+    }
     key = quad_max(key);
+    sum = quad_sum(sum);
+    if (q == 0) atomicMax(&kappa, __float_as_int(sum));
+    __syncthreads();
+    if (threadIdx.x == 0) fix[list[blockIdx.x]] = !(__int_as_float(kappa) <= kFixChunk);
     if (r >= w) return;
-    for (int c = q; c < w; c += 4) inv[ch.inv + r * w + c] = c > r ? 0x8080808080808080ull : put(v[r][c], key, e_c[c]);
+    // W R, columns q, q + 4, ...
+    float dw[kMaxChunk / 4];
+#pragma unroll
+    for (int m = 0; m < kMaxChunk / 4; m++) dw[m] = 0.f;
+#pragma unroll
+    for (int b = 0; b < 4; b++) {
+        if (16 * b > r) break;
+#pragma unroll 4
+        for (int t = 16 * b; t < 16 * b + 16; t++) {
+            const float x = wf[t];
+#pragma unroll
+            for (int m = 0; m < 4 * b + 4; m++) dw[m] += x * reinterpret_cast<const float *>(V + (q + 4 * m) * fx::kLd)[t];
+        }
+    }
+    // digits of the rows of W + W R (the second term where it is the smaller by 2^8 and more)
+    const int E = key - 1022;
+    const float scale = __int_as_float(min(max(127 + 62 - E, 1), 254) << 23);
+#pragma unroll
+    for (int m = 0; m < kMaxChunk / 4; m++) {
+        const int c = q + 4 * m;
+        if (c >= w) continue;
+        const float d = dw[m] * scale;
+        const int64_t add = c <= r && fabsf(d) < 0x1p54f && key != fx::kKeyBad ? __float2ll_rn(d) : 0;
+        inv[ch.inv + r * w + c] = c > r ? 0x8080808080808080ull : put(v[r][c], key, e_c[c]) + (uint64_t)add;
+    }
     if (q == 0) {
         inv_exp[ch.col0 + r] = fx::key_exp(key);
         inv_cexp[ch.col0 + r] = -e_c[r];
@@ -398,7 +491,7 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
             k_inverse<<<nch, 256, kPotrfSmem, st>>>((const float *)lnz, h->d_chunks, list, (float *)h->d_inv);
         else
             k_inverse64<<<nch, 256, kInv64Smem, st>>>((const double *)lnz, h->d_chunks, list, (uint64_t *)h->d_inv,
-                                                      h->d_inv_exp, h->d_inv_exp + s->n);
+                                                      h->d_inv_exp, h->d_inv_exp + s->n, h->d_inv_exp + 2 * s->n);
         E();
         launches++;
     };
@@ -1195,8 +1288,9 @@ int numeric_create(sc_symbolic *s, int precision, sc_numeric **out) {
         bytes += (int64_t)b;
     }
     if (precision == SC_FP64) {
-        if (cudaMalloc((void **)&h->d_inv_exp, (size_t)s->n * 2 * sizeof(int32_t)) != cudaSuccess) return fail(SC_ERR_OOM);
-        bytes += s->n * 2 * (int64_t)sizeof(int32_t);
+        const size_t b = ((size_t)s->n * 2 + s->chunks.size()) * sizeof(int32_t);
+        if (cudaMalloc((void **)&h->d_inv_exp, b) != cudaSuccess) return fail(SC_ERR_OOM);
+        bytes += (int64_t)b;
     }
     if (!P.splits.empty()) {
         // the slice pool; without room for it (or with more rows than a tensor map's

@@ -54,6 +54,18 @@ __device__ __forceinline__ void acc_add_low(Acc96 &a, uint32_t g5, uint32_t g6, 
     a.t += (L >> 32) + (r < lo ? 1 : 0);
     a.r = r;
 }
+// the accumulator, in units of 2^(e - 68), less 1
+__device__ __forceinline__ void acc_sub_one(Acc96 &a, int e) {
+    const int s = 68 - e;  // 1 is 2^s units
+    if (s < 0 || s > 94) return;
+    if (s >= 32) {
+        a.t -= (int64_t)1 << (s - 32);
+    } else {
+        const uint32_t r = a.r;
+        a.r = r - (1u << s);
+        a.t -= a.r > r ? 1 : 0;
+    }
+}
 // the accumulator times 2^(e - 68) when that is outside FP64's normal range
 static __device__ __noinline__ double acc_value_slow(int64_t t, uint32_t r, int e) {
     return scalbn(scalbn((double)t, 32) + (double)r, e - 68);
@@ -87,6 +99,13 @@ __device__ __forceinline__ double acc_value(const Acc96 &a, int e) {
     if (zero) return 0.0;
     if ((unsigned)(sc + 1021) > 2043u) return acc_value_slow(a.t, a.r, e);
     return __hiloint2double((int)((mh + ((uint32_t)(sc + 1022) << 20)) | (s & 0x80000000u)), (int)ml);
+}
+
+// |x| 2^e as FP32, truncated (infinity from its range on)
+__device__ __forceinline__ float size_of(double x, int e) {
+    const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff, f = ex + e - 896;
+    if (ex == 0x7ff || f >= 255) return __int_as_float(0x7f800000);
+    return f <= 0 ? 0.f : __int_as_float(f << 23 | (hi & 0xfffff) << 3);
 }
 
 }  // namespace fx

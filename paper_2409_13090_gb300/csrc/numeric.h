@@ -86,7 +86,7 @@ struct sc_numeric {
     int32_t *d_err = nullptr;         // nonzero after a bounded device wait gave up
     void *d_inv = nullptr;            // inverses of the chunks' diagonal blocks (FP64: the wide ones, as digits)
     uint64_t *d_chunk64 = nullptr;    // FP64: digits of the level's diagonal blocks, from POTRF to TRSM
-    int32_t *d_inv_exp = nullptr;     // FP64: exponents of the inverses' rows, then minus their columns', by column of the matrix
+    int32_t *d_inv_exp = nullptr;     // FP64: exponents of the inverses' rows, then minus their columns', by column of the matrix; then the chunks whose products with them take a second step
     float *d_hi = nullptr;            // SC_TF32X3: tf32(x) of every final factor entry (same layout as Lnz)
     float *d_lo = nullptr;            // SC_TF32X3: tf32(x - hi)
     int32_t nmaps = 0;                // panels with tensor maps (lo maps follow hi maps for SC_TF32X3)

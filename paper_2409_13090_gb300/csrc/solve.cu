@@ -1021,12 +1021,57 @@ struct Sweep64Args {
     int nrhs;
     int64_t vstride;
     const uint64_t *inv;  // digits of the inverses (k_inverse64)
-    const int32_t *inv_exp, *inv_cexp;
+    const int32_t *inv_exp, *inv_cexp, *fix;
     int32_t *f0, *f1;  // forward: arrivals, ready; backward: tile counts, done
     int64_t sstride;
     int32_t *work, *err;
     long long spin_limit;
 };
+
+// Shared memory of a sweep CTA's diagonal step: the tile of L, the inverse, the vector block,
+// their exponents and keys.
+struct Diag64 {
+    uint64_t *l, *w, *vec;
+    int32_t *e_l, *e_w, *e_c;
+    int *key0, *key1;
+};
+// The second step of an ill-conditioned chunk: forward y_c += W (x_c - L_cc y_c), backward
+// z_c += W^T (t_c - L_cc^T z_c), b = x_c or t_c and s = y_c or z_c in global memory (each thread
+// reads the entries that it wrote). Overwrites d.l. key0 is left reset. Not inlined: few chunks
+// take it, and it would hold registers of the others' step.
+template <int NB, bool kBackward>
+__device__ __noinline__ void diag_fix(const double *__restrict__ lnz, const ChunkDev &ch, int nb, const double *b,
+                                      double *s, Diag64 d) {
+    using Fr = fx::Frag<NB>;
+    const int w = ch.w;
+    const int64_t at = (int64_t)ch.col0 * nb;
+    __syncthreads();  // the first step's operands have been read
+    fx::stage_tile<true>(d.l, d.e_l, lnz + ch.off + (int64_t)ch.c0 * ch.ld + ch.c0, ch.ld, w, w);
+    if (threadIdx.x < kRhsBlk) d.key0[threadIdx.x] = d.key1[threadIdx.x] = fx::kKeyNone;
+    Fr v, r;
+    v.load(w, nb, [&](int i, int n) { return __ldcg(s + at + (int64_t)i * nb + n); });
+    __syncthreads();
+    v.keys(nb, kBackward ? d.e_l : nullptr, d.key0);
+    __syncthreads();
+    v.put(nb, kBackward ? d.e_l : nullptr, d.key0, d.vec);
+    __syncthreads();
+    v.template mul<kBackward, false>(d.l, kBackward ? nullptr : d.e_l, d.vec, d.key0, w, w, nb);
+    r.load(w, nb, [&](int i, int n) { return __ldcg(b + at + (int64_t)i * nb + n); });
+#pragma unroll
+    for (int q = 0; q < NB; q++)
+#pragma unroll
+        for (int e = 0; e < 4; e++) r.v[q][e] -= v.v[q][e];
+    r.keys(nb, kBackward ? d.e_w : d.e_c, d.key1);
+    __syncthreads();  // key1; vec, key0 and the tile have been read
+    r.put(nb, kBackward ? d.e_w : d.e_c, d.key1, d.vec);
+    if (threadIdx.x < kRhsBlk) d.key0[threadIdx.x] = fx::kKeyNone;
+    __syncthreads();
+    r.template mul<kBackward, false>(d.w, kBackward ? d.e_c : d.e_w, d.vec, d.key1, w, w, nb);
+    r.each(w, nb, [&](int i, int n, double x) {
+        const int64_t g = at + (int64_t)i * nb + n;
+        s[g] = __ldcg(s + g) + x;
+    });
+}
 
 template <int NB>
 __global__ void __launch_bounds__(256, 2) k_fwd64(Sweep64Args a) {
@@ -1061,7 +1106,7 @@ __global__ void __launch_bounds__(256, 2) k_fwd64(Sweep64Args a) {
         // the tiles of one wide chunk: its first tile alone (cnt 0), or a run of further ones
         const int c = a.tiles[su.t0].chunk;
         const ChunkDev ch = a.chunks[c];
-        const int w = ch.w, g = su.cnt < 0 ? -su.cnt : 1;
+        const int w = ch.w, g = su.cnt < 0 ? -su.cnt : 1, fix = su.cnt == 0 ? a.fix[c] : 0;
         auto stage = [&](int q) {
             const int r0 = a.tiles[su.t0 + q].r0;
             fx::stage_tile(tl_l, e_l, a.lnz + ch.off + (int64_t)r0 * ch.ld + ch.c0, ch.ld,
@@ -1083,6 +1128,11 @@ __global__ void __launch_bounds__(256, 2) k_fwd64(Sweep64Args a) {
             __syncthreads();
             v.template mul<false, false>(tl_w, e_w, vec, key[1], w, w, nb);  // y_c
             v.each(w, nb, [&](int r, int n, double d) { y[(int64_t)(ch.col0 + r) * nb + n] = d; });
+            if (fix) {
+                diag_fix<NB, false>(a.lnz, ch, nb, x, y, Diag64{tl_l, tl_w, vec, e_l, e_w, e_c, key[0], key[1]});
+                v.load(w, nb, [&](int r, int n) { return __ldcg(y + (int64_t)(ch.col0 + r) * nb + n); });
+                stage(0);
+            }
         } else {
             if (threadIdx.x == 0) s_ok = wait_flag(ready + (int64_t)c * kSyncStride, 1, a.err, a.spin_limit, 7);
             __syncthreads();
@@ -1132,8 +1182,7 @@ __global__ void __launch_bounds__(256, 2) k_bwd64(Sweep64Args a) {
         const int bk = ug % nblk;
         const SolveUnit su = a.units[ug / nblk];
         const int nb = min(kRhsBlk, a.nrhs - bk * kRhsBlk);
-        const double *y = a.y + bk * a.vstride;
-        double *z = a.z + bk * a.vstride, *acc = a.acc + bk * a.vstride;
+        double *y = a.y + bk * a.vstride, *z = a.z + bk * a.vstride, *acc = a.acc + bk * a.vstride;
         int32_t *cnt = a.f0 + bk * a.sstride, *done = a.f1 + bk * a.sstride;
         if (su.cnt > 0) {  // narrow tiles, one per warp
             const int wp = threadIdx.x / 32;
@@ -1152,7 +1201,7 @@ __global__ void __launch_bounds__(256, 2) k_bwd64(Sweep64Args a) {
         const bool first = su.cnt == 0;
         const int c = a.tiles[su.t0].chunk;
         const ChunkDev ch = a.chunks[c];
-        const int w = ch.w, g = first ? 1 : -su.cnt;
+        const int w = ch.w, g = first ? 1 : -su.cnt, fix = first ? a.fix[c] : 0;
         if (first) fx::stage_inverse(tl_w, e_w, e_c, a.inv + ch.inv, a.inv_exp + ch.col0, a.inv_cexp + ch.col0, w);
         if (threadIdx.x < 2 * kRhsBlk) key[threadIdx.x / kRhsBlk][threadIdx.x % kRhsBlk] = fx::kKeyNone;
         Fr o;
@@ -1206,12 +1255,16 @@ __global__ void __launch_bounds__(256, 2) k_bwd64(Sweep64Args a) {
 #pragma unroll
             for (int e = 0; e < 4; e++)
                 if (Fr::row(e) < w && Fr::col(b, e) < nb) v.v[b][e] -= o.v[b][e];
+        // (nobody reads y_c after this)
+        if (fix) v.each(w, nb, [&](int r, int n, double d) { y[(int64_t)(ch.col0 + r) * nb + n] = d; });
         v.keys(nb, e_w, key[1]);  // key[1] is untouched since its reset (one tile at most came before)
         __syncthreads();
         v.put(nb, e_w, key[1], vec);
         __syncthreads();
         v.template mul<true, false>(tl_w, e_c, vec, key[1], w, w, nb);
         v.each(w, nb, [&](int r, int n, double d) { z[(int64_t)(ch.col0 + r) * nb + n] = d; });
+        if (fix)
+            diag_fix<NB, true>(a.lnz, ch, nb, y, z, Diag64{tl_l, tl_w, vec, e_l, e_w, e_c, key[0], key[1]});
         __syncthreads();
         if (threadIdx.x == 0) {
             __threadfence();
@@ -1589,7 +1642,8 @@ void launch_sweeps64(sc_numeric *h, int nrhs, int64_t vs, int64_t ss, double *xw
     const int total = h->solve_tiles * nblk;
     const int grid = std::max(1, std::min(total, std::max(1, std::min(p, q)) * h->num_sms));
     Sweep64Args a{(const double *)h->d_lnz, h->d_chunks, h->d_solve_tiles, h->d_solve_units, total, h->d_dep_ptr,
-                  h->d_dep, h->d_counters + nch, h->d_glbind, xw, y, z, acc, nrhs, vs, (const uint64_t *)h->d_inv, h->d_inv_exp, h->d_inv_exp + h->sym->n, sync,
+                  h->d_dep, h->d_counters + nch, h->d_glbind, xw, y, z, acc, nrhs, vs, (const uint64_t *)h->d_inv, h->d_inv_exp, h->d_inv_exp + h->sym->n,
+                  h->d_inv_exp + 2 * h->sym->n, sync,
                   sync + nch * kSyncStride, ss, sync + nblk * ss, h->d_serr, (long long)h->sym->opt.spin_limit};
     k_fwd64<NB><<<grid, 256, smem, st>>>(a);
     a.count = h->d_counters;

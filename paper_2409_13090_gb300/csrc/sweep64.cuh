@@ -18,11 +18,22 @@
 // scale per column, 2^{-c_k} with 2^{c_k} the size of L_kk, which goes into the other factor or
 // the result: the terms of a product then are of the size of their digits, also for
 // D A D with any diagonal D.
+//
+// With W in FP64 the residual x_c - L_cc y_c would be of the size kappa u, kappa =
+// || |W| |L_cc| ||_inf, where substitution leaves u; k_inverse64 gives W to the digits' 62 bits.
+// In the chunks with kappa > kFixChunk, which it marks, y_c <- y_c + W (x_c - L_cc y_c)
+// follows, likewise backward. Restated on the CPU (192 x 192 Gaussian kernels; mean backward error of
+// the solution, eight right-hand sides): substitution 4e-17 to 1e-16; W in FP64 1e-16 at kappa =
+// 29, 1e-15 at 270, 6e-15 at 2000; W in 62 bits 8e-18 to 8e-17 up to 2000, 3e-16 at 18000; with
+// the step 8e-18 to 8e-17. Blocks of diffusion matrices have kappa 4 to 15, at most 71.
 #pragma once
 #include "fx.cuh"
 #include "kernels.cuh"
 
 namespace sc {
+
+constexpr float kFixChunk = 1000.f;
+
 namespace fx {
 
 constexpr int kLd = 66;            // 64-bit words per row of a staged tile or vector (16 bytes of skew)
@@ -34,8 +45,9 @@ __device__ __forceinline__ int exp_key(double x, int e) {
     return ex == 0x7ff || e == kBadExp ? kKeyBad : max(ex, 1) + e;
 }
 
-// Stages a rows x w block (row stride ld, w <= 64) as a 64 x 64 tile of digits and its row
-// exponents: 256 threads, four per row.
+// Stages a rows x w block (row stride ld, w <= 64; kLower: its lower triangle) as a 64 x 64 tile
+// of digits and its row exponents: 256 threads, four per row.
+template <bool kLower = false>
 __device__ __forceinline__ void stage_tile(uint64_t *T, int32_t *rowE, const double *__restrict__ src, int64_t ld,
                                            int rows, int w) {
     const int r = threadIdx.x / 4, q = threadIdx.x % 4;
@@ -55,6 +67,11 @@ __device__ __forceinline__ void stage_tile(uint64_t *T, int32_t *rowE, const dou
             const int c = 8 * (j / 2) + 2 * q + j % 2;
             v[j] = r < rows && c < w ? p[c] : 0.0;
         }
+    }
+    if constexpr (kLower) {
+#pragma unroll
+        for (int j = 0; j < 16; j++)
+            if (8 * (j / 2) + 2 * q + j % 2 > r) v[j] = 0.0;
     }
     uint32_t top = 0;
 #pragma unroll

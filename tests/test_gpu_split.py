@@ -218,3 +218,27 @@ def test_factor_of_ill_conditioned_blocks(length, nugget, n, chunk):
     d = np.sqrt(np.diag(P))
     res = np.abs(P.astype(np.longdouble) - L @ L.T) / np.outer(d, d)
     assert res.max() <= (n + 1) * 2.0 ** -53
+
+
+@pytest.mark.parametrize("nrhs", [1, 9, 20, 33, 70])
+@pytest.mark.parametrize("what,n,chunk", [("1e-8", 192, 64), ("1e-11", 150, 33), ("1e-13", 192, 24), ("1e-5", 131, 64),
+                                          ("fourth difference", 1024, 64)])
+def test_solve_with_ill_conditioned_blocks(what, n, chunk, nrhs):
+    """Gaussian kernels with a nugget, and the 1D fourth difference as one supernode: the plain FP64
+    solve (no refinement) is backward stable, eta <= 1e-14 (the default ir_tol; n u is 1.5e-14 to
+    1.1e-13), for right-hand sides of smooth, random and random A x."""
+    if what == "fourth difference":
+        M = sum(c * np.eye(n, k=k) for k, c in ((-2, 1.0), (-1, -4.0), (0, 6.0), (1, -4.0), (2, 1.0)))
+    else:
+        M = _kernel_matrix(n, 0.05, float(what))
+    A = _dense_sym(M)
+    rng = np.random.default_rng(nrhs)
+    B = rng.uniform(-1.0, 1.0, (n, nrhs))
+    B[:, ::3] = M @ B[:, ::3]
+    B[:, 1::3] = np.cos(np.arange(n) / n * np.arange(1, nrhs + 1)[1::3, None]).T
+    num = sc.Symbolic(A, ordering="natural", chunk=chunk).factor(A.values, precision="fp64")
+    assert num.rc == 0
+    X, info = num.solve(B)
+    eta = oracle.backward_error(A, B, X)
+    assert eta.max() <= 1e-14, eta.max()
+    assert info["converged"] and info["iterations"] == 0
