@@ -169,7 +169,8 @@ typedef struct sc_options {
     const sc_tune_table *tune; /* launch-plan settings (copied), NULL = defaults     */
     int32_t deterministic;     /* 1 = bit-reproducible factor: every entry of L gets its
                                   updates in one fixed order, so two factorizations of
-                                  the same values give the same bits. Needs variant
+                                  the same values give the same bits (by any two handles,
+                                  whatever device memory was free). Needs variant
                                   SC_RL: the U_J products are stored, never accumulated
                                   (no inner-dimension splitting), and each level's
                                   assembly is owned by the targets (a CTA per row slab
@@ -559,6 +560,12 @@ int sc_test_stall_solve(sc_numeric *h, int64_t chunk);
  * Errors: -1 (h NULL), -2 (chunk < 0); the next factorization returns
  * SC_ERR_UNSUPPORTED if h has no per-level kernel or chunk is out of range. */
 int sc_test_stall_factor(sc_numeric *h, int64_t chunk);
+
+/* Test hook: h gives up the device memory for the slices of its FP64 products, as
+ * sc_factor without room for it and sc_solve short of memory do; later
+ * factorizations form the same products without it, to the same bits.
+ * Errors: -1 (h NULL), SC_ERR_UNSUPPORTED when h holds none. */
+int sc_test_drop_slices(sc_numeric *h);
 
 /* Frees h and its device memory. NULL is accepted. */
 void sc_numeric_free(sc_numeric *h);

@@ -128,6 +128,7 @@ def lib():
             "sc_plan_stats": ([P, C.c_int, P, C.c_int], C.c_int),
             "sc_test_stall_solve": ([P, i64], C.c_int),
             "sc_test_stall_factor": ([P, i64], C.c_int),
+            "sc_test_drop_slices": ([P], C.c_int),
             "sc_factor_batch": ([C.c_int, P, P, C.c_int, C.c_int, P, C.POINTER(P), C.POINTER(P), P], C.c_int),
             "sc_tune": ([P, P, C.c_int, C.c_int, C.c_int, P, P, P], C.c_int),
             "sc_check_schedule": ([P, P, C.c_int], C.c_int),
@@ -511,6 +512,12 @@ class Numeric:
         rc = lib().sc_test_stall_factor(self._h, int(chunk))
         if rc:
             raise SCError(rc, "sc_test_stall_factor")
+
+    def drop_slices(self):
+        """Test hook (sc_test_drop_slices): later factorizations run without the memory for slices."""
+        rc = lib().sc_test_drop_slices(self._h)
+        if rc:
+            raise SCError(rc, "sc_test_drop_slices")
 
     def stall_next_solve(self, chunk: int):
         """Test hook (sc_test_stall_solve): the next solve's forward sweep waits at

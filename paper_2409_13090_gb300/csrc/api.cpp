@@ -242,6 +242,11 @@ int sc_test_stall_factor(sc_numeric *h, int64_t chunk) {
     return SC_OK;
 }
 
+int sc_test_drop_slices(sc_numeric *h) {
+    if (!h) return -1;
+    return sc::drop_slices(h) ? SC_OK : SC_ERR_UNSUPPORTED;
+}
+
 void sc_numeric_free(sc_numeric *h) { sc::numeric_free(h); }
 
 const char *sc_strerror(int code) {

@@ -521,6 +521,14 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
         return SC_OK;
     }
     // tiled products of one dependency class on stream ps
+    auto digit_products = [&](int32_t off, int32_t cnt, cudaStream_t ps) {
+        if (h->d_slices)
+            launch_split_gemm((double *)lnz, (double *)pool, h->d_tasks, h->d_gemm + off, cnt, h->d_split_of_task,
+                              h->d_splits, h->d_exps, h->d_slice_maps, h->d_err, (long long)s->opt.spin_limit,
+                              h->num_sms, ps);
+        else
+            k_digit_tiles<<<cnt, 256, 0, ps>>>((double *)lnz, (double *)pool, h->d_tasks, h->d_gemm + off);
+    };
     auto products = [&](const ProdLists &pl, cudaStream_t ps) -> int {
         if (pl.gemm_cnt) {
             B(kProfGemm);
@@ -532,9 +540,7 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
         if constexpr (sizeof(T) == 8) {
             if (pl.sp_cnt) {
                 B(kProfTc);
-                launch_split_gemm((double *)lnz, (double *)pool, h->d_tasks, h->d_gemm + pl.sp_off, pl.sp_cnt,
-                                  h->d_split_of_task, h->d_splits, h->d_exps, h->d_slice_maps, h->d_err,
-                                  (long long)s->opt.spin_limit, h->num_sms, ps);
+                digit_products(pl.sp_off, pl.sp_cnt, ps);
                 E();
                 launches++;
             }
@@ -612,7 +618,7 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
         if constexpr (sizeof(T) == 8) {
             // the level's half of the slice pool was last read by the products of level
             // lv - 2, which this stream has waited for (ev_rest, at level lv - 1)
-            if (p.split_cnt) {
+            if (p.split_cnt && h->d_slices) {
                 B(kProfTc);
                 launch_split((const double *)lnz, h->d_splits, h->d_split_units + p.split_off, p.split_cnt,
                              h->d_slices, h->d_exps, st);
@@ -686,9 +692,7 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
         if constexpr (sizeof(T) == 8) {
             if (p.rlsp_cnt) {
                 B(kProfRlUpd);
-                launch_split_gemm((double *)lnz, (double *)pool, h->d_tasks, h->d_gemm + p.rlsp_off, p.rlsp_cnt,
-                                  h->d_split_of_task, h->d_splits, h->d_exps, h->d_slice_maps, h->d_err,
-                                  (long long)s->opt.spin_limit, h->num_sms, st);
+                digit_products(p.rlsp_off, p.rlsp_cnt, st);
                 E();
                 launches++;
             }
@@ -1292,32 +1296,6 @@ int numeric_create(sc_symbolic *s, int precision, sc_numeric **out) {
         if (cudaMalloc((void **)&h->d_inv_exp, b) != cudaSuccess) return fail(SC_ERR_OOM);
         bytes += (int64_t)b;
     }
-    if (!P.splits.empty()) {
-        // the slice pool; without room for it (or with more rows than a tensor map's
-        // coordinate reaches) every FP64 product stays on the SIMT tiles. It takes at most
-        // half of what is free: a matrix whose factor and solve vectors fit the device
-        // without the pool must not run out of memory because of it.
-        const size_t pool = (size_t)P.slice_pieces * sp::BK * sizeof(uint16_t);
-        size_t free_bytes = 0, total_bytes = 0;
-        if (cudaMemGetInfo(&free_bytes, &total_bytes) != cudaSuccess) return fail(SC_ERR_CUDA);
-        if (P.slice_pieces > INT32_MAX || pool > free_bytes / 2 ||
-            cudaMalloc((void **)&h->d_slices, pool) != cudaSuccess ||
-            cudaMalloc((void **)&h->d_exps, (size_t)P.exps * sizeof(int32_t)) != cudaSuccess) {
-            cudaGetLastError();
-            if (h->d_slices) cudaFree(h->d_slices);
-            h->d_slices = nullptr;
-            P = Plan();
-            build_plan(s, precision, P, h->lookahead, false);
-        } else {
-            bytes += (int64_t)pool + P.exps * (int64_t)sizeof(int32_t);
-            std::vector<CUtensorMap> maps;
-            if ((rc = split_encode_maps(h->d_slices, P.slice_pieces, maps))) return fail(rc);
-            if ((rc = upload(h->d_slice_maps, maps, bytes))) return fail(rc);
-            if ((rc = upload(h->d_splits, P.splits, bytes))) return fail(rc);
-            if ((rc = upload(h->d_split_units, P.split_units, bytes))) return fail(rc);
-            if ((rc = upload(h->d_split_of_task, P.split_of_task, bytes))) return fail(rc);
-        }
-    }
     if (h->fused) {
         build_flow(P, h->lookahead);
         h->flow_tail_off = P.flow_tail_off;
@@ -1387,6 +1365,31 @@ int numeric_create(sc_symbolic *s, int precision, sc_numeric **out) {
                     for (int32_t i = 0; i < s->blk_size[b]; i++) rb[q++] = (int32_t)b;
             }
             if ((rc = upload(h->d_row_blk, rb, bytes))) return fail(rc);
+        }
+    }
+    if (!P.splits.empty()) {
+        // the slice pool, last. It takes at most half of what is free: a matrix whose factor and
+        // solve vectors fit the device without the pool must not run out of memory because of it
+        // (and a solve that does takes it back). Without it, or with more rows than a tensor
+        // map's coordinate reaches, k_digit_tiles forms the same products to the same bits:
+        // 27-point 40^3 factor 13.3 ms with the pool, 27.5 without; 7-point 48^3 16.3 and 49.9.
+        const size_t pool = (size_t)P.slice_pieces * sp::BK * sizeof(uint16_t);
+        size_t free_bytes = 0, total_bytes = 0;
+        if (cudaMemGetInfo(&free_bytes, &total_bytes) != cudaSuccess) return fail(SC_ERR_CUDA);
+        if (P.slice_pieces <= INT32_MAX && pool <= free_bytes / 2 &&
+            cudaMalloc((void **)&h->d_slices, pool) == cudaSuccess) {
+            h->slice_bytes = (int64_t)pool;
+            bytes += h->slice_bytes;
+            std::vector<CUtensorMap> maps;
+            if ((rc = split_encode_maps(h->d_slices, P.slice_pieces, maps))) return fail(rc);
+            if (cudaMalloc((void **)&h->d_exps, (size_t)P.exps * sizeof(int32_t)) != cudaSuccess) return fail(SC_ERR_OOM);
+            bytes += P.exps * (int64_t)sizeof(int32_t);
+            if ((rc = upload(h->d_slice_maps, maps, bytes))) return fail(rc);
+            if ((rc = upload(h->d_splits, P.splits, bytes))) return fail(rc);
+            if ((rc = upload(h->d_split_units, P.split_units, bytes))) return fail(rc);
+            if ((rc = upload(h->d_split_of_task, P.split_of_task, bytes))) return fail(rc);
+        } else {
+            cudaGetLastError();
         }
     }
     *out = h;
@@ -1518,6 +1521,16 @@ int numeric_export_L(const sc_numeric *h, double *out) {
             }
     }
     return SC_OK;
+}
+
+bool drop_slices(sc_numeric *h) {
+    if (!h->d_slices) return false;
+    if (h->gexec) cudaGraphExecDestroy(h->gexec);
+    h->gexec = nullptr;
+    cudaFree(h->d_slices);
+    h->d_slices = nullptr;
+    h->device_bytes -= h->slice_bytes;
+    return true;
 }
 
 void numeric_free(sc_numeric *h) {

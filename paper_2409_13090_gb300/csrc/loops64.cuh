@@ -20,11 +20,10 @@ constexpr int kFxMinK = 6;
 namespace fx {
 
 // Block of A B^T (A and B rows of one panel, row stride ld, K columns; ni <= 16 rows,
-// nj <= 8 columns) subtracted from the rows c0 (the lane's row l / 4) and c1 (row
-// l / 4 + 8) of the target, where j >= lo0, lo1 are not written (entries above the diagonal).
+// nj <= 8 columns): put(e, i, j, v) for the lane's entries inside it, e < 2 in row l / 4, else in row l / 4 + 8.
+template <typename Put>
 __device__ __forceinline__ void loop_block(const double *__restrict__ A, const double *__restrict__ B, int64_t ld, int K,
-                                           int ni, int nj, double *__restrict__ c0, double *__restrict__ c1, int lo0,
-                                           int lo1) {
+                                           int ni, int nj, Put &&put) {
     const int lane = threadIdx.x % 32, g = lane / 4, t = lane % 4;
     const bool a0 = g < ni, a1 = g + 8 < ni, b0 = g < nj;
     const double *pa = A + g * ld, *pb = B + g * ld;
@@ -75,10 +74,9 @@ __device__ __forceinline__ void loop_block(const double *__restrict__ A, const d
 #pragma unroll
     for (int e = 0; e < 4; e++) {
         const int i = g + 8 * (e / 2), j = 2 * t + e % 2, er = e < 2 ? ea0 : ea1, ec = e % 2 ? e1 : e0;
-        if (i >= ni || j >= nj || j >= (e < 2 ? lo0 : lo1)) continue;
-        const double v = er == kBadExp || ec == kBadExp ? __longlong_as_double(0x7ff8000000000000ll)
-                                                        : acc_value(sum[e], er + ec);
-        atomicAdd((e < 2 ? c0 : c1) + j, -v);
+        if (i >= ni || j >= nj) continue;
+        put(e, i, j, er == kBadExp || ec == kBadExp ? __longlong_as_double(0x7ff8000000000000ll)
+                                                    : acc_value(sum[e], er + ec));
     }
 }
 
@@ -125,10 +123,13 @@ __device__ __forceinline__ void loop_item64(double *__restrict__ lnz, const Loop
             const int ia = i0 + lane / 4, ib = ia + 8;
             int lo0 = 0, lo1 = 0;
             double *c0 = C, *c1 = C;
+            // (entries from lo on are above the diagonal)
             if (ia < r1) c0 = target(ia, lo0);
             if (ib < r1) c1 = target(ib, lo1);
-            fx::loop_block(src + i0 * ld, rowsB + j0 * ld, ld, K, min(16, r1 - i0), min(8, nb - j0), c0 + j0, c1 + j0,
-                           lo0 - j0, lo1 - j0);
+            fx::loop_block(src + i0 * ld, rowsB + j0 * ld, ld, K, min(16, r1 - i0), min(8, nb - j0),
+                           [&](int e, int, int j, double v) {
+                               if (j0 + j < (e < 2 ? lo0 : lo1)) atomicAdd((e < 2 ? c0 : c1) + j0 + j, -v);
+                           });
         }
     }
 }
@@ -147,6 +148,33 @@ __global__ void __launch_bounds__(256, 2) k_rlb_loop_warp64(double *__restrict__
                                                             const int32_t *__restrict__ row_blk) {
     const int idx = blockIdx.x * 8 + threadIdx.x / 32;
     if (idx < count) loop_item64(lnz, items[idx], sn, blk, rb_val, row_blk, 0, 1);
+}
+
+// The product tiles of k_split_gemm (128 x 64) straight from the panels, for handles without
+// a slice pool (no memory for it): a warp takes 16 rows, eight columns at a time. The digits, the rows'
+// exponents and the sums are k_split_gemm's, and the sums are exact, so L has the same
+// bits with and without the pool.
+__global__ void __launch_bounds__(256, 2) k_digit_tiles(double *__restrict__ lnz, double *__restrict__ upool,
+                                                        const Task *__restrict__ tasks,
+                                                        const GemmTile *__restrict__ tiles) {
+    const GemmTile tl = tiles[blockIdx.x];
+    const Task tk = tasks[tl.task];
+    const int i0 = tl.tm * 128 + threadIdx.x / 32 * 16, ni = min(16, tk.m - i0);
+    if (ni <= 0) return;
+    const bool lower = tk.flags & kTaskLower, store = tk.flags & kTaskStoreU, excl = tk.flags & kTaskExclusive;
+    double *C = (store ? upool : lnz) + tk.c_off + (int64_t)i0 * tk.ldc;
+#pragma unroll 1
+    for (int j0 = tl.tn * 64; j0 < min(tk.n, tl.tn * 64 + 64); j0 += 8) {
+        if (lower && i0 + ni - 1 < j0) break;
+        fx::loop_block(lnz + tk.a_off + (int64_t)i0 * tk.lds, lnz + tk.b_off + (int64_t)j0 * tk.lds, tk.lds, tk.k, ni,
+                       min(8, tk.n - j0), [&](int, int i, int j, double v) {
+                           if (lower && j0 + j > i0 + i) return;
+                           double *c = C + (int64_t)i * tk.ldc + j0 + j;
+                           if (store) *c = -v;
+                           else if (excl) *c -= v;
+                           else atomicAdd(c, -v);
+                       });
+    }
 }
 
 }  // namespace sc

@@ -96,7 +96,8 @@ struct sc_numeric {
     sc::SplitBlk *d_splits = nullptr;
     sc::SplitUnit *d_split_units = nullptr;
     int32_t *d_split_of_task = nullptr;
-    uint16_t *d_slices = nullptr;
+    uint16_t *d_slices = nullptr;     // NULL: no pool, the products read the panels (k_digit_tiles)
+    int64_t slice_bytes = 0;
     int32_t *d_exps = nullptr;
     CUtensorMap *d_slice_maps = nullptr;
     // solve
@@ -167,4 +168,6 @@ int plan_stats(const sc_symbolic *s, int precision, int64_t *out, int nout);
 int numeric_profile(sc_numeric *h, const double *values, int on_device, cudaStream_t st, double *ms, double *flops,
                     int32_t *launches);
 void numeric_free(sc_numeric *h);
+// Gives the slice pool back (later factorizations: k_digit_tiles, the same bits); false if there is none.
+bool drop_slices(sc_numeric *h);
 }  // namespace sc

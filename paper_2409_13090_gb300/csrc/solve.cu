@@ -1437,6 +1437,16 @@ dim3 vec_grid(const sc_numeric *h, int64_t n, int64_t ncols) {
 
 int set_sweep_attrs();
 
+// cudaMalloc for a solve: without room the factor's slice pool is given back first
+cudaError_t solve_malloc(sc_numeric *h, void **p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && drop_slices(h)) {
+        cudaGetLastError();
+        e = cudaMalloc(p, bytes);
+    }
+    return e;
+}
+
 int ensure_solve(sc_numeric *h, int64_t nrhs) {
     const sc_symbolic *s = h->sym;
     int64_t n = s->n;
@@ -1444,7 +1454,7 @@ int ensure_solve(sc_numeric *h, int64_t nrhs) {
         auto up = [&](auto *&dst, const auto &src) -> int {
             using U = typename std::remove_reference<decltype(src)>::type::value_type;
             size_t b = std::max<size_t>(1, src.size()) * sizeof(U);
-            if (cudaMalloc((void **)&dst, b) != cudaSuccess) return SC_ERR_OOM;
+            if (solve_malloc(h, (void **)&dst, b) != cudaSuccess) return SC_ERR_OOM;
             h->device_bytes += (int64_t)b;
             if (!src.empty() && cudaMemcpy(dst, src.data(), src.size() * sizeof(U), cudaMemcpyHostToDevice) != cudaSuccess)
                 return SC_ERR_CUDA;
@@ -1456,7 +1466,7 @@ int ensure_solve(sc_numeric *h, int64_t nrhs) {
         if ((rc = up(h->d_csr_ptr, s->csr_ptr))) return rc;
         if ((rc = up(h->d_csr_col, s->csr_col))) return rc;
         if ((rc = up(h->d_csr_map, s->csr_map))) return rc;
-        if (cudaMalloc((void **)&h->d_csr_val, std::max<size_t>(1, s->csr_col.size()) * 8) != cudaSuccess)
+        if (solve_malloc(h, (void **)&h->d_csr_val, std::max<size_t>(1, s->csr_col.size()) * 8) != cudaSuccess)
             return SC_ERR_OOM;
         // solve tiles in level order: per chunk, row tiles below the diagonal block
         std::vector<TrsmTile> tiles;
@@ -1570,8 +1580,8 @@ int ensure_solve(sc_numeric *h, int64_t nrhs) {
         // before every solve): per block of right-hand sides, arrivals, backward
         // counters and done flags (nchunks words each, kSyncStride apart); then
         // the two work counters
-        if (cudaMalloc((void **)&h->d_serr, sizeof(int32_t)) != cudaSuccess) return SC_ERR_OOM;
-        if (cudaMalloc((void **)&h->d_red, 4096 * sizeof(double)) != cudaSuccess) return SC_ERR_OOM;
+        if (solve_malloc(h, (void **)&h->d_serr, sizeof(int32_t)) != cudaSuccess) return SC_ERR_OOM;
+        if (solve_malloc(h, (void **)&h->d_red, 4096 * sizeof(double)) != cudaSuccess) return SC_ERR_OOM;
         if (set_sweep_attrs()) return SC_ERR_CUDA;
         h->solve_ready = true;
     }
@@ -1585,17 +1595,17 @@ int ensure_solve(sc_numeric *h, int64_t nrhs) {
         double **d64[] = {&h->d_x, &h->d_r, &h->d_b, &h->d_xbest};
         for (double **p : d64) {
             if (*p) cudaFree(*p);
-            if (cudaMalloc((void **)p, (size_t)n * nrhs * sizeof(double)) != cudaSuccess) return SC_ERR_OOM;
+            if (solve_malloc(h, (void **)p, (size_t)n * nrhs * sizeof(double)) != cudaSuccess) return SC_ERR_OOM;
         }
         const int64_t nblk = (nrhs + kRhsBlk - 1) / kRhsBlk;
         void **dw[] = {&h->d_y, &h->d_z, &h->d_acc, &h->d_xw};
         for (void **p : dw) {
             if (*p) cudaFree(*p);
-            if (cudaMalloc(p, (size_t)n * std::min<int64_t>(nrhs, kRhsBlk) * nblk * h->elt) != cudaSuccess)
+            if (solve_malloc(h, p, (size_t)n * std::min<int64_t>(nrhs, kRhsBlk) * nblk * h->elt) != cudaSuccess)
                 return SC_ERR_OOM;
         }
         if (h->d_sync) cudaFree(h->d_sync);
-        if (cudaMalloc((void **)&h->d_sync,
+        if (solve_malloc(h, (void **)&h->d_sync,
                        (kSyncWords * s->chunks.size() * kSyncStride * nblk + 2) * sizeof(int32_t)) != cudaSuccess)
             return SC_ERR_OOM;
         h->solve_cap = nrhs;
@@ -1842,10 +1852,10 @@ int pcg(sc_numeric *h, int64_t nrhs, cudaStream_t st, double tol, int maxit, dou
         double **arr[] = {&h->d_cgz, &h->d_cgp, &h->d_cgq};
         for (double **p : arr) {
             if (*p) cudaFree(*p);
-            if (cudaMalloc((void **)p, (size_t)n * nrhs * sizeof(double)) != cudaSuccess) return SC_ERR_OOM;
+            if (solve_malloc(h, (void **)p, (size_t)n * nrhs * sizeof(double)) != cudaSuccess) return SC_ERR_OOM;
         }
         if (h->d_cgs) cudaFree(h->d_cgs);
-        if (cudaMalloc((void **)&h->d_cgs, 3 * nrhs * sizeof(double)) != cudaSuccess) return SC_ERR_OOM;
+        if (solve_malloc(h, (void **)&h->d_cgs, 3 * nrhs * sizeof(double)) != cudaSuccess) return SC_ERR_OOM;
         h->cg_cap = nrhs;
     }
     const dim3 g = vec_grid(h, n, nrhs);

@@ -242,3 +242,44 @@ def test_solve_with_ill_conditioned_blocks(what, n, chunk, nrhs):
     eta = oracle.backward_error(A, B, X)
     assert eta.max() <= 1e-14, eta.max()
     assert info["converged"] and info["iterations"] == 0
+
+
+@pytest.mark.parametrize("what", ["dense 700", "dense 700 chunk 24", "deterministic st27", "deterministic lap2d"])
+def test_products_without_the_slice_pool(what):
+    """A handle without memory for the slices forms the same products from the panels: the same
+    bits where the additions have one order (one supernode; deterministic plans)."""
+    if what.startswith("dense"):
+        A = _dense(700, 3)
+        sym = sc.Symbolic(A, ordering="natural", chunk=24 if "24" in what else 64)
+    else:
+        A = inputs.stencil_3d_27pt(13, 11, 12, seed=9) if "st27" in what else inputs.laplacian_2d(83, 71, 0.05)
+        sym = sc.Symbolic(A, ordering="grid_nd", grid=A.grid, merge=0.3, variant="rl", deterministic=True)
+    num = sym.factor(A.values, precision="fp64")
+    p = num.profile(A.values)
+    assert num.rc == 0 and (p["gemm_tc"]["launches"] > 0 or what.endswith("lap2d"))
+    L = num.export_L()
+    try:
+        num.drop_slices()
+    except sc.SCError:
+        assert p["gemm_tc"]["launches"] == 0  # no product large enough
+        return
+    num.refactor(A.values)
+    assert np.array_equal(num.export_L().view(np.uint64), L.view(np.uint64))
+    with pytest.raises(sc.SCError):
+        num.drop_slices()
+    num.refactor(A.values)
+    assert np.array_equal(num.export_L().view(np.uint64), L.view(np.uint64))
+
+
+@pytest.mark.parametrize("variant", ["rlb", "rl"])
+def test_irregular_updates_without_the_slice_pool(variant):
+    """As test_irregular_updates_between_supernodes, by the products from the panels."""
+    A = inputs.stencil_3d_27pt(13, 11, 12, seed=9)
+    sym = sc.Symbolic(A, ordering="grid_nd", grid=A.grid, variant=variant, merge=0.3)
+    num = sym.factor(A.values, precision="fp64")
+    num.drop_slices()
+    num.refactor(A.values)
+    o = oracle.Oracle(A, oracle.nd_grid(*A.grid, 8), pr=True, merge=0.3)
+    assert o.factor() == 0
+    Lo = o.L_supernodal()
+    assert np.abs(num.export_L() - Lo).max() <= TOL * np.abs(Lo).max()
