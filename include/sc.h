@@ -72,7 +72,19 @@ enum sc_ordering {
 };
 enum sc_variant { SC_RLB = 0, SC_RL = 1 };
 /* Arithmetic of the numeric factorization:
- *   SC_FP64  every operation in FP64 (the paper's precision, Sec. 3.1);
+ *   SC_FP64  the factor and the vectors in FP64 (the paper's precision, Sec. 3.1),
+ *            backward stable as with FP64 operations: |A - L L^T| of a few n u
+ *            sqrt(a_ii a_jj), u = 2^-53, and the solution likewise. Pivots, and products too
+ *            small for it, are FP64 operations; the others are formed from whole
+ *            numbers of 62 bits on the tensor cores, summed exactly and rounded once. Those
+ *            have one exponent per row of a block of L (up to 64 columns; in
+ *            products up to their inner dimension) and per 64 entries of a right-hand
+ *            side. So an entry far smaller than the largest beside it is accurate to
+ *            some 2^-60 of that one, not to 2^-53 of itself: in a solution that decays by
+ *            2^40 within 64 unknowns the smallest entries keep 20 bits, by 2^60
+ *            none. With tune.fused = 1 (variant SC_RLB) every operation of the factorization
+ *            and of the solve is an FP64 operation, which keeps them, at two to ten
+ *            times the time;
  *   SC_FP32  factor stored and computed in FP32 (SIMT FMA);
  *   SC_TF32  factor stored in FP32, large update products on the TF32 tensor
  *            cores with FP32 accumulation.
@@ -86,9 +98,9 @@ enum sc_variant { SC_RLB = 0, SC_RL = 1 };
  * ir_tol. */
 enum sc_precision { SC_FP64 = 0, SC_FP32 = 1, SC_TF32 = 2, SC_TF32X3 = 3 };
 
-/* Launch-plan settings (host-side choices only: every setting runs the same
- * kernels on the same data, so the factor agrees with the default plan up to
- * the rounding order of the update sums). A zero field means the library
+/* Launch-plan settings (host-side choices only: the factor agrees with the default
+ * plan's up to the rounding order of the update sums, with SC_FP64 and fused also
+ * up to how products are rounded, see enum sc_precision). A zero field means the library
  * default, given in brackets. sc_tune picks them by timing; a caller may also
  * pass a table through sc_options.tune.
  *   tile_min_entries  an Alg. 5 product (B, B') becomes a tiled task when it
@@ -115,7 +127,8 @@ enum sc_precision { SC_FP64 = 0, SC_FP32 = 1, SC_TF32 = 2, SC_TF32X3 = 3 };
  *   fused             1 = every level of an FP64 / FP32 RLB factorization runs as
  *                     one persistent launch (POTRF, TRSM, products, device loops
  *                     and the previous level's lookahead products, ordered by
- *                     device-side counters), -1 = one launch per kernel class
+ *                     device-side counters; with SC_FP64 by FP64 operations only, in
+ *                     the solve too), -1 = one launch per kernel class
  *                     (each class at its own occupancy) [-1]
  *   tc_wide256        products at least this wide (that would take 128-column
  *                     tiles) take 256-column tensor-core tiles, which read

@@ -483,7 +483,7 @@ int run_levels(sc_numeric *h, cudaStream_t st, Prof *prof = nullptr, cudaStream_
     const double tau = s->opt.pivot_tau;
     // diagonal-block inverses for the solve, all chunks but k_narrow's in one launch
     auto launch_inverses = [&]() {
-        const int32_t nch = h->inv_cnt;
+        const int32_t nch = sizeof(T) == 8 && h->fused ? 0 : h->inv_cnt;  // (FP64 operations only: substitution)
         const int32_t *list = h->d_potrf + h->inv_off;
         if (!nch) return;
         B(kProfPotrf);
@@ -1284,17 +1284,17 @@ int numeric_create(sc_symbolic *s, int precision, sc_numeric **out) {
     // lookahead needs concurrent work: the captured graph's branches, or the fused launches
     h->lookahead = (h->use_graph || h->fused) && s->opt.variant == SC_RLB && kn.lookahead;
     build_plan(s, precision, P, h->lookahead, !h->fused);
-    if (cudaMalloc(&h->d_inv, (size_t)std::max<int64_t>(1, P.inv_size) * h->elt) != cudaSuccess) return fail(SC_ERR_OOM);
-    bytes += P.inv_size * (int64_t)h->elt;
-    if (precision == SC_FP64 && !h->fused) {
-        const size_t b = (size_t)std::max(1, P.chunk64_units) * 256 * sizeof(uint64_t);
-        if (cudaMalloc((void **)&h->d_chunk64, b) != cudaSuccess) return fail(SC_ERR_OOM);
-        bytes += (int64_t)b;
+    const bool digits = precision == SC_FP64 && !h->fused;
+    if (precision != SC_FP64 || digits) {
+        if (cudaMalloc(&h->d_inv, (size_t)std::max<int64_t>(1, P.inv_size) * h->elt) != cudaSuccess) return fail(SC_ERR_OOM);
+        bytes += P.inv_size * (int64_t)h->elt;
     }
-    if (precision == SC_FP64) {
-        const size_t b = ((size_t)s->n * 2 + s->chunks.size()) * sizeof(int32_t);
-        if (cudaMalloc((void **)&h->d_inv_exp, b) != cudaSuccess) return fail(SC_ERR_OOM);
-        bytes += (int64_t)b;
+    if (digits) {
+        const size_t b = (size_t)std::max(1, P.chunk64_units) * 256 * sizeof(uint64_t);
+        const size_t be = ((size_t)s->n * 2 + s->chunks.size()) * sizeof(int32_t);
+        if (cudaMalloc((void **)&h->d_chunk64, b) != cudaSuccess) return fail(SC_ERR_OOM);
+        if (cudaMalloc((void **)&h->d_inv_exp, be) != cudaSuccess) return fail(SC_ERR_OOM);
+        bytes += (int64_t)(b + be);
     }
     if (h->fused) {
         build_flow(P, h->lookahead);

@@ -140,6 +140,48 @@ __global__ void k_perm_out(double *__restrict__ X, int64_t ldx, const T *__restr
     *dst = add ? *dst + (double)z[i] : (double)z[i];
 }
 
+// ---- FP64 operations only (handles with one launch per level): substitution in place of the
+// stored inverses. Stages the chunk's diagonal block L_cc and its reciprocal pivots,
+// scaled for steps of one shuffle and one multiply-add: l[j][k] = L_jk / L_kk (kColumns, forward;
+// j > k), or l[k][j] = L_kj / L_kk (backward; j < k).
+template <bool kColumns>
+__device__ void load_diag(double (*l)[kMaxChunk + 1], double *rinv, const double *lnz, const ChunkDev &ch) {
+    stage_block(l, lnz + ch.off + (int64_t)ch.c0 * ch.ld + ch.c0, ch.ld, ch.w, ch.w);
+    __syncthreads();
+    if (threadIdx.x < ch.w) rinv[threadIdx.x] = 1.0 / l[threadIdx.x][threadIdx.x];
+    __syncthreads();
+    for (int idx = threadIdx.x; idx < ch.w * ch.w; idx += blockDim.x) {
+        const int r = idx / ch.w, c = idx % ch.w;
+        if (r > c) l[r][c] *= kColumns ? rinv[c] : rinv[r];
+    }
+    __syncthreads();
+}
+
+// The substitution for the right-hand sides x (row stride ldv) of a chunk, a warp each (lane i:
+// entries i and i + 32): forward (kColumns) u_j -= M_jk u_k, then v = u / L_kk; backward
+// t_j -= M_kj t_k, then z = t / L_kk. put(row, right-hand side, value).
+template <bool kColumns, typename Put>
+__device__ void substitute(const double (*m)[kMaxChunk + 1], const double *rinv, int w, const double *x, int ldv,
+                           int nb, Put &&put) {
+    const int lane = threadIdx.x % 32;
+    for (int r = threadIdx.x / 32; r < nb; r += blockDim.x / 32) {
+        double x0 = lane < w ? x[lane * ldv + r] : 0.0, x1 = lane + 32 < w ? x[(lane + 32) * ldv + r] : 0.0;
+        for (int q = 0; q < w; q++) {
+            const int k = kColumns ? q : w - 1 - q;
+            const double uk = __shfl_sync(0xffffffffu, k < 32 ? x0 : x1, k & 31);
+            if constexpr (kColumns) {
+                if (lane > k) x0 -= m[lane][k] * uk;
+                if (lane + 32 > k && lane + 32 < w) x1 -= m[lane + 32][k] * uk;
+            } else {
+                if (lane < k) x0 -= m[k][lane] * uk;
+                if (lane + 32 < k) x1 -= m[k][lane + 32] * uk;
+            }
+        }
+        if (lane < w) put(lane, r, x0 * rinv[lane]);
+        if (lane + 32 < w) put(lane + 32, r, x1 * rinv[lane + 32]);
+    }
+}
+
 // Thread mapping of the sweeps' block products (256 threads over a 64-row
 // block and up to 64 right-hand sides): NR rows per thread, from i, R
 // right-hand sides per row from r0. FP32 blocks of more than 16 right-hand
@@ -658,15 +700,15 @@ struct SweepSmem {
 // Forward sweep: one persistent launch over all tiles in level order, every
 // unit all right-hand sides of one block (up to kRhsBlk). A wide chunk's first
 // tile waits until every tile that updates the chunk's rows of x has arrived,
-// solves y_c = L_cc^{-1} x_c once (the stored FP32 inverse as a product, or
-// FP64 substitution), writes y_c and publishes it (ready flag); the chunk's
+// solves y_c = L_cc^{-1} x_c once (the stored FP32 inverse as a product; FP64
+// substitution for a handle with one launch per level), writes y_c and publishes it (ready flag); the chunk's
 // other tiles wait for that flag and read y_c. Every tile stages its rows of L
 // before waiting, subtracts L_{rows,c} y_c from x (atomic adds: tiles of
 // several chunks update the same rows) and counts one arrival at every chunk
 // its rows fall in. A tile only waits for tiles taken earlier (lower levels,
 // or its own chunk's first tile), so the sweep needs no co-residency.
 template <typename T, int RPT>
-__global__ void __launch_bounds__(256, 3) k_fwd(const T *__restrict__ lnz, const ChunkDev *__restrict__ chunks,
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_fwd(const T *__restrict__ lnz, const ChunkDev *__restrict__ chunks,
                                              const TrsmTile *__restrict__ tiles, const SolveUnit *__restrict__ units,
                                              int total, const int32_t *__restrict__ dep_ptr,
                                              const int32_t *__restrict__ dep, const int32_t *__restrict__ need,
@@ -679,6 +721,7 @@ __global__ void __launch_bounds__(256, 3) k_fwd(const T *__restrict__ lnz, const
     extern __shared__ __align__(16) unsigned char smem_fwd[];
     const int ldv = rhs_ld(min(nrhs, kRhsBlk));
     SweepSmem<T> sm(smem_fwd, ldv);
+    __shared__ double rinv[sizeof(T) == 8 ? kMaxChunk : 1];
     __shared__ int s_t, s_ok;
     const int nblk = (nrhs + kRhsBlk - 1) / kRhsBlk;
     for (;;) {
@@ -696,7 +739,7 @@ __global__ void __launch_bounds__(256, 3) k_fwd(const T *__restrict__ lnz, const
                 const int t = su.t0 + wp;
                 const TrsmTile tl = tiles[t];
                 const ChunkDev ch = chunks[tl.chunk];
-                if constexpr (RPT == 1)  // up to kFewRhs right-hand sides
+                if constexpr (RPT == 1 && sizeof(T) == 4)  // up to kFewRhs right-hand sides
                     fwd_tile_few(lnz, ch, tl, t, dep_ptr, dep, need, glbind, x, y, nb, inv, arrive, err, spin_limit);
                 else
                     fwd_tile_warp(lnz, ch, tl, t, dep_ptr, dep, need, glbind, x, y, nb, inv, arrive, err, spin_limit,
@@ -756,14 +799,20 @@ __global__ void __launch_bounds__(256, 3) k_fwd(const T *__restrict__ lnz, const
         // loads that need no other tile: the tile's rows of L (and the diagonal block)
         stage_block(sm.lr, lnz + ch.off + (int64_t)tl.r0 * ch.ld + ch.c0, ch.ld, rows, w);
         if (first) {
-            stage_block(sm.l, inv + ch.inv, w, w, w);
+            if constexpr (sizeof(T) == 4) stage_block(sm.l, inv + ch.inv, w, w, w);
+            else load_diag<true>(sm.l, rinv, lnz, ch);
             if (threadIdx.x == 0)
                 s_ok = wait_flag(arrive + (int64_t)tl.chunk * kSyncStride, need[tl.chunk], err, spin_limit, 5);
             __syncthreads();
             if (!s_ok) break;
             stage_rhs(sm.xin, ldv, x, nb, w, [&](int r) { return ch.col0 + r; });
             __syncthreads();
-            {
+            if constexpr (sizeof(T) == 8) {
+                substitute<true>(sm.l, rinv, w, sm.xin, ldv, nb, [&](int k, int r, double d) {
+                    sm.v[k * ldv + r] = d;
+                    y[(int64_t)(ch.col0 + k) * nb + r] = d;
+                });
+            } else {
                 // y_c = inv(L_cc) x_c: the block's stored inverse (zero above its diagonal)
                 const Map m;
                 if (m.row(0) < w && m.r0 < nb) {
@@ -821,7 +870,7 @@ __global__ void __launch_bounds__(256, 3) k_fwd(const T *__restrict__ lnz, const
 // and marks the chunk done. Narrow chunks' warp tiles add and count, and the
 // last to finish solves.
 template <typename T, int RPT>
-__global__ void __launch_bounds__(256, 3) k_bwd(const T *__restrict__ lnz, const ChunkDev *__restrict__ chunks,
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_bwd(const T *__restrict__ lnz, const ChunkDev *__restrict__ chunks,
                                              const TrsmTile *__restrict__ tiles, const SolveUnit *__restrict__ units,
                                              int total, const int32_t *__restrict__ dep_ptr,
                                              const int32_t *__restrict__ dep, const int32_t *__restrict__ ntiles,
@@ -834,6 +883,7 @@ __global__ void __launch_bounds__(256, 3) k_bwd(const T *__restrict__ lnz, const
     extern __shared__ __align__(16) unsigned char smem_bwd[];
     const int ldv = rhs_ld(min(nrhs, kRhsBlk));
     SweepSmem<T> sm(smem_bwd, ldv);
+    __shared__ double rinv[sizeof(T) == 8 ? kMaxChunk : 1];
     __shared__ int32_t grow[kSolveRows];
     __shared__ int s_t, s_ok;
     const int nblk = (nrhs + kRhsBlk - 1) / kRhsBlk;
@@ -853,7 +903,7 @@ __global__ void __launch_bounds__(256, 3) k_bwd(const T *__restrict__ lnz, const
                 const int t = su.t0 + wp;
                 const TrsmTile tl = tiles[t];
                 const ChunkDev ch = chunks[tl.chunk];
-                if constexpr (RPT == 1)  // up to kFewRhs right-hand sides
+                if constexpr (RPT == 1 && sizeof(T) == 4)  // up to kFewRhs right-hand sides
                     bwd_tile_few(lnz, ch, tl, t, dep_ptr, dep, ntiles, glbind, y, z, acc, nb, inv, cnt, done, err,
                                  spin_limit);
                 else
@@ -918,7 +968,8 @@ __global__ void __launch_bounds__(256, 3) k_bwd(const T *__restrict__ lnz, const
 #pragma unroll
             for (int j = 0; j < Map::R; j++) o[h][j] = T(0);
         if (first) {
-            stage_block(sm.l, inv + ch.inv, w, w, w);
+            if constexpr (sizeof(T) == 4) stage_block(sm.l, inv + ch.inv, w, w, w);
+            else load_diag<false>(sm.l, rinv, lnz, ch);
         }
         if (rows > 0) {
             if (threadIdx.x < rows) grow[threadIdx.x] = glbind[ch.gl + tl.r0 + threadIdx.x];
@@ -964,7 +1015,7 @@ __global__ void __launch_bounds__(256, 3) k_bwd(const T *__restrict__ lnz, const
                 const int k = m.row(h);
                 if (k >= w) continue;
                 T *xi = sm.xin + k * ldv + m.r0, *vi = sm.v + k * ldv + m.r0;
-                if constexpr (Map::R % 4 == 0) {
+                if constexpr (sizeof(T) == 4 && Map::R % 4 == 0) {
                     // whole pieces also at a ragged end: the row's padding is never read
 #pragma unroll
                     for (int j = 0; j < Map::R; j += 4) {
@@ -985,7 +1036,10 @@ __global__ void __launch_bounds__(256, 3) k_bwd(const T *__restrict__ lnz, const
             }
         }
         __syncthreads();
-        {
+        if constexpr (sizeof(T) == 8) {
+            substitute<false>(sm.l, rinv, w, sm.xin, ldv, nb,
+                              [&](int k, int r, double d) { z[(int64_t)(ch.col0 + k) * nb + r] = d; });
+        } else {
             // z_c = inv(L_cc)^T (y_c - acc_c) with the block's stored inverse
             if (m.row(0) < w && m.r0 < nb) {
                 T zo[Map::NR][Map::R];
@@ -1005,7 +1059,7 @@ __global__ void __launch_bounds__(256, 3) k_bwd(const T *__restrict__ lnz, const
     }
 }
 
-// ---- the sweeps of an FP64 factor: the same units, waits and releases as k_fwd
+// ---- the sweeps of an FP64 factor by digits: the same units, waits and releases as k_fwd
 // and k_bwd, products from digits (sweep64.cuh). NB: 8-column blocks of
 // right-hand sides per warp (1, 2, 4 for up to 16, 32, 64).
 struct Sweep64Args {
@@ -1668,12 +1722,18 @@ int set_sweep_attrs() {
     auto set = [&](const void *k, size_t smem) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     };
-    const size_t s32 = solve_smem<float>(kRhsBlk), s64 = fx::sweep64_smem(kRhsBlk);
-    set((const void *)k_fwd<float, 1>, s32), set((const void *)k_bwd<float, 1>, s32);
-    set((const void *)k_fwd<float, 2>, s32), set((const void *)k_bwd<float, 2>, s32);
-    set((const void *)k_fwd<float, 4>, s32), set((const void *)k_bwd<float, 4>, s32);
-    set((const void *)k_fwd<float, 8>, s32), set((const void *)k_bwd<float, 8>, s32);
-    set((const void *)k_fwd<float, 16>, s32), set((const void *)k_bwd<float, 16>, s32);
+    const size_t s64 = fx::sweep64_smem(kRhsBlk);
+    auto both = [&](auto zero) {
+        using T = decltype(zero);
+        const size_t b = solve_smem<T>(kRhsBlk);
+        set((const void *)k_fwd<T, 1>, b), set((const void *)k_bwd<T, 1>, b);
+        set((const void *)k_fwd<T, 2>, b), set((const void *)k_bwd<T, 2>, b);
+        set((const void *)k_fwd<T, 4>, b), set((const void *)k_bwd<T, 4>, b);
+        set((const void *)k_fwd<T, 8>, b), set((const void *)k_bwd<T, 8>, b);
+        set((const void *)k_fwd<T, 16>, b), set((const void *)k_bwd<T, 16>, b);
+    };
+    both(0.f);
+    both(0.0);
     set((const void *)k_fwd64<1>, s64), set((const void *)k_bwd64<1>, s64);
     set((const void *)k_fwd64<2>, s64), set((const void *)k_bwd64<2>, s64);
     set((const void *)k_fwd64<4>, s64), set((const void *)k_bwd64<4>, s64);
@@ -1699,18 +1759,19 @@ int tri_solve(sc_numeric *h, int64_t nrhs, const double *B, int64_t ldb, double 
     }
     SC_CUDA(cudaMemsetAsync(h->d_sync, 0, (nblk * ss + 2) * sizeof(int32_t), st));
     SC_CUDA(cudaMemsetAsync(acc, 0, (size_t)nblk * vs * sizeof(T), st));
-    if constexpr (sizeof(T) == 8) {
-        const int64_t nbm = std::min<int64_t>(nrhs, kRhsBlk);
-        if (nbm <= 16) launch_sweeps64<1>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st);
-        else if (nbm <= 32) launch_sweeps64<2>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st);
-        else launch_sweeps64<4>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st);
+    const int nbm = (int)std::min<int64_t>(nrhs, kRhsBlk);
+    if (sizeof(T) == 8 && !h->fused) {
+        double *x64 = (double *)xw, *y64 = (double *)y, *z64 = (double *)z, *a64 = (double *)acc;
+        if (nbm <= 16) launch_sweeps64<1>(h, (int)nrhs, vs, ss, x64, y64, z64, a64, h->d_sync, nblk, st);
+        else if (nbm <= 32) launch_sweeps64<2>(h, (int)nrhs, vs, ss, x64, y64, z64, a64, h->d_sync, nblk, st);
+        else launch_sweeps64<4>(h, (int)nrhs, vs, ss, x64, y64, z64, a64, h->d_sync, nblk, st);
     } else {
-        switch (rhs_per_thread((int)std::min<int64_t>(nrhs, kRhsBlk))) {
-            case 1: launch_sweeps<float, 1>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st); break;
-            case 2: launch_sweeps<float, 2>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st); break;
-            case 4: launch_sweeps<float, 4>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st); break;
-            case 8: launch_sweeps<float, 8>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st); break;
-            default: launch_sweeps<float, 16>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st); break;
+        switch (rhs_per_thread(nbm)) {
+            case 1: launch_sweeps<T, 1>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st); break;
+            case 2: launch_sweeps<T, 2>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st); break;
+            case 4: launch_sweeps<T, 4>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st); break;
+            case 8: launch_sweeps<T, 8>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st); break;
+            default: launch_sweeps<T, 16>(h, (int)nrhs, vs, ss, xw, y, z, acc, h->d_sync, nblk, st); break;
         }
     }
     launches += 2;

@@ -283,3 +283,45 @@ def test_irregular_updates_without_the_slice_pool(variant):
     assert o.factor() == 0
     Lo = o.L_supernodal()
     assert np.abs(num.export_L() - Lo).max() <= TOL * np.abs(Lo).max()
+
+
+@pytest.mark.parametrize("nrhs", [1, 5, 20, 33, 70])
+@pytest.mark.parametrize("n", [64, 200])
+def test_decaying_solutions_of_a_fused_handle(n, nrhs):
+    """tune.fused = 1 is FP64 operations throughout, also in the solve: a chain of 4 on the
+    diagonal and -1 beside it, as one supernode, with a unit right-hand side. The solution decays by
+    3.7 a step, and nothing cancels in it: every entry has a relative error below 3 u per
+    step and sweep (one division, one product, one rounding) on top of the factor's 3 u
+    per pivot, below 9 n u in all; 10 n u."""
+    A = _dense_sym(4.0 * np.eye(n) - np.eye(n, k=1) - np.eye(n, k=-1))
+    B = np.zeros((n, nrhs))
+    B[np.arange(nrhs) * 3 % n, np.arange(nrhs)] = 1.0
+    num = sc.Symbolic(A, ordering="natural", pr=False, tune=dict(fused=1)).factor(A.values, precision="fp64")
+    assert num.rc == 0
+    X, _ = num.solve(B)
+    # the same elimination in long double
+    one = np.longdouble(1)
+    d, x = np.empty(n, np.longdouble), B.astype(np.longdouble)
+    d[0] = 4
+    for i in range(1, n):
+        d[i] = 4 - one / d[i - 1]
+        x[i] += x[i - 1] / d[i - 1]
+    x[-1] /= d[-1]
+    for i in range(n - 2, -1, -1):
+        x[i] = (x[i] + x[i + 1]) / d[i]
+    assert (np.abs(X - x) <= 10 * n * 2.0 ** -53 * np.abs(x)).all()
+
+
+@pytest.mark.parametrize("nrhs", [1, 2, 4, 7, 16, 31, 64, 130])
+@pytest.mark.parametrize("matrix", ["st27", "dense"])
+def test_solve_of_a_fused_handle(matrix, nrhs):
+    """Substitution with every register layout of the right-hand sides, against the oracle (2 n u of
+    the largest entry rounded up to 1e-12: both matrices are diagonally dominant)."""
+    A = inputs.stencil_3d_27pt(13, 11, 12, seed=9) if matrix == "st27" else _dense(170, 7)
+    kw = dict(ordering="grid_nd", grid=A.grid, merge=0.3) if matrix == "st27" else dict(ordering="natural", chunk=33)
+    o = oracle.Oracle(A, oracle.nd_grid(*A.grid, 8) if matrix == "st27" else None, pr=True)
+    assert o.factor() == 0
+    B = inputs.rhs(A.n, nrhs, nrhs)
+    x0 = o.solve(B)
+    X, _ = sc.Symbolic(A, tune=dict(fused=1), **kw).factor(A.values, precision="fp64").solve(B)
+    assert np.abs(X - x0).max() <= 1e-12 * np.abs(x0).max()
