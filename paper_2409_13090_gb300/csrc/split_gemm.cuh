@@ -10,18 +10,19 @@
 // cheaper.
 //
 // Splitting (k_split): row r of the source columns [kx0, kx0 + K) has the
-// exponent E_r with max |x| < 2^E_r. X = x 2^(62 - E_r), rounded to a whole number
-// (|X| <= 2^62), is written in 8 signed digits of base 256,
+// exponent E_r with max |x| < 2^E_r. X = x 2^(62 - E_r), truncated to a whole number
+// (|X| < 2^62), is written in 8 signed digits of base 256,
 //   X = sum_i d_i 256^(8 - i),  d_i in [-128, 127]  (|d_1| <= 65),
 // which are the bytes of X + 0x8080808080808080 less 128, stored as FP16 (exact).
 // Product: with G_g = sum over i + j = g + 1 of the slice products,
 //   sum_k x_k y_k = 2^(E_r + E_c) sum_{g = 1..8} 2^(-4 - 8 g) G_g,
-// the groups g > 8 left out (below 2^-64 of 2^(E_r + E_c) per term). A group's sum
+// the groups g > 8 left out (fx.cuh: with the truncation a term is below 2^-58.7 of
+// 2^(E_r + E_c) off, random ones 2^-62 on average). A group's sum
 // over 128 columns is a whole number of at most 114944 * 128 < 2^24, so FP32
 // accumulation in TMEM is exact; every 128 columns the groups are added into
 // a 96-bit whole number per entry, and that is rounded to FP64 once at the end.
-// A product of K columns thus has one rounding and the slices' 2^-63, where the FMA
-// chain has K roundings: against 113-bit sums the largest error is 4 to 15 times
+// A product of K columns thus has one rounding and what the digits leave out, relative to its
+// rows' largest entries, where the FMA chain has K roundings: against 113-bit sums the largest error is 4 to 15 times
 // smaller than the FMA chain's (K = 64 .. 512).
 //
 // Tile 128 x 64: the eight groups' accumulators fill the 512 TMEM columns, so the
@@ -56,7 +57,7 @@ static_assert(SMEM <= 227 * 1024, "shared memory per CTA");
 static_assert(S * BN <= 512, "TMEM columns per SM");
 constexpr int kEpiWarps = 16;                   // four per TMEM lane quarter, each 16 columns
 constexpr int kThreads = 32 * (4 + kEpiWarps);  // producer warp, MMA warp, two idle warps, epilogue warps
-// 96 registers a thread. Eight epilogue warps with twice the entries spilled their
+// 96 registers a thread, 132 bytes of spills. Eight epilogue warps with twice the entries spilled their
 // accumulators, and a spill goes to L2 here: the stages leave L1 some 30 KB.
 
 // instruction descriptor: kind::f16, D = F32, A = B = F16, both K-major, M = 128, N = n
