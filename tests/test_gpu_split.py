@@ -325,3 +325,63 @@ def test_solve_of_a_fused_handle(matrix, nrhs):
     x0 = o.solve(B)
     X, _ = sc.Symbolic(A, tune=dict(fused=1), **kw).factor(A.values, precision="fp64").solve(B)
     assert np.abs(X - x0).max() <= 1e-12 * np.abs(x0).max()
+
+
+@pytest.mark.parametrize("blocks", [600, 3000])
+def test_second_pivots_over_the_exponent_range(blocks):
+    """The 2 x 2 blocks of test_pivot_roots_over_the_exponent_range, [[d, a], [a, d]] with |a| <=
+    d / 2: L_11 = sqrt(d - a^2 / d) passes through the updated column. By the CTA-wide POTRF
+    a / d has 2 u and its product with a one FMA: (2 u a^2 / d) / (d - a^2 / d) + u <= 5/3 u;
+    by warps L_10 has 3 u, L_10^2 6 u: at most 3 u. Half of it in the root, whose own
+    error is 3 u: 4.5 u, 4.6 u with the products of these errors."""
+    rng = np.random.default_rng(blocks)
+    d = np.ldexp(rng.uniform(1.0, 2.0, blocks), rng.integers(-1000, 1001, blocks))
+    d[:6] = np.ldexp(1.0, [-1000, -991, -990, 991, 993, 1000])
+    a = d * rng.uniform(-0.5, 0.5, blocks)
+    n = 2 * blocks
+    even = np.arange(0, n, 2)
+    colptr = np.append(np.stack([even // 2 * 3, even // 2 * 3 + 2], 1).ravel(), 3 * blocks)
+    A = inputs.SparseSym(n, colptr.astype(np.int64), np.stack([even, even + 1, even + 1], 1).ravel().astype(np.int32),
+                         np.stack([d, a, d], 1).ravel())
+    num = sc.Symbolic(A, ordering="natural").factor(A.values, precision="fp64")
+    assert num.rc == 0
+    L = num.export_L().reshape(blocks, 2, 2)[:, 1, 1]
+    dl, al = d.astype(np.longdouble), a.astype(np.longdouble)
+    ref = np.sqrt(dl - al / dl * al)
+    assert (np.abs(L - ref) <= 4.6 * 2.0 ** -53 * ref).all()
+
+
+@pytest.mark.parametrize("wa,wc,wb", [(5, 3, 40), (1, 2, 17), (7, 6, 90), (4, 8, 31)])
+def test_small_chunks_with_rows_below(wa, wc, wb):
+    """600 problems of two leaves (wa and wc columns) under one root of wb: 1200 small chunks on a
+    level, taken by a warp each, with the rows below them in whole and ragged runs of 32, and rows
+    of very different scale. L against the oracle's, row by row."""
+    blocks, nb = 600, wa + wc + wb
+    rng = np.random.default_rng(wb)
+    M = np.zeros((nb, nb), dtype=bool)
+    for s in (slice(0, wa), slice(wa, wa + wc)):
+        M[s, s] = M[wa + wc:, s] = True
+    M[wa + wc:, wa + wc:] = True
+    r, c = np.nonzero(np.tril(M).T)[::-1]  # by columns
+    per = np.bincount(c, minlength=nb)
+    rows = (r[None, :] + nb * np.arange(blocks)[:, None]).ravel()
+    colptr = np.concatenate([[0], np.cumsum(np.tile(per, blocks))])
+    cols = (c[None, :] + nb * np.arange(blocks)[:, None]).ravel()
+    v = rng.uniform(-1.0, 1.0, len(rows))
+    n = blocks * nb
+    v[rows == cols] = 2.0 * nb
+    d = 2.0 ** rng.integers(-40, 41, size=n)
+    A = inputs.SparseSym(n, colptr.astype(np.int64), rows.astype(np.int32), v * d[rows] * d[cols])
+    sym = sc.Symbolic(A, ordering="natural")
+    v = sym.view()
+    widths = np.diff(v["sup_ptr"])
+    assert v["nsuper"] == 3 * blocks and sorted(set(widths)) == sorted({wa, wc, wb})
+    num = sym.factor(A.values, precision="fp64")
+    assert num.rc == 0
+    o = oracle.Oracle(A, None, pr=True)
+    assert o.factor() == 0
+    diag = np.empty(n)
+    diag[A.rowind[A.colptr[:-1]]] = A.values[A.colptr[:-1]]
+    scale = np.concatenate([np.repeat(np.sqrt(diag[v["perm"]][v["glbind"][v["gl_ptr"][J]:v["gl_ptr"][J + 1]]]),
+                                      widths[J]) for J in range(v["nsuper"])])
+    assert (np.abs(num.export_L() - o.L_supernodal()) <= TOL * scale).all()
