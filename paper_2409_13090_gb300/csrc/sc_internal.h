@@ -102,9 +102,11 @@ inline int tc_route_width(const Task &t, int src_width, int min_k, int wide_n, b
 // Does an FP64 product run on the tensor cores as products of FP16 slices
 // (split_gemm.cuh)? The source panel needs 16-byte aligned rows (|J| >= 16: row
 // stride a multiple of 4, panel 256-byte aligned; kx0 even), K >= 16, and enough
-// work: a tile of slice products took some 6 us when the line was set (its 36 MMAs
-// one by one; the drain and the write are most of a small one), the time in which an SM's
-// FP64 pipe makes about 24,000 multiply-adds.
+// work. Factorizations with the line at 8192 / 32768 / 131072 multiply-adds: 64^2 0.499 / 0.500
+// / 0.509 ms, 83 x 71 RL 0.635 / 0.648 / 0.648, 30x31x29 7-point 4.46 / 4.47 / 4.64, 48^3 16.33 / 16.29 /
+// 16.49, 37x41x29 graph-ordered 7.87 / 7.82 / 7.84, 24x22x25 27-point 3.23 / 3.27 / 3.37. Thin products
+// (min(m, n) <= 8) above it run as tiles that are mostly padding; left to the
+// warp-block kernel instead the 48^3 step took 18.61 ms for 18.58, graph-ordered 8.99 for 9.05.
 constexpr double kSplitMinWork = 32768;
 inline bool split_route(const Task &t, int src_width) {
     return src_width >= 16 && t.k >= 16 && t.kx0 % 2 == 0 && (double)t.m * t.n * t.k >= kSplitMinWork;
