@@ -445,9 +445,12 @@ int sc_probe_fma_peak(int kind, void *cuda_stream, double *flops_per_s);
  * product tasks, warp-sized tasks, tiled tasks, SIMT tiles, tensor-core tiles,
  * TRSM tiles, RL assembly pairs, device-loop items, warp-block units, SIMT
  * tiles split along the inner dimension (added atomically), target-owned RL
- * assembly slabs (deterministic plans) and the tensor-core tiles that are 256
- * columns wide. SC_FP64 products are counted as the SIMT tiles they cover, also
- * where they run on the tensor cores as products of slices. Errors: -1, -2, -3. */
+ * assembly slabs (deterministic plans), the tensor-core tiles that are 256
+ * columns wide, and the 128 x 64 tiles of SC_FP64 products formed by digits on the
+ * tensor cores (not among the tensor-core tiles before, which are TF32). SC_FP64
+ * products are counted among the SIMT tiles and warp-block units that they would
+ * be, also where they run as digit tiles. Chunks that one warp factors with the
+ * rows below have no TRSM tiles. Errors: -1, -2, -3. */
 int sc_plan_stats(const sc_symbolic *s, int precision, int64_t *out, int nout);
 
 /* Host-side check of the device schedule of s (no device work): recomputes,

@@ -357,7 +357,8 @@ class Symbolic:
         return out
 
     PLAN_KEYS = ["levels", "chunks", "tasks", "warp_tasks", "tiled_tasks", "simt_tiles", "tc_tiles", "trsm_tiles",
-                 "rl_pairs", "loop_items", "thin_units", "split_tiles", "rl_slabs", "tc256_tiles"]
+                 "rl_pairs", "loop_items", "thin_units", "split_tiles", "rl_slabs", "tc256_tiles",
+                 "digit_tiles"]
 
     CHECK_KINDS = {0: "ok", 1: "source range", 2: "target range", 3: "trapezoid", 4: "not an ancestor",
                    5: "level order", 6: "critical flag", 7: "run mapping", 8: "RL pool", 9: "RL relind",

@@ -1198,7 +1198,13 @@ int split_plan_check(const sc_symbolic *s, int64_t *bad_level) {
 
 int plan_stats(const sc_symbolic *s, int precision, int64_t *out, int nout) {
     Plan P;
-    P.fused = true;  // every chunk counted with its TRSM tiles
+    P.fused = fused_plan(s, precision);
+    int64_t digit_tiles = 0;
+    if (precision == SC_FP64 && !P.fused) {
+        Plan D;
+        build_plan(s, precision, D, false, true);
+        for (const LevelPlan &l : D.levels) digit_tiles += l.crit.sp_cnt + l.rest.sp_cnt + l.rlsp_cnt;
+    }
     build_plan(s, precision, P, false, false);  // FP64: the products as the SIMT tiles they cover
     int64_t small_tasks = 0, tile_tasks = 0;
     for (const LevelPlan &l : P.levels) small_tasks += l.small_cnt + l.rls_cnt;
@@ -1207,13 +1213,13 @@ int plan_stats(const sc_symbolic *s, int precision, int64_t *out, int nout) {
     for (const LevelPlan &l : P.levels) {
         tc256_tiles += l.crit.tc256_cnt + l.rest.tc256_cnt;
         tc_tiles += l.crit.tc_cnt + l.crit.tc64_cnt + l.crit.tc256_cnt + l.rest.tc_cnt + l.rest.tc64_cnt +
-                    l.rest.tc256_cnt + l.crit.sp_cnt + l.rest.sp_cnt + l.rlsp_cnt;
+                    l.rest.tc256_cnt;
         simt_tiles += l.crit.gemm_cnt + l.rest.gemm_cnt + l.rlg_cnt;
     }
     for (const GemmTile &g : P.gemm) split_tiles += g.ks >= 0;
     int64_t v[] = {(int64_t)P.levels.size(), (int64_t)P.cd.size(), (int64_t)P.tasks.size(), small_tasks, tile_tasks,
                    simt_tiles, tc_tiles, (int64_t)P.trsm.size(), (int64_t)P.rlpairs.size(), (int64_t)P.loops.size(),
-                   (int64_t)P.thin.size(), split_tiles, (int64_t)P.rlslabs.size(), tc256_tiles};
+                   (int64_t)P.thin.size(), split_tiles, (int64_t)P.rlslabs.size(), tc256_tiles, digit_tiles};
     for (int i = 0; i < nout && i < (int)(sizeof(v) / sizeof(v[0])); i++) out[i] = v[i];
     return SC_OK;
 }

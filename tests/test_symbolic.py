@@ -673,3 +673,17 @@ def test_random_patterns_all_options(seed):
             assert np.array_equal(v[k], getattr(o, k)), (ordering, k)
         chk = sym.check_schedule()
         assert chk["ok"], (ordering, chk)
+
+
+def test_fp64_plan_counts_are_those_of_the_plan_that_runs():
+    """sc_plan_stats on a dense matrix (one supernode): the default FP64 plan has digit tiles and
+    64-row TRSM tiles, the fused one no digit tiles and 16-row TRSM tiles, FP32 no digit tiles."""
+    n = 400
+    A = _dense_spd(n, 4)
+    rows = [n - c for c in range(64, n, 64)]  # rows below each 64-column chunk
+    d = sc.Symbolic(A, ordering="natural").plan_stats("fp64")
+    f = sc.Symbolic(A, ordering="natural", tune=dict(fused=1)).plan_stats("fp64")
+    assert d["digit_tiles"] > 0 and d["trsm_tiles"] == sum(-(-r // 64) for r in rows)
+    assert f["digit_tiles"] == 0 and f["simt_tiles"] == d["simt_tiles"] > 0
+    assert f["trsm_tiles"] == sum(-(-r // 16) for r in rows)
+    assert sc.Symbolic(A, ordering="natural").plan_stats("fp32")["digit_tiles"] == 0
