@@ -1290,17 +1290,32 @@ int numeric_create(sc_symbolic *s, int precision, sc_numeric **out) {
     // lookahead needs concurrent work: the captured graph's branches, or the fused launches
     h->lookahead = (h->use_graph || h->fused) && s->opt.variant == SC_RLB && kn.lookahead;
     build_plan(s, precision, P, h->lookahead, !h->fused);
-    const bool digits = precision == SC_FP64 && !h->fused;
-    if (precision != SC_FP64 || digits) {
+    if (precision != SC_FP64) {
         if (cudaMalloc(&h->d_inv, (size_t)std::max<int64_t>(1, P.inv_size) * h->elt) != cudaSuccess) return fail(SC_ERR_OOM);
         bytes += P.inv_size * (int64_t)h->elt;
-    }
-    if (digits) {
-        const size_t b = (size_t)std::max(1, P.chunk64_units) * 256 * sizeof(uint64_t);
-        const size_t be = ((size_t)s->n * 2 + s->chunks.size()) * sizeof(int32_t);
-        if (cudaMalloc((void **)&h->d_chunk64, b) != cudaSuccess) return fail(SC_ERR_OOM);
-        if (cudaMalloc((void **)&h->d_inv_exp, be) != cudaSuccess) return fail(SC_ERR_OOM);
-        bytes += (int64_t)(b + be);
+    } else if (!h->fused) {
+        // what FP64 by digits holds beside the factor: the inverses and the digits between POTRF
+        // and TRSM (4 to 17 % of the factor's size). Without room an RLB handle runs
+        // by FP64 operations, which hold neither.
+        const size_t b[3] = {(size_t)std::max<int64_t>(1, P.inv_size) * h->elt,
+                             (size_t)std::max(1, P.chunk64_units) * 256 * sizeof(uint64_t),
+                             ((size_t)s->n * 2 + s->chunks.size()) * sizeof(int32_t)};
+        if (cudaMalloc(&h->d_inv, b[0]) == cudaSuccess && cudaMalloc((void **)&h->d_chunk64, b[1]) == cudaSuccess &&
+            cudaMalloc((void **)&h->d_inv_exp, b[2]) == cudaSuccess) {
+            bytes += (int64_t)(b[0] + b[1] + b[2]);
+        } else {
+            if (s->opt.variant != SC_RLB) return fail(SC_ERR_OOM);
+            cudaGetLastError();
+            for (void *p : {h->d_inv, (void *)h->d_chunk64, (void *)h->d_inv_exp})
+                if (p) cudaFree(p);
+            h->d_inv = nullptr;
+            h->d_chunk64 = nullptr;
+            h->d_inv_exp = nullptr;
+            P = Plan();
+            h->fused = P.fused = true;
+            h->lookahead = kn.lookahead;
+            build_plan(s, precision, P, h->lookahead, false);
+        }
     }
     if (h->fused) {
         build_flow(P, h->lookahead);

@@ -385,3 +385,31 @@ def test_small_chunks_with_rows_below(wa, wc, wb):
     scale = np.concatenate([np.repeat(np.sqrt(diag[v["perm"]][v["glbind"][v["gl_ptr"][J]:v["gl_ptr"][J + 1]]]),
                                       widths[J]) for J in range(v["nsuper"])])
     assert (np.abs(num.export_L() - o.L_supernodal()) <= TOL * scale).all()
+
+
+def test_without_memory_for_the_inverses():
+    """With less device memory than FP64 by digits holds beside the factor (all but that much is
+    taken first), an RLB handle runs by FP64 operations."""
+    import torch
+    A = inputs.laplacian_2d(1000, 1000, 0.05)
+    kw = dict(ordering="grid_nd", grid=A.grid, merge=0.125)
+    sym = sc.Symbolic(A, **kw)
+    B = inputs.rhs(A.n, 2, 1)
+    num = sym.factor(A.values, precision="fp64")
+    full = num.info.device_bytes
+    X0, _ = num.solve(B)
+    num.free()
+    small = sc.Symbolic(A, tune=dict(fused=1), **kw).factor(A.values, precision="fp64").info.device_bytes
+    assert full - small > 160 << 20
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    taken = torch.empty(free - small - (64 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        num = sym.factor(A.values, precision="fp64")
+        assert num.rc == 0 and num.info.device_bytes < full - (128 << 20)
+    finally:
+        del taken
+        torch.cuda.empty_cache()
+    X, _ = num.solve(B)
+    assert np.abs(X - X0).max() <= TOL * np.abs(X0).max()
+    assert num.profile(A.values)["gemm_tc"]["launches"] == 0
