@@ -67,8 +67,13 @@ SC_HD inline int block_rows(int rows, int nb, int ni_min, bool lower) {
 }
 
 constexpr int kMaxChunk = 64;
-constexpr int kLoopMinWarps = 1216;  // loop items of narrow supernodes of a level from which a warp takes one
-constexpr int kNarrowMin64 = 1024;  // small chunks of a level from which FP64 takes them by warps
+// Loop items of narrow supernodes of a level from which a warp takes one. FP64 factorizations at
+// 304 / 1216 / 4864: 64^2 0.491 / 0.503 / 0.504 ms, 300 x 280 2.44 / 2.38 / 2.40, 48^3 16.28 / 16.29 / 16.21,
+// 37x41x29 graph-ordered 7.86 / 7.82 / 7.71, 24x22x25 27-point 3.41 / 3.27 / 3.19.
+constexpr int kLoopMinWarps = 1216;
+// Small chunks of a level from which FP64 takes them by warps. At 256 / 1024 / 4096: 300 x 280 2.36 /
+// 2.38 / 2.63 ms, 64 2D matrices 3.65 / 3.64 / 3.68, 48^3 and the others within 0.1 %.
+constexpr int kNarrowMin64 = 1024;
 
 // FP64 POTRF to TRSM: 256-word units of a chunk's digits -- L_cc, the inverses of its
 // 16 x 16 diagonal blocks, exponents.
@@ -83,6 +88,8 @@ constexpr int kNarrowChunk = 16;  // solve tiles of chunks up to this width take
 // FP32: up to 16 columns and 128 rows. FP64, where a warp's multiply-add takes 64 clocks:
 // while it has at most 200 of them in line (7 us; the CTA-wide POTRF and TRSM
 // take some 32 us in two launches) -- w^2 / 2 + 6 w for the pivots and w^2 / 2 for 32 rows.
+// With the line at 100 / 200 / 400: 300 x 280 2.46 / 2.38 / 2.32 ms, 64 2D matrices 4.00 / 3.64 / 3.59, the
+// 3D ones within 0.1 %.
 SC_HD inline bool narrow_chunk(int w, int rows, bool fp64) {
     if (w > kNarrowChunk || rows > 128) return false;
     return !fp64 || w * w / 2 * (1 + (rows + 31) / 32) + 6 * w <= 200;
